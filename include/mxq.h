@@ -152,9 +152,9 @@ int mxq_slice_scale(const void *codes, const uint8_t *scales, size_t n, int bloc
 /*
  * Q_{h->l} for several targets at once (Sec. 3.5, Inference: one stored anchor, lower precisions
  * on demand): the same results as `ntargets` calls of mxq_slice_scale with the same source.
- * Consecutive targets (dst_fmts[0] with [1], [2] with [3]) that form one of the fused pairs --
- * MXINT8 -> {MXINT6, MXINT4}, MXFP8 E4M3 -> {E2M3, E2M1}, {E3M2, E2M1}, {E3M2, E2M3}, in either order
- * -- are produced by ONE pass over the anchor; any other legal target is produced by a pass of its own.
+ * From an 8-bit anchor (MXINT8, MXFP8 E4M3) up to four different lower formats, in any order, are produced by
+ * ONE pass over the anchor (five or more by two passes); a format that occurs a second time, the anchor's own
+ * format and targets of other sources take a pass of their own.
  *   dst_fmts, out_codes, out_scales  [in] HOST arrays of `ntargets` entries (0 <= ntargets <=
  *                                    MXQ_MULTI_TARGETS_MAX); the pointers inside are device pointers
  *                                    with the requirements of mxq_slice_scale; outputs must not
@@ -294,10 +294,10 @@ int mxq_slice_scale_batched(const mxq_ss_item *items, int count, int block,
 /*
  * Whole-model conversion into TWO lower formats from one read of every anchor (Sec. 3.5, Inference: one
  * stored anchor checkpoint, several precisions served at once; Eq. 4-5 applied twice per element): the
- * results of mxq_slice_scale_batched to dst_fmt1 and to dst_fmt2.  For the fused pairs of
- * mxq_slice_scale_multi one launch covers 256 tensors and reads the anchors once (2.34 instead of
- * 3.375 bytes per element for 6-bit + 4-bit targets); any other legal pair of targets runs as two
- * single-target batched passes.  `items` is a HOST array; requirements per pointer as in mxq_slice_scale;
+ * results of mxq_slice_scale_batched to dst_fmt1 and to dst_fmt2.  For two different lower formats of an
+ * 8-bit anchor one launch covers 256 tensors and reads the anchors once (2.34 instead of 3.375 bytes per
+ * element for 6-bit + 4-bit targets); any other legal pair of targets runs as two single-target batched
+ * passes.  `items` is a HOST array; requirements per pointer as in mxq_slice_scale;
  * block must be 32, 64 or 128; outputs must not overlap the inputs or one another.  Nothing is allocated
  * on the device.
  */

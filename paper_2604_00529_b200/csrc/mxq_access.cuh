@@ -209,28 +209,30 @@ __device__ __forceinline__ void store_bytes(void* p, const uint32_t (&w)[NW])
 // there, and a whole tile leaves as ONE bulk copy shared -> global issued by one lane (the copy
 // engine writes full lines; no cluster, no tensor map, no multicast).  Only the ragged last tile of
 // a tensor is copied out by the lanes as 16-byte pieces.
-// Measured at 2^26 codes: MXINT8 -> MXINT6 and E4M3 -> E2M3 / E3M2 4 - 8 % faster than direct stores;
-// the 20-, 12- and 10-byte pieces of the 5- and 3-bit streams are faster stored directly (2 - 8 %).
+// Measured at 2^26 codes: MXINT8 -> MXINT6 and E4M3 -> E2M3 / E3M2 4 - 8 % faster than direct stores, the
+// BF16 quantizers to 5 bits (10 bytes per lane, five 2-byte stores) 38.9 -> 33.3 us (MXINT5) and 35.4 -> 32.9 us
+// (E2M2); the 20-, 12- and 6-byte pieces of the other 5-, 6- and 3-bit streams are faster stored directly
+// (2 - 10 %).
 
 // store instructions a lane needs for a direct store of OB bytes
 __host__ __device__ constexpr int direct_store_count(int bytes) { return bytes / piece_align(bytes); }
 
 template <int OB>
 struct StagedTile {
-    static constexpr bool use = direct_store_count(OB) > 5 || OB == 24;
+    static constexpr bool use = direct_store_count(OB) > 5 || OB == 24 || OB == 10;
 };
 
 // Copy the first `nbytes` bytes of a warp's staging area to `gdst`; both are 16-byte aligned and
 // TILE_BYTES (a multiple of 16) is the size of a whole tile.  Every lane of the warp calls it, after
-// writing its own pieces to the area with ordinary stores.
+// writing its own pieces to the area with ordinary stores.  The copy may still be reading the area on
+// return: stage_wait() comes before the area is rewritten and before the warp leaves.
 template <int TILE_BYTES>
-__device__ __forceinline__ void flush_stage(const uint8_t* stage, uint8_t* gdst, uint32_t nbytes)
+__device__ __forceinline__ void flush_stage_async(const uint8_t* stage, uint8_t* gdst, uint32_t nbytes)
 {
     static_assert(TILE_BYTES % 16 == 0, "a bulk copy moves multiples of 16 bytes");
     const uint32_t lane = threadIdx.x & 31;
     if (nbytes == TILE_BYTES) {
-        // the lanes' writes become visible to the copy engine, then one lane hands it the tile and
-        // waits until the engine has read the area (it may be rewritten or released afterwards)
+        // the lanes' writes become visible to the copy engine, then one lane hands it the tile
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         bool ok = true;
@@ -240,9 +242,7 @@ __device__ __forceinline__ void flush_stage(const uint8_t* stage, uint8_t* gdst,
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                          :: "l"(gdst), "r"(saddr), "r"(TILE_BYTES) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
-        __syncwarp();
         return;
     }
     __syncwarp();
@@ -252,7 +252,21 @@ __device__ __forceinline__ void flush_stage(const uint8_t* stage, uint8_t* gdst,
     }
     const uint32_t done = nbytes & ~15u;                        // a ragged tensor end: up to 15 bytes
     if (done + lane < nbytes) st_u8(gdst + done + lane, stage[done + lane]);
+}
+
+// All but the last PENDING copies of this warp have read their areas; every lane calls it.
+template <int PENDING>
+__device__ __forceinline__ void stage_wait()
+{
+    if ((threadIdx.x & 31) == 0) asm volatile("cp.async.bulk.wait_group.read %0;" :: "n"(PENDING) : "memory");
     __syncwarp();
+}
+
+template <int TILE_BYTES>
+__device__ __forceinline__ void flush_stage(const uint8_t* stage, uint8_t* gdst, uint32_t nbytes)
+{
+    flush_stage_async<TILE_BYTES>(stage, gdst, nbytes);
+    stage_wait<0>();
 }
 
 // ---- bitstream of element codes in registers -------------------------------------------------

@@ -6,7 +6,6 @@
 #include "mxq_launch.h"
 
 namespace mxq {
-
 namespace {
 
 inline bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
@@ -159,17 +158,33 @@ int mxq_slice_scale_multi(const void* codes, const uint8_t* scales, size_t n, in
         MXQ_DEBUG_EXPECT(out_scales[k], n / (size_t)block);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int t = 0;
-    while (t < ntargets) {
-        if (t + 1 < ntargets) {
-            const int rc = launch_slice_scale2(codes, scales, n, block, src_fmt, dst_fmts[t], dst_fmts[t + 1], out_codes[t],
-                                               out_scales[t], out_codes[t + 1], out_scales[t + 1], s);
-            if (rc == MXQ_OK) { t += 2; continue; }
-            if (rc != MXQ_ERR_PAIR) return rc;          // no fused kernel for this pair: one at a time
+    auto single = [&](int t) {
+        return launch_slice_scale(codes, scales, n, block, src_fmt, dst_fmts[t], out_codes[t], out_scales[t], s);
+    };
+    // Different lower formats of an anchor share passes: four per pass, five or six as three and the rest (a
+    // pass re-reads the anchor; one more target in a pass does not).  A repeated format, the anchor's own and
+    // other sources take a pass of their own.
+    int fmts[MXQ_MULTI_TARGETS_MAX], nset = 0;
+    SsOut outs[MXQ_MULTI_TARGETS_MAX];
+    for (int t = 0; t < ntargets; ++t) {
+        bool alone = !slice_scale_set_anchor(src_fmt) || dst_fmts[t] == src_fmt;
+        for (int k = 0; k < nset; ++k) alone |= fmts[k] == dst_fmts[t];
+        if (alone) {
+            if (int rc = single(t)) return rc;
+            continue;
         }
-        if (int rc = launch_slice_scale(codes, scales, n, block, src_fmt, dst_fmts[t], out_codes[t], out_scales[t], s))
+        fmts[nset] = dst_fmts[t];
+        outs[nset++] = SsOut{static_cast<uint8_t*>(out_codes[t]), out_scales[t]};
+    }
+    for (int at = 0; at < nset;) {
+        const int left = nset - at, take = left <= kSetTargetsMax ? left : 3;
+        if (take == 1) {
+            return launch_slice_scale(codes, scales, n, block, src_fmt, fmts[at], outs[at].codes, outs[at].scales, s);
+        }
+        if (int rc = launch_slice_scale_set(static_cast<const uint8_t*>(codes), scales, n, block, src_fmt, take, fmts + at,
+                                            outs + at, s))
             return rc;
-        ++t;
+        at += take;
     }
     return MXQ_OK;
 }
@@ -442,8 +457,8 @@ int mxq_slice_scale_pair_batched(const mxq_ss_pair_item* items, int count, int b
             !aligned(it.scales, 16) || !aligned(it.out_scales1, 16) || !aligned(it.out_scales2, 16))
             return MXQ_ERR_ALIGN;
     }
-    if (!slice_scale2_is_fused(src_fmt, dst_fmt1, dst_fmt2)) {
-        // no fused kernel for this pair of targets: one single-target batched pass each
+    if (!slice_scale_set_anchor(src_fmt) || dst_fmt1 == dst_fmt2 || dst_fmt1 == src_fmt || dst_fmt2 == src_fmt) {
+        // not two different lower formats of an anchor: one single-target batched pass each
         std::vector<mxq_ss_item> one((size_t)count);
         for (int t = 0; t < 2; ++t) {
             for (int i = 0; i < count; ++i) {
@@ -468,12 +483,12 @@ int mxq_slice_scale_pair_batched(const mxq_ss_pair_item* items, int count, int b
         MXQ_DEBUG_EXPECT(items[i].out_scales2, items[i].n / (size_t)block);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    std::vector<Ss2DeviceItem> chunk;
-    chunk.reserve(kSs2BatchItemsMax);
+    std::vector<SsPairDeviceItem> chunk;
+    chunk.reserve(kSsPairItemsMax);
     size_t tiles = 0;
     auto flush = [&]() -> int {
         if (chunk.empty()) return MXQ_OK;
-        const int rc = launch_slice_scale2_batched(chunk.data(), (int)chunk.size(), tiles, src_fmt, dst_fmt1, dst_fmt2, s);
+        const int rc = launch_slice_scale_pair_batched(chunk.data(), (int)chunk.size(), tiles, src_fmt, dst_fmt1, dst_fmt2, s);
         chunk.clear();
         tiles = 0;
         return rc;
@@ -481,19 +496,17 @@ int mxq_slice_scale_pair_batched(const mxq_ss_pair_item* items, int count, int b
     for (int i = 0; i < count; ++i) {
         const mxq_ss_pair_item& it = items[i];
         if (it.n == 0) continue;
-        Ss2DeviceItem d;
+        SsPairDeviceItem d;
         d.codes = static_cast<const uint8_t*>(it.codes);
         d.scales = it.scales;
-        d.out_codes1 = static_cast<uint8_t*>(it.out_codes1);
-        d.out_scales1 = it.out_scales1;
-        d.out_codes2 = static_cast<uint8_t*>(it.out_codes2);
-        d.out_scales2 = it.out_scales2;
+        d.out[0] = SsOut{static_cast<uint8_t*>(it.out_codes1), it.out_scales1};
+        d.out[1] = SsOut{static_cast<uint8_t*>(it.out_codes2), it.out_scales2};
         d.nunits = it.n / 32;
         d.nscales = it.n / (size_t)block;
         d.tile_begin = tiles;
-        tiles += ss2_batched_tiles(d.nunits);
+        tiles += ss_pair_batched_tiles(d.nunits);
         chunk.push_back(d);
-        if ((int)chunk.size() == kSs2BatchItemsMax)
+        if ((int)chunk.size() == kSsPairItemsMax)
             if (int rc = flush()) return rc;
     }
     return flush();

@@ -19,6 +19,7 @@
 // by byte permutes and one multiply, the sm_100a narrowing conversion instructions for MXFP.
 #pragma once
 #include <cstdint>
+#include <tuple>
 #include <type_traits>
 #include <utility>
 #include <cuda_runtime.h>
@@ -155,61 +156,55 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v)
 // Q_f: quantize (Eq. 1-3)
 // ------------------------------------------------------------------------------------------
 
-// Four 6-bit codes, one per byte, -> the 24-bit stream c0 | c1 << 6 | c2 << 12 | c3 << 18 in bits
-// 31..8 of the result (bits 7..0 clear).  Every field only ever moves LEFT relative to c3, so the
-// moves are multiply-adds (the multiply pipe) instead of shifts and selects on the logic pipe:
-// with the codes in bits 7..2 of their bytes, w + 3 (w & 0x00FF00FF) multiplies bytes 0 and 2 by 4,
-// which joins each byte pair into a 12-bit field (bits 15..4 and 31..20); y + 15 (y & 0xFFFF) then
-// multiplies the low field by 16, which joins the two.
-__device__ __forceinline__ uint32_t squeeze6_top(uint32_t w)           // codes in bits 7..2, bits 1..0 clear
-{
-    const uint32_t y = (w & 0x00FF00FFu) * 3u + w;
-    return (y & 0x0000FFFFu) * 15u + y;
-}
-
-__device__ __forceinline__ uint32_t squeeze6_low(uint32_t w)           // codes in bits 5..0, bits 7..6 clear
-{
-    const uint32_t y = (w & 0x00FF00FFu) * 12u + w * 4u;
-    return (y & 0x0000FFFFu) * 15u + y;
-}
-
-// Four such streams (each in bits 31..8 of its word) -> three 32-bit words: whole bytes, so three
-// byte permutes.
-__device__ __forceinline__ void join24(uint32_t z0, uint32_t z1, uint32_t z2, uint32_t z3, uint32_t& o0, uint32_t& o1,
-                                       uint32_t& o2)
-{
-    o0 = __byte_perm(z0, z1, 0x5321);
-    o1 = __byte_perm(z1, z2, 0x6532);
-    o2 = __byte_perm(z2, z3, 0x7653);
-}
-
-// Four B-bit codes, one per byte with the upper bits clear, -> one 4B-bit value (c0 | c1 << B | ...).
-// Two shift-and-select steps: bytes to 2B-bit fields in the 16-bit halves, halves to one field.
-// Whatever a shift drags along falls where the next select takes the other operand.
+// Four B-bit codes, one per byte, -> their 4B-bit stream c0 | c1 << B | c2 << 2B | c3 << 3B in the TOP bits of
+// the result (the bits below clear).  Every field only ever moves LEFT relative to c3, so the moves are
+// multiply-adds (the multiply pipe) instead of shifts and selects on the logic pipe: with the codes in the
+// top bits of their bytes, w + (2^(8-B) - 1) (w & 0x00FF00FF) moves bytes 0 and 2 up by 8 - B, which joins each
+// byte pair into a 2B-bit field at the top of its half; y + (2^(16-2B) - 1) (y & 0xFFFF) joins the two fields.
 template <int B>
-__device__ __forceinline__ uint32_t squeeze_bytes(uint32_t x)
+__device__ __forceinline__ uint32_t squeeze_top(uint32_t w)            // codes in the top B bits, the rest clear
 {
-    static_assert(B >= 1 && B <= 7, "codes narrower than a byte");
-    constexpr uint32_t kEven = ((1u << B) - 1u) * 0x00010001u;           // the fields of bytes 0 and 2
-    constexpr uint32_t kLow = (1u << (2 * B)) - 1u;
-    const uint32_t y = (x & kEven) | ((x >> (8 - B)) & ~kEven);
-    return (y & kLow) | ((y >> (16 - 2 * B)) & ~kLow);
+    constexpr int D = 8 - B;
+    const uint32_t y = (w & 0x00FF00FFu) * ((1u << D) - 1u) + w;
+    return (y & 0x0000FFFFu) * ((1u << (2 * D)) - 1u) + y;
 }
 
-// NZ words holding four clean B-bit codes each (one per byte) -> the little-endian bitstream.
-template <int B, int NZ, int NW>
-__device__ __forceinline__ void pack_code_bytes(const uint32_t (&z)[NZ], uint32_t (&out)[NW])
+template <int B>
+__device__ __forceinline__ uint32_t squeeze_low(uint32_t w)            // codes in the low B bits, the rest clear
 {
-    constexpr int W = 4 * B;                                             // bits per squeezed word
+    constexpr int D = 8 - B;
+    const uint32_t y = (w & 0x00FF00FFu) * (((1u << D) - 1u) << D) + w * (1u << D);
+    return (y & 0x0000FFFFu) * ((1u << (2 * D)) - 1u) + y;
+}
+
+// NZ streams of four B-bit codes, each in the top 4B bits of its word (the rest clear) -> the little-endian
+// bitstream.  Pieces that move left are multiply-adds, pieces that move right shift-adds; for 6 bits the
+// pieces are whole bytes and three byte permutes join four streams.
+template <int B, int NZ, int NW>
+__device__ __forceinline__ void pack_streams(const uint32_t (&z)[NZ], uint32_t (&out)[NW])
+{
+    constexpr int W = 4 * B;                                             // bits per stream
     static_assert(NW * 32 >= NZ * W, "output too small");
-    static_for<NZ>([&](auto j) {
-        constexpr int J = decltype(j)::value;
-        constexpr int off = J * W, wi = off >> 5, sh = off & 31;
-        const uint32_t q = squeeze_bytes<B>(z[J]);
-        if constexpr (sh == 0) out[wi] = q;
-        else out[wi] |= q << sh;
-        if constexpr (sh + W > 32) out[wi + 1] = q >> (32 - sh);
-    });
+    if constexpr (B == 6 && NZ % 4 == 0) {
+#pragma unroll
+        for (int g = 0; g < NZ / 4; ++g) {
+            out[3 * g + 0] = __byte_perm(z[4 * g + 0], z[4 * g + 1], 0x5321);
+            out[3 * g + 1] = __byte_perm(z[4 * g + 1], z[4 * g + 2], 0x6532);
+            out[3 * g + 2] = __byte_perm(z[4 * g + 2], z[4 * g + 3], 0x7653);
+        }
+    } else {
+        static_for<NZ>([&](auto j) {
+            constexpr int J = decltype(j)::value;
+            constexpr int off = J * W, wi = off >> 5, sh = off & 31;
+            // the field has to go from bit 32 - W to bit sh
+            uint32_t v;
+            if constexpr (sh <= 32 - W) v = z[J] >> (32 - W - sh);
+            else v = z[J] * (1u << (sh - (32 - W)));
+            if constexpr (sh == 0) out[wi] = v;
+            else out[wi] += v;
+            if constexpr (sh + W > 32) out[wi + 1] = z[J] >> (64 - W - sh);
+        });
+    }
 }
 
 // MXINT codes of four consecutive elements (Eq. 3), one per byte in the low F::bits bits.
@@ -277,15 +272,10 @@ __device__ __forceinline__ void quantize_unit(const uint32_t (&w)[8], float inv,
 #pragma unroll
             for (int j = 0; j < NQ / 2; ++j)
                 out[j] = __byte_perm(z[2 * j] | (z[2 * j] >> 4), z[2 * j + 1] | (z[2 * j + 1] >> 4), 0x6420);
-        } else if constexpr (F::bits == 6 && NQ % 4 == 0) {
-#pragma unroll
-            for (int g = 0; g < NQ / 4; ++g) {
-                const uint32_t s0 = squeeze6_low(z[4 * g]), s1 = squeeze6_low(z[4 * g + 1]), s2 = squeeze6_low(z[4 * g + 2]),
-                               s3 = squeeze6_low(z[4 * g + 3]);
-                join24(s0, s1, s2, s3, out[3 * g + 0], out[3 * g + 1], out[3 * g + 2]);
-            }
         } else {
-            pack_code_bytes<F::bits>(z, out);
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) z[j] = squeeze_low<F::bits>(z[j]);
+            pack_streams<F::bits>(z, out);
         }
     } else if constexpr (!F::hw_cvt) {
         // E3M3 / E2M2: four elements at a time through the hardware neighbour format
@@ -294,10 +284,11 @@ __device__ __forceinline__ void quantize_unit(const uint32_t (&w)[8], float inv,
         const float inv_k = inv * SoftFp<F>::pre_scale;          // exact: both are powers of two
         static_for<NQ>([&](auto qi) {
             constexpr int Q = decltype(qi)::value;
-            z[Q] = quantize_fp_soft_quad<F>(unit_elem<T, 4 * Q>(w) * inv_k, unit_elem<T, 4 * Q + 1>(w) * inv_k,
-                                            unit_elem<T, 4 * Q + 2>(w) * inv_k, unit_elem<T, 4 * Q + 3>(w) * inv_k);
+            z[Q] = squeeze_low<F::bits>(
+                quantize_fp_soft_quad<F>(unit_elem<T, 4 * Q>(w) * inv_k, unit_elem<T, 4 * Q + 1>(w) * inv_k,
+                                         unit_elem<T, 4 * Q + 2>(w) * inv_k, unit_elem<T, 4 * Q + 3>(w) * inv_k));
         });
-        pack_code_bytes<F::bits>(z, out);
+        pack_streams<F::bits>(z, out);
     } else {
         static_for<T::epl / 2>([&](auto i) {
             constexpr int I = decltype(i)::value;
@@ -594,6 +585,16 @@ __host__ __device__ __forceinline__ int find_item(const ITEM* items, const TileI
     return lo;
 }
 
+// A tile of the batched kernels is what one CTA converts, THREADS / 32 consecutive warp tiles of ONE tensor: the owner
+// is found once per CTA from the block index, by uniform instructions, and the tensor's pointers live in uniform
+// registers.  (With a lookup per warp tile they took two registers each in every lane.)  The calling warp's
+// tile in the tensor that starts at CTA tile `tile_begin`:
+template <int THREADS>
+__device__ __forceinline__ size_t item_warp_tile(size_t tile_begin)
+{
+    return (blockIdx.x - tile_begin) * (THREADS / 32) + (threadIdx.x >> 5);
+}
+
 // The fake-quant of a whole set of tensors (every quantized weight of a model in one QAT step, Eq. 6)
 // in one launch: the tiles of all tensors laid end to end, the item table in the kernel's parameters.
 struct FqDeviceItem {
@@ -680,28 +681,33 @@ quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk, int count, si
 // 0xFF/0x00 mask by a multiply-add with 255^-1 (mod 2^32), which runs on the multiply pipe:
 // mask = 255 * sum(s_i 256^i), hence mask * 255^-1 = sum(s_i 256^i) exactly.
 // (Checked against the scalar definition for all 2^32 input words on the host.)
+struct Int8Word {
+    uint32_t full, mag;      // 0xFF in the negative bytes; |p| per byte
+};
+
+// What every target needs of four codes (|p| = a + s: one multiply-add; 0x80 reads 128).
+__device__ __forceinline__ Int8Word int8_word(uint32_t x)
+{
+    constexpr uint32_t kInv255 = 0xFEFEFEFFu;
+    Int8Word w;
+    asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(w.full) : "r"(x));         // selector bit 3: replicate the byte's sign
+    w.mag = w.full * kInv255 + (x ^ w.full);
+    return w;
+}
+
 template <int BL>
-__device__ __forceinline__ uint32_t ss_int8_word_top(uint32_t x)
+__device__ __forceinline__ uint32_t ss_int8_word_top(const Int8Word& w)
 {
     constexpr int de = 8 - BL;
     constexpr uint32_t k01 = 0x01010101u;
     constexpr uint32_t kInv255 = 0xFEFEFEFFu;
     constexpr uint32_t kH = k01 * (1u << (de - 1));            // rounding increment
     constexpr uint32_t kTop = k01 * ((0xFFu << de) & 0xFFu);   // the top BL bits of every byte
-    uint32_t full, ov;
-    asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(full) : "r"(x)); // selector bit 3: replicate the byte's sign
-    const uint32_t a = x ^ full;
-    const uint32_t t = a + (full * kInv255 + kH);
+    const uint32_t t = w.mag + kH;
+    uint32_t ov;
     asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(ov) : "r"(t));   // 0xFF where the magnitude clips
-    const uint32_t m = (t ^ ov ^ full) & kTop;
-    return (full * (kInv255 << de) + m) & kTop;
-}
-
-// The same four codes in the low BL bits of their bytes.
-template <int BL>
-__device__ __forceinline__ uint32_t ss_int8_word(uint32_t x)
-{
-    return ss_int8_word_top<BL>(x) >> (8 - BL);
+    const uint32_t m = (t ^ ov ^ w.full) & kTop;
+    return (w.full * (kInv255 << de) + m) & kTop;
 }
 
 __device__ __forceinline__ bool has_e4m3_nan(uint32_t x)
@@ -723,11 +729,9 @@ __device__ __forceinline__ void e4m3_word_to_f16(uint32_t w, uint32_t& a, uint32
 
 // two FP16 pairs (four E4M3 codes of one word), already divided by 2^de, as four FP32 values
 template <int DE>
-__device__ __forceinline__ void e4m3_word_scaled(uint32_t w, float (&f)[4])
+__device__ __forceinline__ void e4m3_pairs_scaled(uint32_t a, uint32_t b, float (&f)[4])
 {
     constexpr uint32_t kHalf = (uint32_t)(15 - DE) << 10;      // 2^-de as FP16
-    uint32_t a, b;
-    e4m3_word_to_f16(w, a, b);
     asm("{ .reg .b16 l, h; .reg .b32 a, b;\n"
         "  mul.rn.f16x2 a, %4, %6;  mul.rn.f16x2 b, %5, %6;\n"
         "  mov.b32 {l, h}, a;  cvt.f32.f16 %0, l;  cvt.f32.f16 %1, h;\n"
@@ -735,29 +739,55 @@ __device__ __forceinline__ void e4m3_word_scaled(uint32_t w, float (&f)[4])
         : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]) : "r"(a), "r"(b), "r"(kHalf | (kHalf << 16)));
 }
 
-// four E4M3 codes (one word) -> four 6-bit codes, one per byte
+// Four E4M3 codes, given as two FP16 pairs, in a 5-, 6- or 7-bit MXFP format, the codes in the top bits of their
+// bytes.  `nans` has 0x7F in the bytes whose anchor code was a NaN code (see e4m3_word_clean).
+//   E2M3, E3M2: divided by 2^de (exact in FP16), widened to FP32, narrowing conversion.
+//   E3M3      : no narrowing instruction, but it is E4M3 with fewer binades (see SoftFp): the same through the
+//               conversion to E4M3 of the value divided by a further 2^4.
+//   E2M2      : the same through E5M2 (bias 15, a further 2^14), whose conversion takes the FP16 pair itself, without
+//               the trip through FP32 (the E4M3 conversion of FP16 pairs is slower than that trip).  The FP16 product
+//               is exact where it matters: it loses bits only below the smallest halfway point 2^-17, where every
+//               value rounds to zero either way (anchor codes have four significant bits).
+// Nothing is clipped: the largest anchor value 448 / 2^de (7, 28, 28, 7) does not exceed the target's largest
+// (7.5, 28, 30, 7).
 template <class FL>
-__device__ __forceinline__ uint32_t ss_e4m3_word_to6(uint32_t w)
+__device__ __forceinline__ uint32_t ss_e4m3_pairs_top(uint32_t a, uint32_t b, uint32_t nans)
 {
-    static_assert(FL::bits == 6 && FL::hw_cvt, "6-bit target with a narrowing cvt");
-    float f[4];
-    e4m3_word_scaled<8 - FL::emax>(w, f);
-    uint32_t d;
-    if constexpr (FL::id == MXQ_FP6_E2M3)
-        asm("{ .reg .b16 l, h; cvt.rn.satfinite.e2m3x2.f32 l, %2, %1; cvt.rn.satfinite.e2m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
-            : "=r"(d) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
-    else
-        asm("{ .reg .b16 l, h; cvt.rn.satfinite.e3m2x2.f32 l, %2, %1; cvt.rn.satfinite.e3m2x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
-            : "=r"(d) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
-    return d;
+    constexpr int de = 8 - FL::emax, D = 8 - FL::bits;
+    constexpr uint32_t k01 = 0x01010101u;
+    constexpr uint32_t kMag = k01 * FL::max_mag;
+    uint32_t c;
+    if constexpr (FL::id == MXQ_FP5_E2M2) {
+        constexpr uint32_t kHalf = 1u << (24 - (de + 14));           // 2^-20 as an FP16 subnormal
+        asm("{ .reg .b16 l, h; .reg .b32 a, b; mul.rn.f16x2 a, %1, %3; mul.rn.f16x2 b, %2, %3;\n"
+            "  cvt.rn.satfinite.e5m2x2.f16x2 l, a; cvt.rn.satfinite.e5m2x2.f16x2 h, b; mov.b32 %0, {l, h}; }"
+            : "=r"(c) : "r"(a), "r"(b), "r"(kHalf | (kHalf << 16)));
+        return ((c & kMag) << D) | (c & 0x80808080u);
+    } else {
+        constexpr int k = FL::id == MXQ_FP7_E3M3 ? 4 : 0;
+        float f[4];
+        e4m3_pairs_scaled<de + k>(a, b, f);
+        if constexpr (FL::id == MXQ_FP7_E3M3)
+            asm("{ .reg .b16 l, h; cvt.rn.satfinite.e4m3x2.f32 l, %2, %1; cvt.rn.satfinite.e4m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
+                : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
+        else if constexpr (FL::id == MXQ_FP6_E2M3)
+            asm("{ .reg .b16 l, h; cvt.rn.satfinite.e2m3x2.f32 l, %2, %1; cvt.rn.satfinite.e2m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
+                : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
+        else
+            asm("{ .reg .b16 l, h; cvt.rn.satfinite.e3m2x2.f32 l, %2, %1; cvt.rn.satfinite.e3m2x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
+                : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
+        if constexpr (FL::mu == 3) c |= nans & kMag;
+        if constexpr (FL::id == MXQ_FP7_E3M3) return ((c & kMag) << D) | (c & 0x80808080u);
+        else return c << D;
+    }
 }
 
-// eight E4M3 codes (two words) -> eight E2M1 codes in one word
-__device__ __forceinline__ uint32_t ss_e4m3_words_to_e2m1(uint32_t w0, uint32_t w1)
+// eight E4M3 codes (two words, given as their four FP16 pairs) -> eight E2M1 codes in one word
+__device__ __forceinline__ uint32_t ss_e4m3_pairs_to_e2m1(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1)
 {
     float f[4], g[4];
-    e4m3_word_scaled<6>(w0, f);
-    e4m3_word_scaled<6>(w1, g);
+    e4m3_pairs_scaled<6>(a0, b0, f);
+    e4m3_pairs_scaled<6>(a1, b1, g);
     uint32_t d;
     asm("{ .reg .b8 a, b, c, e;\n"
         "  cvt.rn.satfinite.e2m1x2.f32 a, %2, %1;  cvt.rn.satfinite.e2m1x2.f32 b, %4, %3;\n"
@@ -767,31 +797,8 @@ __device__ __forceinline__ uint32_t ss_e4m3_words_to_e2m1(uint32_t w0, uint32_t 
     return d;
 }
 
-// Eq. 5 for the two MXFP targets without a narrowing instruction, E3M3 (7 bits, de = 4) and E2M2
-// (5 bits, de = 6), on four E4M3 codes per register (no NaN codes among them): the anchor values
-// divided by 2^(de + k) = 2^8 (exact in FP16), converted to the hardware neighbour format whose grid is
-// 2^-k times the target's (see SoftFp), the one code above the target's largest clipped back.
-template <class FL>
-__device__ __forceinline__ uint32_t ss_e4m3_word_soft(uint32_t x)
-{
-    using S = SoftFp<FL>;
-    constexpr uint32_t k01 = 0x01010101u;
-    constexpr int de = 8 - FL::emax;
-    uint32_t c;
-    float f[4];
-    e4m3_word_scaled<de + S::k>(x, f);
-    if constexpr (S::e3m3)
-        asm("{ .reg .b16 l, h; cvt.rn.satfinite.e4m3x2.f32 l, %2, %1; cvt.rn.satfinite.e4m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
-            : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
-    else
-        asm("{ .reg .b16 l, h; cvt.rn.satfinite.e3m2x2.f32 l, %2, %1; cvt.rn.satfinite.e3m2x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
-            : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
-    uint32_t mag = c & (k01 * S::hw_mag_mask);
-    mag -= (mag >> (FL::bits - 1)) & k01;
-    return mag | ((c >> 1) & (k01 << (FL::bits - 1)));
-}
-
-// Every legal pair, one element at a time (exact, slow): the reference path inside the kernels.
+// Every legal pair, one element at a time (exact, slow): for sources that are not an 8-bit anchor and for units
+// with E4M3 NaN codes.
 template <class FH, class FL, int NWI, int NWO>
 __device__ __forceinline__ void ss_unit_by_element(const uint32_t (&in)[NWI], uint32_t (&out)[NWO])
 {
@@ -807,13 +814,6 @@ __device__ __forceinline__ void ss_unit_by_element(const uint32_t (&in)[NWI], ui
     });
 }
 
-template <class FH, class FL>
-__host__ __device__ constexpr bool ss_e4m3_has_fast_path()
-{
-    return FH::id == MXQ_FP8_E4M3 && FL::id != MXQ_FP8_E4M3 &&
-           (FL::hw_cvt || FL::id == MXQ_FP7_E3M3 || FL::id == MXQ_FP5_E2M2);
-}
-
 __device__ __forceinline__ bool unit_has_e4m3_nan(const uint32_t (&in)[8])
 {
     bool nan = false;
@@ -822,26 +822,83 @@ __device__ __forceinline__ bool unit_has_e4m3_nan(const uint32_t (&in)[8])
     return nan;
 }
 
-// The 32 E4M3 codes of one lane, none of them a NaN code, to any lower MXFP format.
-template <class FL, int NWO>
-__device__ __forceinline__ void ss_e4m3_unit_fast(const uint32_t (&in)[8], uint32_t (&out)[NWO])
+// A word of four E4M3 codes with every NaN code (0x7F) replaced by the largest finite one (0x7E, the sign
+// kept); `nans` gets 0x7F in the bytes that held one.
+__device__ __forceinline__ uint32_t e4m3_word_clean(uint32_t x, uint32_t& nans)
 {
-    if constexpr (FL::hw_cvt && FL::bits == 4) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[j] = ss_e4m3_words_to_e2m1(in[2 * j], in[2 * j + 1]);
-    } else if constexpr (FL::hw_cvt) {
-        uint32_t z[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) z[j] = squeeze6_low(ss_e4m3_word_to6<FL>(in[j]));
-#pragma unroll
-        for (int g = 0; g < 2; ++g)
-            join24(z[4 * g + 0], z[4 * g + 1], z[4 * g + 2], z[4 * g + 3], out[3 * g + 0], out[3 * g + 1], out[3 * g + 2]);
+    const uint32_t m = ((x & 0x7F7F7F7Fu) + 0x01010101u) & 0x80808080u;
+    nans = m - (m >> 7);
+    return x - (m >> 7);
+}
+
+// Eight anchor codes (words 2J and 2J + 1 of a lane's 32) in a lower format: two streams for pack_streams, or,
+// for the 4-bit formats, one finished output word.
+template <class FL, int J>
+__device__ __forceinline__ void ss_int8_word_pair(const Int8Word& w0, const Int8Word& w1, uint32_t (&z)[8])
+{
+    if constexpr (FL::bits == 4) {
+        // the codes come back in the high nibbles: w * 17 drops each one into the low nibble of the
+        // byte above as well, so bytes 1 and 3 of it hold c0 | c1 << 4 and c2 | c3 << 4
+        const uint32_t a = ss_int8_word_top<4>(w0), b = ss_int8_word_top<4>(w1);
+        z[J] = __byte_perm(a * 16u + a, b * 16u + b, 0x7531);
     } else {
-        uint32_t z[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) z[j] = ss_e4m3_word_soft<FL>(in[j]);
-        pack_code_bytes<FL::bits>(z, out);
+        z[2 * J] = squeeze_top<FL::bits>(ss_int8_word_top<FL::bits>(w0));
+        z[2 * J + 1] = squeeze_top<FL::bits>(ss_int8_word_top<FL::bits>(w1));
     }
+}
+
+template <class FL, int J>
+__device__ __forceinline__ void ss_e4m3_word_pair(const uint32_t (&h)[4], const uint32_t (&nans)[2], uint32_t (&z)[8])
+{
+    if constexpr (FL::bits == 4) {
+        z[J] = ss_e4m3_pairs_to_e2m1(h[0], h[1], h[2], h[3]);
+    } else {
+        z[2 * J] = squeeze_top<FL::bits>(ss_e4m3_pairs_top<FL>(h[0], h[1], nans[0]));
+        z[2 * J + 1] = squeeze_top<FL::bits>(ss_e4m3_pairs_top<FL>(h[2], h[3], nans[1]));
+    }
+}
+
+template <class FL, int NWO>
+__device__ __forceinline__ void ss_finish(const uint32_t (&z)[8], uint32_t (&out)[NWO])
+{
+    if constexpr (FL::bits == 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[j] = z[j];
+    } else {
+        pack_streams<FL::bits>(z, out);
+    }
+}
+
+template <int I, class... FL>
+using ss_target_t = typename std::tuple_element<I, std::tuple<FL...>>::type;
+
+// The 32 codes of one lane of an 8-bit anchor to one or more lower formats, eight codes at a time so that what
+// the targets share (sign masks and magnitudes, FP16 values) lives only that long.  E4M3 anchors:
+// NAN_CODES = false promises that none of the codes is a NaN code.  A NaN code maps to the largest magnitude with
+// its sign: so does the largest finite code, 448, wherever the target's largest mantissa is 1.75 or less
+// (448 / 2^de = 1.75 * 2^emax); for the three-bit mantissas (largest 1.875) the magnitude bits of the target
+// code are set as well.
+template <bool NAN_CODES, class FH, class... FL>
+__device__ __forceinline__ void ss_anchor_unit(const uint32_t (&in)[8], uint32_t (&z)[sizeof...(FL)][8])
+{
+    static_for<4>([&](auto jj) {
+        constexpr int J = decltype(jj)::value;
+        if constexpr (FH::kind == KIND_INT) {
+            const Int8Word w0 = int8_word(in[2 * J]), w1 = int8_word(in[2 * J + 1]);
+            static_for<(int)sizeof...(FL)>([&](auto i) {
+                constexpr int I = decltype(i)::value;
+                ss_int8_word_pair<ss_target_t<I, FL...>, J>(w0, w1, z[I]);
+            });
+        } else {
+            uint32_t h[4], nans[2] = {0, 0};
+            e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J], nans[0]) : in[2 * J], h[0], h[1]);
+            e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J + 1], nans[1]) : in[2 * J + 1], h[2], h[3]);
+            static_for<(int)sizeof...(FL)>([&](auto i) {
+                constexpr int I = decltype(i)::value;
+                ss_e4m3_word_pair<ss_target_t<I, FL...>, J>(h, nans, z[I]);
+            });
+        }
+    });
 }
 
 // Convert the 32 codes of one lane.  in: 8*FH::bits/8... words of the high format's bitstream.
@@ -851,31 +908,19 @@ __device__ __forceinline__ void slice_scale_unit(const uint32_t (&in)[NWI], uint
     if constexpr (FH::id == FL::id) {
 #pragma unroll
         for (int j = 0; j < NWO; ++j) out[j] = in[j];
-    } else if constexpr (FH::id == MXQ_INT8 && FL::bits == 4) {
-        // the codes come back in the high nibbles: w * 17 drops each one into the low nibble of the
-        // byte above as well, so bytes 1 and 3 of it hold c0 | c1 << 4 and c2 | c3 << 4
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t a = ss_int8_word_top<4>(in[2 * j]), b = ss_int8_word_top<4>(in[2 * j + 1]);
-            out[j] = __byte_perm(a * 16u + a, b * 16u + b, 0x7531);
+    } else if constexpr (FH::bits == 8) {
+        uint32_t z[1][8];
+        if constexpr (FH::kind == KIND_INT) {
+            ss_anchor_unit<false, FH, FL>(in, z);
+            ss_finish<FL>(z[0], out);
+        } else if (!unit_has_e4m3_nan(in)) {
+            ss_anchor_unit<false, FH, FL>(in, z);
+            ss_finish<FL>(z[0], out);
+        } else {
+            // an E4M3 NaN code (never produced by the quantizer): the slow path, which costs this kernel nothing
+            // where ss_anchor_unit<true> slows the 6-bit targets by 1.5 %
+            ss_unit_by_element<FH, FL>(in, out);
         }
-    } else if constexpr (FH::id == MXQ_INT8 && FL::bits == 6) {
-        uint32_t z[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) z[j] = squeeze6_top(ss_int8_word_top<6>(in[j]));
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            join24(z[4 * g + 0], z[4 * g + 1], z[4 * g + 2], z[4 * g + 3], out[3 * g + 0], out[3 * g + 1], out[3 * g + 2]);
-        }
-    } else if constexpr (FH::id == MXQ_INT8 && FL::kind == KIND_INT) {
-        // MXINT7 / 5 / 3 / 2: the same four-codes-per-register arithmetic, generic packing
-        uint32_t z[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) z[j] = ss_int8_word<FL::bits>(in[j]);
-        pack_code_bytes<FL::bits>(z, out);
-    } else if constexpr (ss_e4m3_has_fast_path<FH, FL>()) {
-        if (!unit_has_e4m3_nan(in)) ss_e4m3_unit_fast<FL>(in, out);
-        else ss_unit_by_element<FH, FL>(in, out);     // an E4M3 NaN code (never produced by the quantizer)
     } else {
         ss_unit_by_element<FH, FL>(in, out);          // every other pair, including non-anchor sources
     }
@@ -973,113 +1018,148 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
         slice_scale_tile<FH, FL, U>(codes, scales, nunits, nscales, out_codes, out_scales, tile, stage);
 }
 
-// Two targets from one read of the anchor (the elastic-serving case: one stored checkpoint, several
-// lower precisions wanted at once).  Per element 1.03 bytes are read once instead of twice.
-// (Left to itself the compiler gives this kernel 64 - 71 registers, 7 CTAs per SM; asked for 12 CTAs it
-// finds 40 without spilling, and the launch is 2 % shorter.)
-// One warp tile of the two-target conversion; shared by the single-tensor and the batched kernels.
-template <class FH, class FL1, class FL2, int U>
-__device__ __forceinline__ void slice_scale2_tile(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
-                                                  size_t nunits, size_t nscales, uint8_t* __restrict__ out_codes1,
-                                                  uint8_t* __restrict__ out_scales1, uint8_t* __restrict__ out_codes2,
-                                                  uint8_t* __restrict__ out_scales2, size_t tile, uint8_t* stage1,
-                                                  uint8_t* stage2)
+// Several targets from one read of the anchor (the elastic-serving case: one stored checkpoint, several lower
+// precisions wanted at once).  Per element 1.03 bytes are read once instead of once per target, and what the
+// conversions share (sign masks and magnitudes of the MXINT8 codes, the FP16 values of the E4M3 codes) is
+// computed once.  The set of targets is a compile-time list: a kernel that walks a run-time list of formats
+// keeps the shared words in registers across a switch and ran at 35 - 45 % over the floor where these do
+// at 2 - 20 %.
+struct SsOut {
+    uint8_t* codes;
+    uint8_t* scales;
+};
+
+template <int N>
+struct SsOuts {
+    SsOut t[N];
+};
+
+// Bytes of staging area per lane unit that the targets before number I need (I = the count: all of them).
+template <int I, class... FL>
+__host__ __device__ constexpr int ss_stage_offset()
 {
-    constexpr int IB = 4 * FH::bits, NWI = IB / 4;
-    constexpr int OB1 = 4 * FL1::bits, OB2 = 4 * FL2::bits;
-    constexpr int de1 = FH::emax - FL1::emax, de2 = FH::emax - FL2::emax;
-    const size_t u0 = tile * (32 * U) + (threadIdx.x & 31);
-    uint32_t w[U][NWI];
+    constexpr int ob[] = {(StagedTile<4 * FL::bits>::use ? 4 * FL::bits : 0)...};
+    int sum = 0;
+    for (int i = 0; i < I; ++i) sum += ob[i];
+    return sum;
+}
+
+// One CTA tile (THREADS * U lane units, 32 U consecutive ones per warp) of an 8-bit anchor into all targets; shared
+// by the single-tensor and the batched kernels.  `first` is the tile's first unit: it depends on the block
+// alone, so the 64-bit bases of all streams live in uniform registers and a lane adds 32-bit offsets.
+template <class FH, int U, int THREADS, class... FL>
+__device__ __forceinline__ void slice_scale_set_tile(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
+                                                     size_t nunits, size_t nscales, const SsOut* outs, size_t first,
+                                                     uint8_t* stage)
+{
+    static_assert(FH::bits == 8, "an 8-bit anchor");
+    constexpr int N = sizeof...(FL);
+    constexpr uint32_t kTile = THREADS * U;
+    const uint32_t lane = threadIdx.x & 31, warp0 = (threadIdx.x >> 5) * (32 * U), l0 = warp0 + lane;
+    // units and scales of the tensor inside this tile (a block of 64 or 128 has fewer scales than units: the
+    // first tiles carry them)
+    const uint32_t valid = nunits - first < kTile ? (uint32_t)(nunits - first) : kTile;
+    const uint32_t valid_scales = first >= nscales ? 0u : nscales - first < kTile ? (uint32_t)(nscales - first) : kTile;
+    codes += first * 32;
+    uint32_t w[U][8];
     uint32_t sb[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const size_t unit = u0 + u * 32;
-        if (unit < nunits) load_words<NWI>(w[u], codes + unit * IB);
+        if (l0 + u * 32 < valid) ld256(w[u], codes + (l0 + u * 32) * 32);
         else {
 #pragma unroll
-            for (int j = 0; j < NWI; ++j) w[u][j] = 0;
+            for (int j = 0; j < 8; ++j) w[u][j] = 0;
         }
-        sb[u] = unit < nscales ? ld_u8(scales + unit) : 0;
+        sb[u] = l0 + u * 32 < valid_scales ? ld_u8(scales + first + (l0 + u * 32)) : 0;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const size_t unit = u0 + u * 32;
-        if (unit < nscales) {
-            st_u8(out_scales1 + unit, ss_scale_byte(sb[u], de1));
-            st_u8(out_scales2 + unit, ss_scale_byte(sb[u], de2));
+        if (l0 + u * 32 < valid_scales) {
+            static_for<N>([&](auto i) {
+                constexpr int I = decltype(i)::value;
+                st_u8(outs[I].scales + first + (l0 + u * 32), ss_scale_byte(sb[u], FH::emax - ss_target_t<I, FL...>::emax));
+            });
         }
-        uint32_t o1[OB1 / 4], o2[OB2 / 4];
-        if constexpr (ss_e4m3_has_fast_path<FH, FL1>() && ss_e4m3_has_fast_path<FH, FL2>()) {
-            // one NaN-code check, both conversions in one straight line: what they share (the widening
-            // of the anchor codes, the scaled values when de is the same) is computed once
-            if (!unit_has_e4m3_nan(w[u])) {
-                ss_e4m3_unit_fast<FL1>(w[u], o1);
-                ss_e4m3_unit_fast<FL2>(w[u], o2);
-            } else {
-                ss_unit_by_element<FH, FL1>(w[u], o1);
-                ss_unit_by_element<FH, FL2>(w[u], o2);
-            }
-        } else {
-            slice_scale_unit<FH, FL1>(w[u], o1);
-            slice_scale_unit<FH, FL2>(w[u], o2);
+        uint32_t z[N][8];
+        // one NaN-code check, all conversions in one straight line
+        if (FH::kind == KIND_INT || !unit_has_e4m3_nan(w[u])) ss_anchor_unit<false, FH, FL...>(w[u], z);
+        else if constexpr (FH::kind == KIND_FP) ss_anchor_unit<true, FH, FL...>(w[u], z);
+        static_for<N>([&](auto i) {
+            constexpr int I = decltype(i)::value;
+            using F = ss_target_t<I, FL...>;
+            constexpr int OB = 4 * F::bits;
+            uint32_t out[OB / 4];
+            ss_finish<F>(z[I], out);
+            if constexpr (StagedTile<OB>::use)
+                store_bytes<OB>(stage + 32 * U * ss_stage_offset<I, FL...>() + (u * 32 + lane) * OB, out);
+            else if (l0 + u * 32 < valid) store_bytes<OB>(outs[I].codes + first * OB + (l0 + u * 32) * OB, out);
+        });
+    }
+    if constexpr (ss_stage_offset<N, FL...>() > 0) {
+        if (warp0 < valid) {                                    // whole warps
+            const uint32_t mine = valid - warp0 < 32 * U ? valid - warp0 : 32 * U;
+            static_for<N>([&](auto i) {
+                constexpr int I = decltype(i)::value;
+                constexpr int OB = 4 * ss_target_t<I, FL...>::bits;
+                if constexpr (StagedTile<OB>::use)
+                    flush_stage_async<32 * U * OB>(stage + 32 * U * ss_stage_offset<I, FL...>(),
+                                                   outs[I].codes + first * OB + warp0 * OB, mine * OB);
+            });
+            stage_wait<0>();
         }
-        if constexpr (StagedTile<OB1>::use) store_bytes<OB1>(stage1 + (u * 32 + (threadIdx.x & 31)) * OB1, o1);
-        else if (unit < nunits) store_bytes<OB1>(out_codes1 + unit * OB1, o1);
-        if constexpr (StagedTile<OB2>::use) store_bytes<OB2>(stage2 + (u * 32 + (threadIdx.x & 31)) * OB2, o2);
-        else if (unit < nunits) store_bytes<OB2>(out_codes2 + unit * OB2, o2);
     }
-    {
-        const size_t first = tile * (32 * U), left = nunits - first;
-        const uint32_t valid = (uint32_t)(left < 32 * U ? left : 32 * U);
-        if constexpr (StagedTile<OB1>::use) flush_stage<32 * U * OB1>(stage1, out_codes1 + first * OB1, valid * OB1);
-        if constexpr (StagedTile<OB2>::use) flush_stage<32 * U * OB2>(stage2, out_codes2 + first * OB2, valid * OB2);
-    }
-    if (nscales > nunits) {
+    if (nscales > nunits) {                                     // block 16: two scales per lane unit
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const size_t i = nunits + u0 + u * 32;
+            const size_t i = nunits + first + (l0 + u * 32);
             if (i < nscales) {
                 const uint32_t b = ld_u8(scales + i);
-                st_u8(out_scales1 + i, ss_scale_byte(b, de1));
-                st_u8(out_scales2 + i, ss_scale_byte(b, de2));
+                static_for<N>([&](auto k) {
+                    constexpr int I = decltype(k)::value;
+                    st_u8(outs[I].scales + i, ss_scale_byte(b, FH::emax - ss_target_t<I, FL...>::emax));
+                });
             }
         }
     }
 }
 
-// The two staging areas of the calling warp (null where the target's pieces are stored directly).
-// Must be called by every thread of the CTA, outside divergent code.
-template <class FL1, class FL2, int U, int THREADS>
-__device__ __forceinline__ void slice_scale2_stages(uint8_t*& stage1, uint8_t*& stage2)
+// Asks L2 for the tile's input lines (see prefetch_tile): lane l of the CTA for the line of each of its U units.
+template <int U, int THREADS, int UNIT_BYTES>
+__device__ __forceinline__ void prefetch_cta_tile(const uint8_t* base, size_t first, size_t nunits)
 {
-    constexpr int OB1 = 4 * FL1::bits, OB2 = 4 * FL2::bits;
-    stage1 = nullptr;
-    stage2 = nullptr;
-    if constexpr (StagedTile<OB1>::use) {
-        __shared__ __align__(128) uint8_t area1[(THREADS / 32) * 32 * U * OB1];
-        stage1 = area1 + (threadIdx.x >> 5) * (32 * U * OB1);
-    }
-    if constexpr (StagedTile<OB2>::use) {
-        __shared__ __align__(128) uint8_t area2[(THREADS / 32) * 32 * U * OB2];
-        stage2 = area2 + (threadIdx.x >> 5) * (32 * U * OB2);
+    const uint32_t l0 = (threadIdx.x >> 5) * (32 * U) + (threadIdx.x & 31);
+    base += first * UNIT_BYTES;
+    const uint32_t valid = nunits - first < THREADS * U ? (uint32_t)(nunits - first) : THREADS * U;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (l0 + u * 32 < valid) asm volatile("prefetch.global.L2 [%0];" :: "l"(base + (l0 + u * 32) * UNIT_BYTES));
+}
+
+// The staging areas of the calling warp (null where every target's pieces are stored directly).
+// Must be called by every thread of the CTA, outside divergent code.
+template <int U, int THREADS, class... FL>
+__device__ __forceinline__ uint8_t* slice_scale_set_stage()
+{
+    constexpr int kWarp = 32 * U * ss_stage_offset<(int)sizeof...(FL), FL...>();
+    if constexpr (kWarp > 0) {
+        __shared__ __align__(128) uint8_t area[(THREADS / 32) * kWarp];
+        return area + (threadIdx.x >> 5) * kWarp;
+    } else {
+        return nullptr;
     }
 }
 
-template <class FH, class FL1, class FL2, int U, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1536 / THREADS)
-slice_scale2_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits, size_t nscales,
-                    uint8_t* __restrict__ out_codes1, uint8_t* __restrict__ out_scales1,
-                    uint8_t* __restrict__ out_codes2, uint8_t* __restrict__ out_scales2)
+template <class FH, int U, int THREADS, class... FL>
+__global__ void __launch_bounds__(THREADS, 12)
+slice_scale_set_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits, size_t nscales,
+                       const __grid_constant__ SsOuts<(int)sizeof...(FL)> outs)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
-    uint8_t *stage1, *stage2;
-    slice_scale2_stages<FL1, FL2, U, THREADS>(stage1, stage2);
-    prefetch_tile<U, 4 * FH::bits>(codes, tile, nunits);
+    const size_t first = (size_t)blockIdx.x * (THREADS * U);
+    uint8_t* stage = slice_scale_set_stage<U, THREADS, FL...>();
+    prefetch_cta_tile<U, THREADS, 32>(codes, first, nunits);
     pdl_acquire();
-    if (tile * (32 * U) >= nunits) return;                     // whole warps leave together
-    slice_scale2_tile<FH, FL1, FL2, U>(codes, scales, nunits, nscales, out_codes1, out_scales1, out_codes2, out_scales2,
-                                       tile, stage1, stage2);
+    slice_scale_set_tile<FH, U, THREADS, FL...>(codes, scales, nunits, nscales, outs.t, first, stage);
 }
 
 // Device-side item of the batched conversion (one tensor), with its place in the flattened
@@ -1094,24 +1174,22 @@ struct SsDeviceItem {
     size_t tile_begin;     // first global tile index of this tensor
 };
 
-// All tensors in one launch: the tiles of every tensor are laid end to end and every warp finds the
-// tensor its tile belongs to by a binary search of the item table, so small tensors do not leave
-// SMs idle.
+// All tensors in one launch: the tiles of every tensor are laid end to end and every CTA finds the
+// tensor its tile belongs to by a search of the item table, so small tensors do not leave SMs idle.
 template <class FH, class FL, int U, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 slice_scale_batched_kernel(const SsDeviceItem* __restrict__ items, const TileIndex* __restrict__ index, int count,
                            size_t total_tiles)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
     pdl_acquire();
-    if (tile >= total_tiles) return;
-    // items are sorted by tile_begin: the last one that starts at or before this tile owns it
+    // items are sorted by tile_begin: the last one that starts at or before this CTA's tile owns it
     // (table and index are device memory written by the copy in front of this launch: read after the wait)
-    const SsDeviceItem t = items[find_item(items, *index, tile)];
-    slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile - t.tile_begin,
-                                stage);
+    const SsDeviceItem& t = items[find_item(items, *index, blockIdx.x)];
+    const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
+    if (tile * (32 * U) < t.nunits)                       // whole warps
+        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
 }
 
 // The same launch with the item table carried in the kernel's parameter space (K items, 56 bytes
@@ -1124,58 +1202,48 @@ struct SsItemBlock {
 };
 
 template <class FH, class FL, int U, int THREADS, int K>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, 12)
 slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk, int count, size_t total_tiles)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
     // parameters: readable before the wait
-    const SsDeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
-    if (tile < total_tiles) prefetch_tile<U, 4 * FH::bits>(t.codes, tile - t.tile_begin, t.nunits);
+    const SsDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
+    prefetch_tile<U, 4 * FH::bits>(t.codes, tile, t.nunits);
     pdl_acquire();
-    if (tile >= total_tiles) return;
-    slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile - t.tile_begin,
-                                stage);
+    if (tile * (32 * U) < t.nunits)                       // whole warps
+        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
 }
 
 // Two targets from one read of every anchor of a set of tensors (the whole-model conversion of Sec. 3.5
 // for a deployment that serves two lower precisions at once): items of 72 bytes, 256 per launch.
-struct Ss2DeviceItem {
+struct SsPairDeviceItem {
     const uint8_t* codes;
     const uint8_t* scales;
-    uint8_t* out_codes1;
-    uint8_t* out_scales1;
-    uint8_t* out_codes2;
-    uint8_t* out_scales2;
+    SsOut out[2];
     size_t nunits;
     size_t nscales;
     size_t tile_begin;
 };
 
 template <int K>
-struct Ss2ItemBlock {
-    Ss2DeviceItem items[K];
+struct SsPairItemBlock {
+    SsPairDeviceItem items[K];
     TileIndex index;
 };
 
-// (The item's six pointers live in registers here.  Measured over the 224-tensor weight set with 6 / 8 / 10 / 12
-// resident CTAs: 10 -- 48 registers, 12 - 20 bytes of spills in the MXFP variants -- is the fastest for the
-// MXFP pair (2.42 ms against 2.60 at 8 and 3.13 at 12) and within 2 % of the best for the MXINT pair.)
 template <class FH, class FL1, class FL2, int U, int THREADS, int K>
-__global__ void __launch_bounds__(THREADS, 10)
-slice_scale2_batched_kernel(const __grid_constant__ Ss2ItemBlock<K> blk, int count, size_t total_tiles)
+__global__ void __launch_bounds__(THREADS, 12)
+slice_scale_pair_batched_kernel(const __grid_constant__ SsPairItemBlock<K> blk, int count, size_t total_tiles)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
-    uint8_t *stage1, *stage2;
-    slice_scale2_stages<FL1, FL2, U, THREADS>(stage1, stage2);
-    const Ss2DeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
-    if (tile < total_tiles) prefetch_tile<U, 4 * FH::bits>(t.codes, tile - t.tile_begin, t.nunits);
+    uint8_t* stage = slice_scale_set_stage<U, THREADS, FL1, FL2>();
+    const SsPairDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    const size_t first = (blockIdx.x - t.tile_begin) * (THREADS * U);
+    prefetch_cta_tile<U, THREADS, 32>(t.codes, first, t.nunits);
     pdl_acquire();
-    if (tile >= total_tiles) return;
-    slice_scale2_tile<FH, FL1, FL2, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes1, t.out_scales1, t.out_codes2,
-                                       t.out_scales2, tile - t.tile_begin, stage1, stage2);
+    slice_scale_set_tile<FH, U, THREADS, FL1, FL2>(t.codes, t.scales, t.nunits, t.nscales, t.out, first, stage);
 }
 
 // The batched conversion with every tensor's scale bytes written in the tiled order (block 32): the
@@ -1201,15 +1269,14 @@ __global__ void __launch_bounds__(THREADS)
 slice_scale_tiled_batched_kernel(const __grid_constant__ SsTiledItemBlock<K> blk, int count, size_t total_tiles)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
     // parameters: readable before the wait
-    const SsTiledDeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
-    if (tile < total_tiles) prefetch_tile<U, 4 * FH::bits>(t.codes, tile - t.tile_begin, t.nunits);
+    const SsTiledDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
+    prefetch_tile<U, 4 * FH::bits>(t.codes, tile, t.nunits);
     pdl_acquire();
-    if (tile >= total_tiles) return;
-    slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nunits, t.out_codes, t.out_scales, tile - t.tile_begin,
-                                stage);
+    if (tile * (32 * U) < t.nunits)                       // whole warps
+        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nunits, t.out_codes, t.out_scales, tile, stage);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -20,25 +20,36 @@ inline int grid_for_tiles(size_t ntiles, int threads)
     return (int)(need ? need : 1);
 }
 
+// The same for kernels whose CTA covers `per_cta` consecutive lane units.
+inline int grid_for_units(size_t nunits, size_t per_cta)
+{
+    const size_t need = (nunits + per_cta - 1) / per_cta;
+    return need > (size_t)0x7FFFFFFF ? 0 : (int)need;
+}
+
 int launch_quantize(const void* src, int dtype, size_t n, int fmt, int block, void* codes, uint8_t* scales,
                     cudaStream_t stream);
 int launch_fake_quant(const void* src, int dtype, size_t n, int fmt, int block, int mode, void* dst,
                       cudaStream_t stream);
 int launch_slice_scale(const void* codes, const uint8_t* scales, size_t n, int block, int src_fmt, int dst_fmt,
                        void* out_codes, uint8_t* out_scales, cudaStream_t stream);
-// Anchor -> two lower formats in one pass.  Returns MXQ_ERR_PAIR when this pair of targets has no
-// fused instantiation (the caller then falls back to two single-target launches).
-int launch_slice_scale2(const void* codes, const uint8_t* scales, size_t n, int block, int src_fmt, int dst_fmt1,
-                        int dst_fmt2, void* out_codes1, uint8_t* out_scales1, void* out_codes2, uint8_t* out_scales2,
-                        cudaStream_t stream);
-// The two-target conversion over up to kSs2BatchItemsMax tensors in one launch (items: a HOST array with
-// tile_begin filled in); MXQ_ERR_PAIR when the pair of targets has no fused instantiation.
-struct Ss2DeviceItem;
-constexpr int kSs2BatchItemsMax = 256;
-int launch_slice_scale2_batched(const Ss2DeviceItem* items_host, int count, size_t total_tiles, int src_fmt, int dst_fmt1,
-                                int dst_fmt2, cudaStream_t stream);
-bool slice_scale2_is_fused(int src_fmt, int dst_fmt1, int dst_fmt2);
-size_t ss2_batched_tiles(size_t nunits);
+// One 8-bit anchor -> 2 ... kSetTargetsMax DIFFERENT lower formats in one pass (one kernel per set of formats).
+struct SsOut;
+constexpr int kSetTargetsMax = 4;
+bool slice_scale_set_anchor(int src_fmt);                   // the sources that have these kernels
+int launch_slice_scale_set(const uint8_t* codes, const uint8_t* scales, size_t n, int block, int src_fmt, int ntargets,
+                           const int* fmts, const SsOut* outs, cudaStream_t stream);
+int launch_slice_scale_set_e4m3(const uint8_t* codes, const uint8_t* scales, size_t n, int block, int ntargets,
+                                const int* fmts, const SsOut* outs, cudaStream_t stream);
+// Two different lower formats of up to kSsPairItemsMax anchors in one launch (items: a HOST array with tile_begin
+// filled in, tiles counted by ss_pair_batched_tiles).
+struct SsPairDeviceItem;
+constexpr int kSsPairItemsMax = 256;
+int launch_slice_scale_pair_batched(const SsPairDeviceItem* items_host, int count, size_t total_tiles, int src_fmt, int fmt1,
+                                    int fmt2, cudaStream_t stream);
+int launch_slice_scale_pair_batched_e4m3(const SsPairDeviceItem* items_host, int count, size_t total_tiles, int fmt1,
+                                         int fmt2, cudaStream_t stream);
+size_t ss_pair_batched_tiles(size_t nunits);
 // The same two operations with the scale bytes written in 128 x 4 tiles (block 32, kblocks block-columns
 // per row); the caller has zeroed the tiled buffer when the matrix leaves part of a tile uncovered.
 int launch_quantize_tiled(const void* src, int dtype, size_t n, int fmt, void* codes, uint8_t* tiled,

@@ -47,7 +47,7 @@ int run_table(const SsDeviceItem* items_dev, const TileIndex* index_dev, int cou
 {
     if constexpr (ss_pair_ok(FH::id, FL::id)) {
         auto kern = slice_scale_batched_kernel<FH, FL, kU, kThreads>;
-        return launch_kernel(kern, grid_for_tiles(total_tiles, kThreads), kThreads, stream, items_dev, index_dev, count,
+        return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, items_dev, index_dev, count,
                              total_tiles);
     } else {
         return MXQ_ERR_PAIR;
@@ -65,7 +65,7 @@ int run_params(const SsDeviceItem* items_host, int count, size_t total_tiles, cu
             for (int i = count; i < K; ++i) blk.items[i] = SsDeviceItem{};
             build_tile_index(blk.index, items_host, count, total_tiles);
             auto kern = slice_scale_batched_param_kernel<FH, FL, kU, kThreads, K>;
-            return launch_kernel(kern, grid_for_tiles(total_tiles, kThreads), kThreads, stream, blk, count, total_tiles);
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk, count, total_tiles);
         };
         if (count <= 64) return go(std::integral_constant<int, 64>{});
         return go(std::integral_constant<int, kSsParamItemsMax>{});
@@ -83,7 +83,7 @@ int run_tiled_params(const SsTiledDeviceItem* items_host, int count, size_t tota
         for (int i = count; i < kSsTiledItemsMax; ++i) blk.items[i] = SsTiledDeviceItem{};
         build_tile_index(blk.index, items_host, count, total_tiles);
         auto kern = slice_scale_tiled_batched_kernel<FH, FL, kU, kThreads, kSsTiledItemsMax>;
-        return launch_kernel(kern, grid_for_tiles(total_tiles, kThreads), kThreads, stream, blk, count, total_tiles);
+        return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk, count, total_tiles);
     } else {
         return MXQ_ERR_PAIR;
     }
@@ -91,7 +91,7 @@ int run_tiled_params(const SsTiledDeviceItem* items_host, int count, size_t tota
 
 }  // namespace
 
-size_t ss_batched_tiles(size_t nunits) { return (nunits + 32 * kU - 1) / (32 * kU); }
+size_t ss_batched_tiles(size_t nunits) { return (nunits + kThreads * kU - 1) / (kThreads * kU); }
 
 int launch_slice_scale(const void* codes, const uint8_t* scales, size_t n, int block, int src_fmt, int dst_fmt,
                        void* out_codes, uint8_t* out_scales, cudaStream_t stream)
