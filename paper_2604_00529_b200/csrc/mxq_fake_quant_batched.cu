@@ -6,8 +6,8 @@ namespace mxq {
 namespace {
 
 constexpr int kU = 1;
-// consecutive warp tiles of one tensor per warp: 2 amortises the tensor lookup (the whole weight set to
-// MXINT4 through the anchor 4.29 -> 4.00 ms, to E2M1 4.17 -> 4.02 ms, to E2M3 unchanged); 4 is slower again
+// Consecutive warp tiles of one tensor per warp: 1 / 2 / 4 take 996 / 1013 / 1098 us (FP32, MXINT4 through the anchor),
+// 547 / 498 / 542 us (BF16, the same) and 539 / 499 / 543 us (BF16, E2M3) over four decoder layers.
 constexpr int kR = 2;
 constexpr int kThreads = 128;
 
@@ -17,12 +17,13 @@ int run(const FqDeviceItem* items_host, int count, size_t total_tiles, cudaStrea
     if constexpr (BLOCK < T::epl) {
         return MXQ_ERR_BLOCK;
     } else {
-        FqItemBlock<kFqBatchItemsMax> blk;
-        for (int i = 0; i < count; ++i) blk.items[i] = items_host[i];
-        for (int i = count; i < kFqBatchItemsMax; ++i) blk.items[i] = FqDeviceItem{};
-        build_tile_index(blk.index, items_host, count, total_tiles);
-        auto kern = fake_quant_batched_kernel<T, F, BLOCK, MODE, kU, kR, kThreads, kFqBatchItemsMax>;
-        return launch_kernel(kern, grid_for_tiles(total_tiles, kThreads), kThreads, stream, blk, count, total_tiles);
+        return with_item_capacity<kFqBatchItemsMax>(count, [&](auto k) {
+            constexpr int K = decltype(k)::value;
+            FqItemBlock<K> blk;
+            fill_item_block(blk, items_host, count, total_tiles);
+            auto kern = fake_quant_batched_kernel<T, F, BLOCK, MODE, kU, kR, kThreads, K>;
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
+        });
     }
 }
 
@@ -49,12 +50,11 @@ int by_mode(int mode, int block, const FqDeviceItem* items_host, int count, size
 
 }  // namespace
 
-size_t fq_batched_tiles(size_t nunits) { return (nunits + 32 * kU * kR - 1) / (32 * kU * kR); }
+size_t fq_batched_tiles(size_t nunits) { return (nunits + kThreads * kU * kR - 1) / (kThreads * kU * kR); }
 
 int launch_fake_quant_batched(const FqDeviceItem* items_host, int count, size_t total_tiles, int dtype, int fmt,
                               int block, int mode, cudaStream_t stream)
 {
-    if (count > kFqBatchItemsMax) return MXQ_ERR_SIZE;
     MXQ_DISPATCH_FORMAT(fmt, {
         if (dtype == MXQ_F32) return by_mode<F32, F>(mode, block, items_host, count, total_tiles, stream);
         return by_mode<BF16, F>(mode, block, items_host, count, total_tiles, stream);

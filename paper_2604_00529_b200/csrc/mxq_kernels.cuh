@@ -545,10 +545,9 @@ fake_quant_kernel(const uint8_t* src, size_t nunits, uint8_t* dst)   // dst may 
 
 // Which tensor of a batch owns a tile.  The batched kernels lay the tiles of all tensors end to end;
 // the items (sorted by tile_begin) ride in the kernel parameters.  A plain binary search over a few
-// hundred items costs eight dependent constant-memory reads and some fifty instructions per warp
-// tile, 10 - 20 % of such a kernel.  The host therefore adds a coarse index: the tile space is cut
-// into at most 256 segments of 2^shift tiles, coarse[k] is the item that owns the first tile of
-// segment k (coarse[last + 1] the last item), and a tile's owner lies between the entries of its
+// hundred items costs eight dependent constant-memory reads.  The host therefore adds a coarse index: the
+// tile space is cut into at most 256 segments of 2^shift tiles, coarse[k] is the item that owns the first
+// tile of segment k (coarse[last + 1] the last item), and a tile's owner lies between the entries of its
 // segment's two ends -- usually the same item or neighbours, so the search that remains takes zero
 // to two steps.
 struct TileIndex {
@@ -587,7 +586,8 @@ __host__ __device__ __forceinline__ int find_item(const ITEM* items, const TileI
 
 // A tile of the batched kernels is what one CTA converts, THREADS / 32 consecutive warp tiles of ONE tensor: the owner
 // is found once per CTA from the block index, by uniform instructions, and the tensor's pointers live in uniform
-// registers.  (With a lookup per warp tile they took two registers each in every lane.)  The calling warp's
+// registers.  (With a lookup per warp tile they took two registers each in every lane: MXINT8 -> MXINT4 over four
+// decoder layers 219 -> 208 us, BF16 -> MXINT8 over eight 840 -> 804 us with one lookup per CTA.)  The calling warp's
 // tile in the tensor that starts at CTA tile `tile_begin`:
 template <int THREADS>
 __device__ __forceinline__ size_t item_warp_tile(size_t tile_begin)
@@ -612,21 +612,16 @@ struct FqItemBlock {
 
 template <class T, class F, int BLOCK, int MODE, int U, int R, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS, 14)
-fake_quant_batched_kernel(const __grid_constant__ FqItemBlock<K> blk, int count, size_t total_tiles)
+fake_quant_batched_kernel(const __grid_constant__ FqItemBlock<K> blk)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     // the item table is a kernel parameter, so the lookup may run before the dependency wait
-    const FqDeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
-    // A tile of the batch is R consecutive warp tiles of ONE tensor, converted one after the other: the
-    // lookup above (some 25 instructions per thread) is paid once per R * 32 * U lane units.
-    const size_t first = (tile - t.tile_begin) * R;
-    if (tile < total_tiles) {
+    const FqDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    // a warp converts R consecutive warp tiles of the tensor, one after the other
+    const size_t first = item_warp_tile<THREADS>(t.tile_begin) * R;
 #pragma unroll
-        for (int r = 0; r < R; ++r) prefetch_tile<U, 32>(t.src, first + r, t.nunits);
-    }
+    for (int r = 0; r < R; ++r) prefetch_tile<U, 32>(t.src, first + r, t.nunits);
     pdl_acquire();
-    if (tile >= total_tiles) return;                      // whole warps leave together
 #pragma unroll 1
     for (int r = 0; r < R; ++r)
         if ((first + r) * (32 * U) < t.nunits) fake_quant_tile<T, F, BLOCK, MODE, U>(t.src, t.nunits, t.dst, first + r);
@@ -650,16 +645,17 @@ struct QItemBlock {
 
 template <class T, class F, int BLOCK, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS, 14)     // 14 resident CTAs: the MXINT8 anchor of the 224-tensor set 3.01 ms against 3.30
-quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk, int count, size_t total_tiles)
+quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     uint8_t* stage = quantize_stage<T, F, U, THREADS>();
-    const QDeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
-    if (tile < total_tiles) prefetch_tile<U, 32>(t.src, tile - t.tile_begin, t.nunits);
+    // the item table is a kernel parameter, so the lookup may run before the dependency wait
+    const QDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
+    prefetch_tile<U, 32>(t.src, tile, t.nunits);
     pdl_acquire();
-    if (tile >= total_tiles) return;                      // whole warps leave together
-    quantize_tile<T, F, BLOCK, U>(t.src, t.nunits, t.codes, t.scales, tile - t.tile_begin, stage);
+    if (tile * (32 * U) < t.nunits)                       // whole warps
+        quantize_tile<T, F, BLOCK, U>(t.src, t.nunits, t.codes, t.scales, tile, stage);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1022,8 +1018,9 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
 // precisions wanted at once).  Per element 1.03 bytes are read once instead of once per target, and what the
 // conversions share (sign masks and magnitudes of the MXINT8 codes, the FP16 values of the E4M3 codes) is
 // computed once.  The set of targets is a compile-time list: a kernel that walks a run-time list of formats
-// keeps the shared words in registers across a switch and ran at 35 - 45 % over the floor where these do
-// at 2 - 20 %.
+// keeps the shared words in registers across a switch and took 38 - 46 us for MXINT8 -> {7, 5, 3} bits of 2^25.8
+// codes (block 64) where these take 31 (a pass per target: 53; the bytes alone: 26).  Compiled for 12 resident
+// CTAs (40 registers): 10 take 32 us, 14 spill and take 33, one unit per lane at 16 CTAs takes 35.
 struct SsOut {
     uint8_t* codes;
     uint8_t* scales;
@@ -1178,8 +1175,7 @@ struct SsDeviceItem {
 // tensor its tile belongs to by a search of the item table, so small tensors do not leave SMs idle.
 template <class FH, class FL, int U, int THREADS>
 __global__ void __launch_bounds__(THREADS)
-slice_scale_batched_kernel(const SsDeviceItem* __restrict__ items, const TileIndex* __restrict__ index, int count,
-                           size_t total_tiles)
+slice_scale_batched_kernel(const SsDeviceItem* __restrict__ items, const TileIndex* __restrict__ index)
 {
     pdl_release();
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
@@ -1203,7 +1199,7 @@ struct SsItemBlock {
 
 template <class FH, class FL, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS, 12)
-slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk, int count, size_t total_tiles)
+slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
 {
     pdl_release();
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
@@ -1235,7 +1231,7 @@ struct SsPairItemBlock {
 
 template <class FH, class FL1, class FL2, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS, 12)
-slice_scale_pair_batched_kernel(const __grid_constant__ SsPairItemBlock<K> blk, int count, size_t total_tiles)
+slice_scale_pair_batched_kernel(const __grid_constant__ SsPairItemBlock<K> blk)
 {
     pdl_release();
     uint8_t* stage = slice_scale_set_stage<U, THREADS, FL1, FL2>();
@@ -1266,7 +1262,7 @@ struct SsTiledItemBlock {
 
 template <class FH, class FL, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS)
-slice_scale_tiled_batched_kernel(const __grid_constant__ SsTiledItemBlock<K> blk, int count, size_t total_tiles)
+slice_scale_tiled_batched_kernel(const __grid_constant__ SsTiledItemBlock<K> blk)
 {
     pdl_release();
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
@@ -1478,16 +1474,15 @@ struct DqItemBlock {
 
 template <class F, class T, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS)
-dequantize_batched_kernel(const __grid_constant__ DqItemBlock<K> blk, int count, size_t total_tiles, int shift,
-                          int scales_per_unit)
+dequantize_batched_kernel(const __grid_constant__ DqItemBlock<K> blk, int shift, int scales_per_unit)
 {
     pdl_release();
-    const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
-    const DqDeviceItem& t = blk.items[tile < total_tiles ? find_item(blk.items, blk.index, tile) : 0];
+    const DqDeviceItem& t = blk.items[find_item(blk.items, blk.index, blockIdx.x)];
+    const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
     pdl_acquire();
-    if (tile >= total_tiles) return;
-    if constexpr (T::size == 4) dequantize_wide_tile<F, T, U>(t.codes, t.scales, t.nunits, shift, t.dst, tile - t.tile_begin);
-    else dequantize_tile<F, T, U>(t.codes, t.scales, t.nunits, shift, scales_per_unit, t.dst, tile - t.tile_begin);
+    if (tile * (32 * U) >= t.nunits) return;              // whole warps
+    if constexpr (T::size == 4) dequantize_wide_tile<F, T, U>(t.codes, t.scales, t.nunits, shift, t.dst, tile);
+    else dequantize_tile<F, T, U>(t.codes, t.scales, t.nunits, shift, scales_per_unit, t.dst, tile);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -3,6 +3,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "../../include/mxq.h"
@@ -100,6 +101,28 @@ int launch_slice_scale_tiled_batched(const SsTiledDeviceItem* items_host, int co
 // tiles one tensor of `nunits` lane units occupies in the batched kernel's tile space
 size_t ss_batched_tiles(size_t nunits);
 
+// Item tables ride in the kernel parameters, and a launch pays for their size (host time per launch on the B200
+// box: 2.3 us with 64 bytes of parameters, 2.4 with 4 KB, 3.6 with 16 KB, 5.0 - 5.5 with 32 KB).  So every batched
+// kernel exists with a small table, for the sets of a few layers, and with the largest one.
+constexpr int kSmallBatchItems = 64;
+template <int KMAX, class FN>
+inline int with_item_capacity(int count, FN&& fn)
+{
+    if (count > KMAX) return MXQ_ERR_SIZE;
+    if (count <= kSmallBatchItems) return fn(std::integral_constant<int, kSmallBatchItems>{});
+    return fn(std::integral_constant<int, KMAX>{});
+}
+
+// The table block of a batched kernel: `count` items (a HOST array with tile_begin filled in) and the tile index.
+template <class BLK, class ITEM>
+inline void fill_item_block(BLK& blk, const ITEM* items, int count, size_t total_tiles)
+{
+    constexpr int K = (int)(sizeof(blk.items) / sizeof(blk.items[0]));
+    for (int i = 0; i < count; ++i) blk.items[i] = items[i];
+    for (int i = count; i < K; ++i) blk.items[i] = ITEM{};
+    build_tile_index(blk.index, items, count, total_tiles);
+}
+
 // Expands the body once per element format with NAME bound to mxq::Fmt<id>.
 #define MXQ_DISPATCH_FORMAT_AS(fmt, NAME, ...)                                      \
     switch (fmt) {                                                                  \
@@ -123,7 +146,7 @@ size_t ss_batched_tiles(size_t nunits);
 // Launches `kern` on `stream` with programmatic stream serialization allowed (see pdl_release /
 // pdl_acquire in mxq_access.cuh).  Returns MXQ_OK or MXQ_ERR_CUDA.
 template <class... KArgs, class... Args>
-inline int launch_kernel(void (*kern)(KArgs...), int grid, int threads, cudaStream_t stream, Args... args)
+inline int launch_kernel(void (*kern)(KArgs...), int grid, int threads, cudaStream_t stream, const Args&... args)
 {
     if (grid <= 0) return MXQ_ERR_SIZE;
 #ifdef MXQ_DEBUG
@@ -142,7 +165,12 @@ inline int launch_kernel(void (*kern)(KArgs...), int grid, int threads, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) {
+    // (the arguments go by address: an item table is copied once, into the launch itself)
+    auto launch = [&](const KArgs&... a) {
+        void* p[] = {const_cast<void*>(static_cast<const void*>(&a))...};
+        return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), p);
+    };
+    if (launch(args...) != cudaSuccess) {
         (void)cudaGetLastError();
         return MXQ_ERR_CUDA;
     }

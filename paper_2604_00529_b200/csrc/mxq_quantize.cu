@@ -42,12 +42,13 @@ int run_batched(const QDeviceItem* items_host, int count, size_t total_tiles, cu
     if constexpr (BLOCK < T::epl) {
         return MXQ_ERR_BLOCK;
     } else {
-        QItemBlock<kQBatchItemsMax> blk;
-        for (int i = 0; i < count; ++i) blk.items[i] = items_host[i];
-        for (int i = count; i < kQBatchItemsMax; ++i) blk.items[i] = QDeviceItem{};
-        build_tile_index(blk.index, items_host, count, total_tiles);
-        auto kern = quantize_batched_kernel<T, F, BLOCK, kU, kThreads, kQBatchItemsMax>;
-        return launch_kernel(kern, grid_for_tiles(total_tiles, kThreads), kThreads, stream, blk, count, total_tiles);
+        return with_item_capacity<kQBatchItemsMax>(count, [&](auto k) {
+            constexpr int K = decltype(k)::value;
+            QItemBlock<K> blk;
+            fill_item_block(blk, items_host, count, total_tiles);
+            auto kern = quantize_batched_kernel<T, F, BLOCK, kU, kThreads, K>;
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
+        });
     }
 }
 
@@ -90,12 +91,11 @@ int launch_quantize_tiled(const void* src, int dtype, size_t n, int fmt, void* c
     return MXQ_ERR_FORMAT;
 }
 
-size_t q_batched_tiles(size_t nunits) { return (nunits + 32 * kU - 1) / (32 * kU); }
+size_t q_batched_tiles(size_t nunits) { return (nunits + kThreads * kU - 1) / (kThreads * kU); }
 
 int launch_quantize_batched(const QDeviceItem* items_host, int count, size_t total_tiles, int dtype, int fmt, int block,
                             cudaStream_t stream)
 {
-    if (count > kQBatchItemsMax) return MXQ_ERR_SIZE;
     MXQ_DISPATCH_FORMAT(fmt, {
         if (dtype == MXQ_F32) return batched_by_block<F32, F>(block, items_host, count, total_tiles, stream);
         return batched_by_block<BF16, F>(block, items_host, count, total_tiles, stream);

@@ -47,8 +47,7 @@ int run_table(const SsDeviceItem* items_dev, const TileIndex* index_dev, int cou
 {
     if constexpr (ss_pair_ok(FH::id, FL::id)) {
         auto kern = slice_scale_batched_kernel<FH, FL, kU, kThreads>;
-        return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, items_dev, index_dev, count,
-                             total_tiles);
+        return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, items_dev, index_dev);
     } else {
         return MXQ_ERR_PAIR;
     }
@@ -58,17 +57,13 @@ template <class FH, class FL>
 int run_params(const SsDeviceItem* items_host, int count, size_t total_tiles, cudaStream_t stream)
 {
     if constexpr (ss_pair_ok(FH::id, FL::id)) {
-        auto go = [&](auto k) {
+        return with_item_capacity<kSsParamItemsMax>(count, [&](auto k) {
             constexpr int K = decltype(k)::value;
             SsItemBlock<K> blk;
-            for (int i = 0; i < count; ++i) blk.items[i] = items_host[i];
-            for (int i = count; i < K; ++i) blk.items[i] = SsDeviceItem{};
-            build_tile_index(blk.index, items_host, count, total_tiles);
+            fill_item_block(blk, items_host, count, total_tiles);
             auto kern = slice_scale_batched_param_kernel<FH, FL, kU, kThreads, K>;
-            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk, count, total_tiles);
-        };
-        if (count <= 64) return go(std::integral_constant<int, 64>{});
-        return go(std::integral_constant<int, kSsParamItemsMax>{});
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
+        });
     } else {
         return MXQ_ERR_PAIR;
     }
@@ -78,12 +73,13 @@ template <class FH, class FL>
 int run_tiled_params(const SsTiledDeviceItem* items_host, int count, size_t total_tiles, cudaStream_t stream)
 {
     if constexpr (ss_pair_ok(FH::id, FL::id) && FL::kind == KIND_FP) {
-        SsTiledItemBlock<kSsTiledItemsMax> blk;
-        for (int i = 0; i < count; ++i) blk.items[i] = items_host[i];
-        for (int i = count; i < kSsTiledItemsMax; ++i) blk.items[i] = SsTiledDeviceItem{};
-        build_tile_index(blk.index, items_host, count, total_tiles);
-        auto kern = slice_scale_tiled_batched_kernel<FH, FL, kU, kThreads, kSsTiledItemsMax>;
-        return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk, count, total_tiles);
+        return with_item_capacity<kSsTiledItemsMax>(count, [&](auto k) {
+            constexpr int K = decltype(k)::value;
+            SsTiledItemBlock<K> blk;
+            fill_item_block(blk, items_host, count, total_tiles);
+            auto kern = slice_scale_tiled_batched_kernel<FH, FL, kU, kThreads, K>;
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
+        });
     } else {
         return MXQ_ERR_PAIR;
     }
@@ -115,7 +111,6 @@ int launch_slice_scale_tiled(const void* codes, const uint8_t* scales, size_t n,
 int launch_slice_scale_tiled_batched(const SsTiledDeviceItem* items_host, int count, size_t total_tiles, int src_fmt,
                                      int dst_fmt, cudaStream_t stream)
 {
-    if (count > kSsTiledItemsMax) return MXQ_ERR_SIZE;
     MXQ_DISPATCH_FORMAT_AS(src_fmt, FH, {
         MXQ_DISPATCH_FORMAT_AS(dst_fmt, FL, { return run_tiled_params<FH, FL>(items_host, count, total_tiles, stream); });
     });
@@ -134,7 +129,6 @@ int launch_slice_scale_batched(const SsDeviceItem* items_dev, const TileIndex* i
 int launch_slice_scale_batched_params(const SsDeviceItem* items_host, int count, size_t total_tiles, int src_fmt,
                                       int dst_fmt, cudaStream_t stream)
 {
-    if (count > kSsParamItemsMax) return MXQ_ERR_SIZE;
     MXQ_DISPATCH_FORMAT_AS(src_fmt, FH, {
         MXQ_DISPATCH_FORMAT_AS(dst_fmt, FL, { return run_params<FH, FL>(items_host, count, total_tiles, stream); });
     });

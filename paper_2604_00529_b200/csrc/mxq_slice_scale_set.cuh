@@ -107,17 +107,16 @@ template <class FH, unsigned MASK>
 int run_pair_batched(const SsPairDeviceItem* items_host, int count, size_t total_tiles, bool swap, cudaStream_t stream)
 {
     if constexpr (set_size(MASK) == 2) {
-        SsPairItemBlock<kSsPairItemsMax> blk;
-        for (int i = 0; i < count; ++i) {
-            blk.items[i] = items_host[i];
-            if (swap) std::swap(blk.items[i].out[0], blk.items[i].out[1]);
-        }
-        for (int i = count; i < kSsPairItemsMax; ++i) blk.items[i] = SsPairDeviceItem{};
-        build_tile_index(blk.index, items_host, count, total_tiles);
-        auto kern = slice_scale_pair_batched_kernel<FH, Fmt<SetFormats<FH>::fmt[set_member(MASK, 0)]>,
-                                                    Fmt<SetFormats<FH>::fmt[set_member(MASK, 1)]>, kSetU, kSetThreads,
-                                                    kSsPairItemsMax>;
-        return launch_kernel(kern, grid_for_units(total_tiles, 1), kSetThreads, stream, blk, count, total_tiles);
+        return with_item_capacity<kSsPairItemsMax>(count, [&](auto k) {
+            constexpr int K = decltype(k)::value;
+            SsPairItemBlock<K> blk;
+            fill_item_block(blk, items_host, count, total_tiles);
+            if (swap)
+                for (int i = 0; i < count; ++i) std::swap(blk.items[i].out[0], blk.items[i].out[1]);
+            auto kern = slice_scale_pair_batched_kernel<FH, Fmt<SetFormats<FH>::fmt[set_member(MASK, 0)]>,
+                                                        Fmt<SetFormats<FH>::fmt[set_member(MASK, 1)]>, kSetU, kSetThreads, K>;
+            return launch_kernel(kern, grid_for_units(total_tiles, 1), kSetThreads, stream, blk);
+        });
     } else {
         return MXQ_ERR_PAIR;
     }
@@ -135,7 +134,6 @@ int launch_pair_batched(const SsPairDeviceItem* items_host, int count, size_t to
                         cudaStream_t stream)
 {
     static constexpr auto table = pair_table<FH>(std::make_index_sequence<(size_t)1 << SetFormats<FH>::count>{});
-    if (count > kSsPairItemsMax) return MXQ_ERR_SIZE;
     const int a = set_index<FH>(fmt1), b = set_index<FH>(fmt2);
     if (a < 0 || b < 0 || a == b) return MXQ_ERR_PAIR;
     return table[1u << a | 1u << b](items_host, count, total_tiles, a > b, stream);
