@@ -197,8 +197,7 @@ int mxq_tile_scales(const uint8_t *scales, size_t rows, size_t kblocks, uint8_t 
  * pass.  The element codes are the same plain packed streams.  MXFP formats only (the formats the
  * block-scaled multiply takes; MXQ_ERR_FORMAT otherwise), block == 32 only (MXQ_ERR_BLOCK), cols a
  * multiple of 32 and rows * cols / 32 below 2^32 (MXQ_ERR_SIZE).  When rows is not a multiple of 128
- * or cols / 32 not a multiple of 4, the tiled buffer is first cleared on `stream`, so that the
- * uncovered part of the edge tiles reads 0.
+ * or cols / 32 not a multiple of 4, the kernel also writes the uncovered part of the edge tiles, as 0.
  *   src / codes, scales   [in]  device, as for mxq_quantize / mxq_slice_scale (plain stored scales)
  *   codes / out_codes     [out] device, mxq_codes_bytes(rows * cols, fmt) bytes, 32-byte aligned
  *   tiled_scales          [out] device, mxq_tiled_scales_bytes(rows, cols / 32) bytes, 16-byte aligned
@@ -320,7 +319,7 @@ int mxq_slice_scale_pair_batched(const mxq_ss_pair_item *items, int count, int b
  * multiplies): item i is a row-major [rows, cols] matrix, and its results are those of
  * mxq_slice_scale_tiled on it.  MXFP formats and block == 32 only, as there.  The items travel in
  * the kernel's parameter space, 256 per launch (more items: more launches); nothing is allocated.
- * Tiled buffers of matrices that do not cover whole tiles are cleared on `stream` first.
+ * The uncovered part of edge tiles is written as 0 by the same launch.
  */
 typedef struct mxq_ss_tiled_item {
     const void *codes;            /* [in]  device, anchor codes of rows * cols elements */

@@ -88,6 +88,12 @@ __device__ __forceinline__ void st_u8(uint8_t* p, uint32_t v)
     *p = (uint8_t)v;
 }
 
+__device__ __forceinline__ void st_u32(uint8_t* p, uint32_t v)          // p 4-byte aligned
+{
+    MXQ_CHECKED(p, 4, return)
+    *reinterpret_cast<uint32_t*>(p) = v;
+}
+
 // ---- compile-time sized pieces --------------------------------------------------------------
 
 // Largest power of two (<= 32) dividing `bytes`: the alignment every lane's piece keeps when

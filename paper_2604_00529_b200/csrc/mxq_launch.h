@@ -52,7 +52,7 @@ int launch_slice_scale_pair_batched_e4m3(const SsPairDeviceItem* items_host, int
                                          int fmt2, cudaStream_t stream);
 size_t ss_pair_batched_tiles(size_t nunits);
 // The same two operations with the scale bytes written in 128 x 4 tiles (block 32, kblocks block-columns
-// per row); the caller has zeroed the tiled buffer when the matrix leaves part of a tile uncovered.
+// per row; bytes of a tile that the matrix does not cover are written as 0).
 int launch_quantize_tiled(const void* src, int dtype, size_t n, int fmt, void* codes, uint8_t* tiled,
                           uint32_t kblocks, cudaStream_t stream);
 int launch_slice_scale_tiled(const void* codes, const uint8_t* scales, size_t n, int src_fmt, int dst_fmt,
@@ -100,6 +100,7 @@ int launch_slice_scale_tiled_batched(const SsTiledDeviceItem* items_host, int co
                                      int dst_fmt, cudaStream_t stream);
 // tiles one tensor of `nunits` lane units occupies in the batched kernel's tile space
 size_t ss_batched_tiles(size_t nunits);
+size_t ss_tiled_batched_tiles(const SsTiledDeviceItem& item);      // the same with the padding of its scale tiles
 
 // Item tables ride in the kernel parameters, and a launch pays for their size (host time per launch on the B200
 // box: 2.3 us with 64 bytes of parameters, 2.4 with 4 KB, 3.6 with 16 KB, 5.0 - 5.5 with 32 KB).  So every batched

@@ -71,17 +71,6 @@ int check_tiled(size_t rows, size_t cols, int block, size_t* n, uint32_t* kblock
     return MXQ_OK;
 }
 
-// Tiles that the matrix covers only in part keep byte 0 where no block lands: clear the buffer first.
-int clear_partial_tiles(uint8_t* tiled, size_t rows, size_t kblocks, cudaStream_t s)
-{
-    if (rows % 128 == 0 && kblocks % 4 == 0) return MXQ_OK;
-    if (cudaMemsetAsync(tiled, 0, tiled_bytes(rows, kblocks), s) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return MXQ_ERR_CUDA;
-    }
-    return MXQ_OK;
-}
-
 }  // namespace
 
 }  // namespace mxq
@@ -120,7 +109,6 @@ int mxq_quantize_tiled(const void* src, int src_dtype, size_t rows, size_t cols,
     if (!src || !codes || !tiled_scales) return MXQ_ERR_NULL;
     if (!aligned(src, 32) || !aligned(codes, 32) || !aligned(tiled_scales, 16)) return MXQ_ERR_ALIGN;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (int rc = clear_partial_tiles(tiled_scales, rows, kblocks, s)) return rc;
     MXQ_DEBUG_SCOPE();
     MXQ_DEBUG_EXPECT(src, n * (src_dtype == MXQ_F32 ? 4u : 2u));
     MXQ_DEBUG_EXPECT(codes, n * (size_t)fmt_info(fmt).bits / 8);
@@ -141,7 +129,6 @@ int mxq_slice_scale_tiled(const void* codes, const uint8_t* scales, size_t rows,
     if (!aligned(codes, 32) || !aligned(out_codes, 32) || !aligned(scales, 16) || !aligned(out_tiled_scales, 16))
         return MXQ_ERR_ALIGN;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (int rc = clear_partial_tiles(out_tiled_scales, rows, kblocks, s)) return rc;
     MXQ_DEBUG_SCOPE();
     MXQ_DEBUG_EXPECT(codes, n * (size_t)fmt_info(src_fmt).bits / 8);
     MXQ_DEBUG_EXPECT(scales, n / 32);
@@ -194,15 +181,14 @@ int mxq_slice_scale_tiled_batched(const mxq_ss_tiled_item* items, int count, int
         const mxq_ss_tiled_item& it = items[i];
         if (it.rows == 0 || it.cols == 0) continue;
         const uint32_t kblocks = (uint32_t)(it.cols / 32);
-        if (int rc = clear_partial_tiles(it.out_tiled_scales, it.rows, kblocks, s)) return rc;
         SsTiledDeviceItem d;
         d.codes = static_cast<const uint8_t*>(it.codes);
         d.scales = it.scales;
         d.out_codes = static_cast<uint8_t*>(it.out_codes);
-        d.out_scales = make_tiled_scales(it.out_tiled_scales, kblocks);
+        d.out_scales = make_tiled_scales(it.out_tiled_scales, kblocks, (uint32_t)it.rows);
         d.nunits = it.rows * it.cols / 32;
         d.tile_begin = tiles;
-        tiles += ss_batched_tiles(d.nunits);
+        tiles += ss_tiled_batched_tiles(d);
         chunk.push_back(d);
         if ((int)chunk.size() == kSsTiledItemsMax)
             if (int rc = flush()) return rc;

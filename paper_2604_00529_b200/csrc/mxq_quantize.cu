@@ -70,8 +70,8 @@ int run_tiled(const void* src, size_t n, void* codes, const TiledScales& tiled, 
     if constexpr (F::kind == KIND_FP) {
         auto kern = quantize_kernel<T, F, 32, kU, kThreads, TiledScales>;
         const size_t nunits = n / T::epl;
-        const size_t ntiles = (nunits + 32 * kU - 1) / (32 * kU);
-        return launch_kernel(kern, grid_for_tiles(ntiles, kThreads), kThreads, stream,
+        const size_t ctas = (nunits + kThreads * kU - 1) / (kThreads * kU) + tiled_pad_ctas(tiled, kThreads);
+        return launch_kernel(kern, grid_for_units(ctas, 1), kThreads, stream,
                              static_cast<const uint8_t*>(src), nunits, static_cast<uint8_t*>(codes), tiled);
     } else {
         return MXQ_ERR_FORMAT;
@@ -83,7 +83,7 @@ int run_tiled(const void* src, size_t n, void* codes, const TiledScales& tiled, 
 int launch_quantize_tiled(const void* src, int dtype, size_t n, int fmt, void* codes, uint8_t* tiled,
                           uint32_t kblocks, cudaStream_t stream)
 {
-    const TiledScales sink = make_tiled_scales(tiled, kblocks);
+    const TiledScales sink = make_tiled_scales(tiled, kblocks, (uint32_t)(n / 32 / kblocks));
     MXQ_DISPATCH_FORMAT(fmt, {
         if (dtype == MXQ_F32) return run_tiled<F32, F>(src, n, codes, sink, stream);
         return run_tiled<BF16, F>(src, n, codes, sink, stream);

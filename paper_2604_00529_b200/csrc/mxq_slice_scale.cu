@@ -33,8 +33,8 @@ int run_single_tiled(const void* codes, const uint8_t* scales, size_t n, void* o
     if constexpr (ss_pair_ok(FH::id, FL::id) && FL::kind == KIND_FP) {
         auto kern = slice_scale_kernel<FH, FL, kU, kThreads, TiledScales>;
         const size_t nunits = n / 32;
-        const size_t ntiles = (nunits + 32 * kU - 1) / (32 * kU);
-        return launch_kernel(kern, grid_for_tiles(ntiles, kThreads), kThreads, stream, static_cast<const uint8_t*>(codes),
+        const size_t ctas = (nunits + kThreads * kU - 1) / (kThreads * kU) + tiled_pad_ctas(out_tiled, kThreads);
+        return launch_kernel(kern, grid_for_units(ctas, 1), kThreads, stream, static_cast<const uint8_t*>(codes),
                              scales, nunits, nunits, static_cast<uint8_t*>(out_codes), out_tiled);
     } else {
         return MXQ_ERR_PAIR;
@@ -87,6 +87,11 @@ int run_tiled_params(const SsTiledDeviceItem* items_host, int count, size_t tota
 
 }  // namespace
 
+size_t ss_tiled_batched_tiles(const SsTiledDeviceItem& item)
+{
+    return ss_batched_tiles(item.nunits) + tiled_pad_ctas(item.out_scales, kThreads);
+}
+
 size_t ss_batched_tiles(size_t nunits) { return (nunits + kThreads * kU - 1) / (kThreads * kU); }
 
 int launch_slice_scale(const void* codes, const uint8_t* scales, size_t n, int block, int src_fmt, int dst_fmt,
@@ -101,7 +106,7 @@ int launch_slice_scale(const void* codes, const uint8_t* scales, size_t n, int b
 int launch_slice_scale_tiled(const void* codes, const uint8_t* scales, size_t n, int src_fmt, int dst_fmt,
                              void* out_codes, uint8_t* out_tiled, uint32_t kblocks, cudaStream_t stream)
 {
-    const TiledScales sink = make_tiled_scales(out_tiled, kblocks);
+    const TiledScales sink = make_tiled_scales(out_tiled, kblocks, (uint32_t)(n / 32 / kblocks));
     MXQ_DISPATCH_FORMAT_AS(src_fmt, FH, {
         MXQ_DISPATCH_FORMAT_AS(dst_fmt, FL, { return run_single_tiled<FH, FL>(codes, scales, n, out_codes, sink, stream); });
     });

@@ -11,7 +11,7 @@ import torch
 
 import paper_2604_00529_b200 as mxq
 from oracle import mxq_oracle as orc
-from tests.gpu_util import FP_FORMATS, INT_FORMATS, Guarded, bits_equal, to_dev, to_host
+from gpu_util import FP_FORMATS, INT_FORMATS, Guarded, bits_equal, to_dev, to_host
 
 LOWER = {"int8": INT_FORMATS[1:], "e4m3": FP_FORMATS[1:]}
 
