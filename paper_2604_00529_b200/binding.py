@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Optional, Sequence, Tuple
 
 import torch
@@ -59,6 +60,11 @@ class _TiledItem(ctypes.Structure):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_host = None            # the native module _mxq_host (csrc/host_calls.cpp): the plain case of the per-tensor calls
+
+#: the entry points that _mxq_host calls
+_HOST_CALLS = ("mxq_quantize", "mxq_slice_scale", "mxq_slice_scale_multi", "mxq_dequantize", "mxq_tiled_scales_bytes",
+               "mxq_quantize_tiled", "mxq_slice_scale_tiled", "mxq_fake_quant", "mxq_fake_quant_bwd", "mxq_codes_bytes")
 
 
 def library_path() -> str:
@@ -67,12 +73,18 @@ def library_path() -> str:
 
 def load_library() -> ctypes.CDLL:
     """Load libmxq.so (built in-tree by ``python -m paper_2604_00529_b200.build``)."""
-    global _lib
+    global _lib, _host
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
         raise ImportError("libmxq.so is not built: run `python -m paper_2604_00529_b200.build` "
                           "(there is no fallback path)")
+    if _host is None:
+        try:
+            from . import _mxq_host
+        except ImportError as e:
+            raise ImportError("_mxq_host.so is not built for this torch: run `python -m paper_2604_00529_b200.build`") from e
+        _host = _mxq_host
     L = ctypes.CDLL(_LIB_PATH)
     vp, sz, i = ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int
     L.mxq_status_string.argtypes = [i]
@@ -116,6 +128,7 @@ def load_library() -> ctypes.CDLL:
     for name in ("mxq_quantize", "mxq_slice_scale", "mxq_dequantize", "mxq_fake_quant", "mxq_fake_quant_bwd",
                  "mxq_slice_scale_batched"):
         getattr(L, name).restype = i
+    _host.bind({name: ctypes.cast(getattr(L, name), vp).value for name in _HOST_CALLS}, FORMATS, torch.nn.Parameter)
     _lib = L
     return L
 
@@ -173,7 +186,10 @@ def _check(rc: int, what: str) -> None:
 def quantize(src: torch.Tensor, fmt: str, block: int = 32, codes: Optional[torch.Tensor] = None,
              scales: Optional[torch.Tensor] = None, stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """mxq_quantize: returns (packed codes uint8[n*bits/8], scales uint8[n/block])."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.quantize(src, fmt, block, codes, scales, stream)
+    if out is not None:
+        return out
     n = src.numel()
     if codes is None:
         codes = torch.empty(codes_bytes(n, fmt), dtype=torch.uint8, device=src.device)
@@ -188,7 +204,10 @@ def slice_scale(codes: torch.Tensor, scales: torch.Tensor, n: int, src_fmt: str,
                 out_codes: Optional[torch.Tensor] = None, out_scales: Optional[torch.Tensor] = None,
                 stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """mxq_slice_scale: anchor codes + scales -> lower-format codes + scales."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.slice_scale(codes, scales, n, src_fmt, dst_fmt, block, out_codes, out_scales, stream)
+    if out is not None:
+        return out
     if out_codes is None:
         out_codes = torch.empty(codes_bytes(n, dst_fmt), dtype=torch.uint8, device=codes.device)
     if out_scales is None:
@@ -202,7 +221,10 @@ def slice_scale(codes: torch.Tensor, scales: torch.Tensor, n: int, src_fmt: str,
 def slice_scale_multi(codes: torch.Tensor, scales: torch.Tensor, n: int, src_fmt: str, dst_fmts: Sequence[str],
                       block: int = 32, outs: Optional[Sequence[Tuple[torch.Tensor, torch.Tensor]]] = None, stream=None):
     """mxq_slice_scale_multi: one anchor -> several lower formats; returns [(codes, scales), ...]."""
-    L = load_library()
+    L = _lib or load_library()
+    made = _host.slice_scale_multi(codes, scales, n, src_fmt, dst_fmts, block, outs, stream)
+    if made is not None:
+        return made
     k = len(dst_fmts)
     if outs is None:
         outs = [(torch.empty(codes_bytes(n, f), dtype=torch.uint8, device=codes.device),
@@ -218,7 +240,10 @@ def slice_scale_multi(codes: torch.Tensor, scales: torch.Tensor, n: int, src_fmt
 def dequantize(codes: torch.Tensor, scales: torch.Tensor, n: int, fmt: str, block: int = 32,
                dtype: torch.dtype = torch.float32, dst: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """mxq_dequantize: V^ = X P as float32 or bfloat16."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.dequantize(codes, scales, n, fmt, block, dtype, dst, stream)
+    if out is not None:
+        return out
     if dst is None:
         dst = torch.empty(n, dtype=dtype, device=codes.device)
     _check(L.mxq_dequantize(_dev(codes, "codes"), _dev(scales, "scales"), n, FORMATS[fmt], block, _dev(dst, "dst"),
@@ -245,7 +270,10 @@ def tile_scales(scales: torch.Tensor, rows: int, kblocks: int, tiled: Optional[t
 def quantize_tiled(src: torch.Tensor, fmt: str, block: int = 32, codes: Optional[torch.Tensor] = None,
                    tiled_scales: Optional[torch.Tensor] = None, stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """mxq_quantize_tiled: a 2-D [rows, cols] tensor -> (packed codes, scale bytes in the 128 x 4 tiled order)."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.quantize_tiled(src, fmt, block, codes, tiled_scales, stream)
+    if out is not None:
+        return out
     if src.dim() != 2:
         raise ValueError("quantize_tiled takes a [rows, cols] matrix")
     rows, cols = src.shape
@@ -263,7 +291,10 @@ def slice_scale_tiled(codes: torch.Tensor, scales: torch.Tensor, rows: int, cols
                       out_tiled_scales: Optional[torch.Tensor] = None, stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """mxq_slice_scale_tiled: anchor codes + plain scales of a [rows, cols] matrix -> lower-format codes and
     scale bytes in the 128 x 4 tiled order."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.slice_scale_tiled(codes, scales, rows, cols, src_fmt, dst_fmt, block, out_codes, out_tiled_scales, stream)
+    if out is not None:
+        return out
     if out_codes is None:
         out_codes = torch.empty(codes_bytes(rows * cols, dst_fmt), dtype=torch.uint8, device=codes.device)
     if out_tiled_scales is None:
@@ -277,7 +308,10 @@ def slice_scale_tiled(codes: torch.Tensor, scales: torch.Tensor, rows: int, cols
 def fake_quant(src: torch.Tensor, fmt: str, block: int = 32, mode: int = FQ_DIRECT,
                dst: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """mxq_fake_quant: quantize-dequantize in one pass (dst may be src)."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.fake_quant(src, fmt, block, mode, dst, stream)
+    if out is not None:
+        return out
     if dst is None:
         dst = torch.empty_like(src)
     _check(L.mxq_fake_quant(_dev(src, "src"), _dtype_id(src), src.numel(), FORMATS[fmt], block, mode,
@@ -381,7 +415,10 @@ def dequantize_batched(items, fmt: str, block: int = 32, stream=None) -> None:
 
 def fake_quant_bwd(grad_out: torch.Tensor, grad_in: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """mxq_fake_quant_bwd: straight-through gradient (identity)."""
-    L = load_library()
+    L = _lib or load_library()
+    out = _host.fake_quant_bwd(grad_out, grad_in, stream)
+    if out is not None:
+        return out
     if grad_in is None:
         grad_in = torch.empty_like(grad_out)
     _check(L.mxq_fake_quant_bwd(_dev(grad_out, "grad_out"), _dtype_id(grad_out), grad_out.numel(),
@@ -389,19 +426,27 @@ def fake_quant_bwd(grad_out: torch.Tensor, grad_in: Optional[torch.Tensor] = Non
     return grad_in
 
 
+#: the calls that can be prepared, in the order of _mxq_host.run_prepared's kinds
+_PREPARED = ("mxq_quantize", "mxq_slice_scale", "mxq_dequantize", "mxq_fake_quant", "mxq_fake_quant_bwd")
+
+
 class PreparedCall:
     """One C-ABI call with its arguments already marshalled, for buffers that persist (a model's
     weights and their code buffers): ``prepare_*`` checks and converts the arguments once, calling the
     object enqueues the operation on the current stream (or on ``stream``).  It keeps the tensors alive.
-    Per call this leaves the stream lookup and the foreign call itself (about 2 us instead of 5)."""
+    Per call this leaves the stream lookup and the launch."""
 
-    __slots__ = ("fn", "args", "what", "keep")
+    __slots__ = ("fn", "args", "what", "keep", "kind", "packed")
 
     def __init__(self, fn, args, what, keep):
         self.fn, self.args, self.what, self.keep = fn, args, what, keep
+        self.kind, self.packed = _PREPARED.index(what), struct.pack("9q", *args, *(0,) * (9 - len(args)))
 
     def __call__(self, stream=None) -> None:
-        rc = self.fn(*self.args, _stream(stream))
+        if stream is None:
+            rc = _host.run_prepared(self.kind, self.packed)
+        else:
+            rc = self.fn(*self.args, _stream(stream))
         if rc != 0:
             raise MxqError(rc, self.what)
 
@@ -466,7 +511,10 @@ def fake_quant_ste(x: torch.Tensor, fmt: str, block: int = 32, mode: int = FQ_VI
     """W_t of Eq. 6 as a differentiable function of W: the value is ``fake_quant(x, fmt, block, mode)``,
     the gradient passes straight through (``copy_grad`` hands autograd a fresh copy instead of the
     incoming tensor)."""
-    return _FakeQuantSTE.apply(x, fmt, block, mode, copy_grad)
+    if _lib is None:
+        load_library()
+    y = _host.fake_quant_ste(x, fmt, block, mode, copy_grad)
+    return y if y is not None else _FakeQuantSTE.apply(x, fmt, block, mode, copy_grad)
 
 
 class ItemTable:

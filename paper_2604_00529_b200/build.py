@@ -3,7 +3,8 @@
     python -m paper_2604_00529_b200.build [--force] [--debug]
 
 One object per translation unit under ``_build/`` (compiled in parallel), linked into
-``paper_2604_00529_b200/libmxq.so``; then ``mxq_abi_timing``, a small C-level caller of the ABI.  A unit is rebuilt when it or any header is newer than
+``paper_2604_00529_b200/libmxq.so``; then ``mxq_abi_timing``, a small C-level caller of the ABI, and ``_mxq_host.so``,
+the native part of the Python binding.  A unit is rebuilt when it or any header is newer than
 its object.
 """
 from __future__ import annotations
@@ -18,6 +19,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libmxq.so")
+HOST_MODULE = os.path.join(HERE, "_mxq_host.so")       # the binding's native calls (csrc/host_calls.cpp)
 TIMING_EXE = os.path.join(HERE, "mxq_abi_timing")      # C-level caller of the ABI (csrc/abi_timing.cu)
 UNITS = ["mxq_api", "mxq_quantize", "mxq_slice_scale", "mxq_dequantize", "mxq_fake_quant", "mxq_static_batch", "mxq_slice_scale_multi", "mxq_slice_scale_multi_fp", "mxq_layout", "mxq_fake_quant_batched"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-std=c++20", "-O3", "-lineinfo",
@@ -51,7 +53,33 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     """Builds libmxq.so (and mxq_abi_timing); with debug=True builds libmxq_debug.so instead."""
     if debug:
         return _build_library(os.path.join(ROOT, "_build_debug"), DEBUG_LIB, ["-DMXQ_DEBUG"], force, verbose, timing=False)
-    return _build_library(OBJ_DIR, LIB, [], force, verbose, timing=True)
+    lib = _build_library(OBJ_DIR, LIB, [], force, verbose, timing=True)
+    build_host_module(force)
+    return lib
+
+
+def build_host_module(force: bool = False) -> str:
+    """Builds _mxq_host.so, the CPython module that binding.py imports, against the installed torch."""
+    src = os.path.join(CSRC, "host_calls.cpp")
+    if not (force or _stale(HOST_MODULE, [src, os.path.join(ROOT, "include", "mxq.h")])):
+        return HOST_MODULE
+    import sysconfig
+
+    import torch
+    top = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    tmp = HOST_MODULE + ".tmp.%d" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
+    for d in (os.path.join(top, "include"), os.path.join(top, "include", "torch", "csrc", "api", "include"),
+              os.path.join(cuda, "include"), sysconfig.get_paths()["include"]):
+        cmd += ["-isystem", d]
+    cmd += [src, "-o", tmp, "-L" + os.path.join(top, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed: %s\n%s" % (" ".join(cmd), r.stderr))
+    os.replace(tmp, HOST_MODULE)
+    return HOST_MODULE
 
 
 def _build_library(obj_dir: str, lib: str, extra, force: bool, verbose: bool, timing: bool) -> str:

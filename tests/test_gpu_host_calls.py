@@ -1,0 +1,138 @@
+"""The native part of the binding takes the plain case of a call and leaves every other one to the general
+path: the same results with and without given outputs, on given streams, for subclasses and wrapped tensors,
+the same errors as ever, and the straight-through estimator inside autograd."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2604_00529_b200 as mxq
+from paper_2604_00529_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def general(monkeypatch):
+    """Runs a call through the general path alone."""
+    class Off:
+        def __getattr__(self, name):
+            return (lambda *a: 1) if name == "run_prepared" else (lambda *a: None)
+
+    def run(fn):
+        host = binding._host
+        binding._host = Off()
+        try:
+            return fn()
+        finally:
+            binding._host = host
+    mxq.load_library()
+    return run
+
+
+def same(a, b):
+    if isinstance(a, torch.Tensor):
+        return a.dtype == b.dtype and a.shape == b.shape and a.device == b.device and torch.equal(
+            a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+    return type(a) is type(b) and len(a) == len(b) and all(same(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("shape", [(1, 32), (7, 96), (130, 256)])
+def test_native_calls_equal_the_general_path(general, dtype, shape):
+    x = torch.randn(*shape, device="cuda").to(dtype)
+    n = x.numel()
+    codes, scales = mxq.quantize(x, "e4m3")
+    dst = torch.empty(n, dtype=dtype, device="cuda")
+    calls = [
+        lambda: mxq.quantize(x, "int6"),
+        lambda: mxq.quantize(torch.nn.Parameter(x), "e2m1", 32),
+        lambda: mxq.quantize(x, "e4m3", codes=torch.empty_like(codes), scales=torch.empty_like(scales)),
+        lambda: mxq.slice_scale(codes, scales, n, "e4m3", "e2m3"),
+        lambda: mxq.slice_scale_multi(codes, scales, n, "e4m3", ["e2m3", "e2m1", "e3m3"]),
+        lambda: mxq.slice_scale_multi(codes, scales, n, "e4m3", []),
+        lambda: mxq.dequantize(codes, scales, n, "e4m3", dtype=dtype),
+        lambda: mxq.dequantize(codes, scales, n, "e4m3"),
+        lambda: mxq.dequantize(codes, scales, n, "e4m3", dst=dst),
+        lambda: mxq.quantize_tiled(x, "e3m2"),
+        lambda: mxq.slice_scale_tiled(codes, scales, *shape, "e4m3", "e2m1"),
+        lambda: mxq.fake_quant(x, "int4", 16, mxq.FQ_VIA_ANCHOR),
+        lambda: mxq.fake_quant_bwd(x),
+        lambda: mxq.fake_quant(x, "int4", stream=torch.cuda.Stream()) if torch.cuda.synchronize() is None else None,
+    ]
+    for call in calls:
+        got = call()
+        torch.cuda.synchronize()
+        want = general(call)
+        torch.cuda.synchronize()
+        assert same(got, want)
+    low, low_scales = torch.empty(n // 2, dtype=torch.uint8, device="cuda"), torch.empty_like(scales)
+    p = mxq.prepare_slice_scale(codes, scales, n, "e4m3", "e2m1", 32, low, low_scales)
+    p()
+    assert same((low, low_scales), general(lambda: mxq.slice_scale(codes, scales, n, "e4m3", "e2m1")))
+
+
+def test_refused_calls_stay_refused():
+    x = torch.randn(64, 64, device="cuda")
+    codes, scales = mxq.quantize(x, "int8")
+    n = x.numel()
+    for error, call in [
+        (ValueError, lambda: mxq.quantize(x.t(), "int8")),
+        (ValueError, lambda: mxq.quantize(x.cpu(), "int8")),
+        (TypeError, lambda: mxq.quantize(x.half(), "int8")),
+        (KeyError, lambda: mxq.quantize(x, "int9")),
+        (mxq.MxqError, lambda: mxq.quantize(x.view(-1)[:40], "int8")),
+        (mxq.MxqError, lambda: mxq.quantize(x.view(-1)[1:33], "int8")),
+        (mxq.MxqError, lambda: mxq.quantize(x, "int8", 48)),
+        (mxq.MxqError, lambda: mxq.quantize(x, "int8", 0)),
+        (mxq.MxqError, lambda: mxq.slice_scale(codes, scales, n, "int8", "e2m1")),
+        (mxq.MxqError, lambda: mxq.slice_scale_multi(codes, scales, n, "int8", ["int4", "e2m1"])),
+        (ValueError, lambda: mxq.dequantize(codes, scales.cpu(), n, "int8")),
+        (TypeError, lambda: mxq.dequantize(codes, scales, n, "int8", dtype=torch.float16)),
+        (ValueError, lambda: mxq.quantize_tiled(x.view(-1), "e4m3")),
+        (mxq.MxqError, lambda: mxq.quantize_tiled(x, "int8")),
+        (mxq.MxqError, lambda: mxq.fake_quant(x, "int4", 32, 7)),
+        (ValueError, lambda: mxq.fake_quant_ste(x.t().requires_grad_(), "int4")),
+        (RuntimeError, lambda: torch.func.vmap(lambda t: mxq.fake_quant(t, "int4"))(x)),
+        (RuntimeError, lambda: torch.func.vmap(lambda t: t * mxq.fake_quant_ste(x, "int4").sum())(x)),
+        (RuntimeError, lambda: torch.func.grad(lambda t: mxq.fake_quant_ste(t, "int4").sum())(x)),
+    ]:
+        with pytest.raises(error):
+            call()
+
+
+@pytest.mark.parametrize("copy_grad", [False, True])
+def test_straight_through_gradient(general, copy_grad):
+    x = torch.randn(8, 64, device="cuda").requires_grad_()
+    g = torch.randn(8, 64, device="cuda")
+
+    def step():
+        y = mxq.fake_quant_ste(x * 2, "e2m1", 32, mxq.FQ_VIA_ANCHOR, copy_grad)
+        return (y.detach(), *torch.autograd.grad(y * 3, x, g, retain_graph=True))
+
+    assert same(step(), general(step))
+    with torch.no_grad():
+        assert not mxq.fake_quant_ste(x, "e2m1").requires_grad
+    assert not mxq.fake_quant_ste(x.detach(), "e2m1").requires_grad
+    (first,) = torch.autograd.grad(mxq.fake_quant_ste(x, "e2m1", copy_grad=copy_grad).pow(3).sum(), x, create_graph=True)
+    assert first.requires_grad != copy_grad                     # the copied gradient is a constant, as through the general path
+
+
+def test_graph_capture_and_side_stream():
+    x = torch.randn(64, 128, device="cuda")
+    want = [t.clone() for t in mxq.quantize(x, "e4m3")]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        mxq.quantize(x, "e4m3")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        codes, scales = mxq.quantize(x, "e4m3")
+        low = mxq.slice_scale(codes, scales, x.numel(), "e4m3", "e2m1")
+    codes.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert same((codes, scales), tuple(want))
+    assert np.array_equal(low[0].cpu().numpy(), mxq.slice_scale(*want, x.numel(), "e4m3", "e2m1")[0].cpu().numpy())
