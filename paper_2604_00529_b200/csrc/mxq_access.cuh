@@ -88,6 +88,18 @@ __device__ __forceinline__ void st_u8(uint8_t* p, uint32_t v)
     *p = (uint8_t)v;
 }
 
+__device__ __forceinline__ uint32_t ld_u16(const uint8_t* p)              // p 2-byte aligned
+{
+    MXQ_CHECKED(p, 2, return 0)
+    return *reinterpret_cast<const uint16_t*>(p);
+}
+
+__device__ __forceinline__ void st_u16(uint8_t* p, uint32_t v)
+{
+    MXQ_CHECKED(p, 2, return)
+    *reinterpret_cast<uint16_t*>(p) = (uint16_t)v;
+}
+
 __device__ __forceinline__ void st_u32(uint8_t* p, uint32_t v)          // p 4-byte aligned
 {
     MXQ_CHECKED(p, 4, return)

@@ -20,13 +20,19 @@ int run(const void* codes, const uint8_t* scales, size_t n, int block, void* dst
         return launch_kernel(kern, grid_for_tiles((nunits + 32 * kU - 1) / (32 * kU), kThreads), kThreads, stream,
                              static_cast<const uint8_t*>(codes), scales, nunits, shift, static_cast<uint8_t*>(dst));
     } else {
-        // 16-bit output: lane units of 32 codes
-        auto kern = dequantize_kernel<F, T, kU, kThreads>;
-        const size_t nunits = n / 32;
+        // 16-bit output: lane units of 32 codes, two per thread, but one where two leave the chip idle (see
+        // grid_is_small): 2^22.1 codes from L2 to BF16, MXINT4 5.8 -> 3.2 us, E2M3 6.5 -> 3.2, and behind the conversion that wrote
+        // them (both launches) MXINT4 unchanged, E2M3 7.7 ... 13 -> 6.0; 2^23 codes E2M3 5.8 -> 4.2 and 11.6 -> 8.6, but MXINT4
+        // 7.2 -> 8.1: 4-bit codes and narrower keep two from half that size on.  2^24 codes: 2 - 5 % slower.
+        const size_t ctas = (n / 32 + kThreads * kU - 1) / (kThreads * kU);
+        const bool one = grid_is_small(F::bits > 4 ? ctas : 2 * ctas);
+        auto kern = one ? dequantize_kernel<F, T, 1, kThreads> : dequantize_kernel<F, T, kU, kThreads>;
+        const size_t nunits = n / 32, per_tile = one ? 32 : 32 * kU;
+        const size_t ntiles = (nunits + per_tile - 1) / per_tile;
         int shift = 0, per_unit = 1;
         if (block == 16) per_unit = 2;
         else while ((32 << shift) < block) ++shift;
-        return launch_kernel(kern, grid_for_tiles((nunits + 32 * kU - 1) / (32 * kU), kThreads), kThreads, stream,
+        return launch_kernel(kern, grid_for_tiles(ntiles, kThreads), kThreads, stream,
                              static_cast<const uint8_t*>(codes), scales, nunits, shift, per_unit,
                              static_cast<uint8_t*>(dst));
     }

@@ -988,8 +988,10 @@ __device__ __forceinline__ uint8_t ss_scale_byte(uint32_t b, int de)
 
 // One warp tile (32 U lane units) of one tensor; shared by the single-tensor and the batched
 // kernels.  The scale bytes are an element-wise stream of their own: lane unit i also converts
-// scale i, and scale nunits + i when the block is smaller than a lane unit (block 16).
-template <class FH, class FL, int U, class SCALES>
+// scale i, or, with HALVES (block 16, two scales per lane unit), its own two as one 16-bit access: MXINT8 -> MXINT4 of
+// 2^25 codes 9.7 us, E4M3 -> E2M3 10.9, where a second pass over the upper half of the scales took 10.7 and 12.7.  (A
+// run-time choice between the two forms cost the larger blocks 2 - 9 %.)
+template <class FH, class FL, int U, bool HALVES, class SCALES>
 __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
                                                  size_t nunits, size_t nscales, uint8_t* __restrict__ out_codes,
                                                  const SCALES& out_scales, size_t tile, uint8_t* stage)
@@ -1008,12 +1010,17 @@ __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ cod
 #pragma unroll
             for (int j = 0; j < NWI; ++j) w[u][j] = 0;
         }
-        sb[u] = unit < nscales ? ld_u8(scales + unit) : 0;
+        if constexpr (HALVES) sb[u] = unit < nunits ? ld_u16(scales + unit * 2) : 0;
+        else sb[u] = unit < nscales ? ld_u8(scales + unit) : 0;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const size_t unit = u0 + u * 32;
-        if (unit < nscales) put_scale(out_scales, unit, ss_scale_byte(sb[u], de));
+        if constexpr (HALVES) {
+            if (unit < nunits) st_u16(out_scales + unit * 2, ss_scale_byte(sb[u] & 0xFFu, de) | ss_scale_byte(sb[u] >> 8, de) << 8);
+        } else {
+            if (unit < nscales) put_scale(out_scales, unit, ss_scale_byte(sb[u], de));
+        }
         uint32_t out[NWO];
         slice_scale_unit<FH, FL>(w[u], out);
         if constexpr (StagedTile<OB>::use) store_bytes<OB>(stage + (u * 32 + (threadIdx.x & 31)) * OB, out);
@@ -1022,12 +1029,15 @@ __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ cod
     if constexpr (StagedTile<OB>::use) {
         const size_t first = tile * (32 * U), left = nunits - first;
         flush_stage<32 * U * OB>(stage, out_codes + first * OB, (uint32_t)(left < 32 * U ? left : 32 * U) * OB);
-    }
-    if (nscales > nunits) {
+    }    if constexpr (!HALVES) {
+        // (Not reached by the entry points, whose block 16 takes HALVES; without it the compiler's schedule for the larger
+        // blocks is slower: MXINT8 -> MXINT4 of 2^24 codes and back to FP32 17.5 us against 17.2.)
+        if (nscales > nunits) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const size_t i = nunits + u0 + u * 32;
-            if (i < nscales) put_scale(out_scales, i, ss_scale_byte(ld_u8(scales + i), de));
+            for (int u = 0; u < U; ++u) {
+                const size_t i = nunits + u0 + u * 32;
+                if (i < nscales) put_scale(out_scales, i, ss_scale_byte(ld_u8(scales + i), de));
+            }
         }
     }
 }
@@ -1058,7 +1068,7 @@ __host__ __device__ constexpr int slice_scale_min_ctas()
     else return FH::kind == KIND_INT ? 10 : 14;
 }
 
-template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*>
+template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*, bool HALVES = false>
 __global__ void __launch_bounds__(THREADS, slice_scale_min_ctas<FH, SCALES>())
 slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits,
                    size_t nscales, uint8_t* __restrict__ out_codes, SCALES out_scales)
@@ -1070,7 +1080,7 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
     prefetch_tile<U, 4 * FH::bits>(codes, tile, nunits);
     pdl_acquire();
     if (tile * (32 * U) < nunits)
-        slice_scale_tile<FH, FL, U>(codes, scales, nunits, nscales, out_codes, out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, HALVES>(codes, scales, nunits, nscales, out_codes, out_scales, tile, stage);
 }
 
 // Several targets from one read of the anchor (the elastic-serving case: one stored checkpoint, several lower
@@ -1079,7 +1089,8 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
 // computed once.  The set of targets is a compile-time list: a kernel that walks a run-time list of formats
 // keeps the shared words in registers across a switch and took 38 - 46 us for MXINT8 -> {7, 5, 3} bits of 2^25.8
 // codes (block 64) where these take 31 (a pass per target: 53; the bytes alone: 26).  Compiled for 12 resident
-// CTAs (40 registers): 10 take 32 us, 14 spill and take 33, one unit per lane at 16 CTAs takes 35.
+// CTAs (40 registers): 10 take 32 us, 14 spill and take 33, one unit per lane at 16 CTAs takes 35.  Sets of four spill at 12
+// (MXINT8 -> {7, 6, 4, 2} of 2^24 codes 12.9 us) and get 10 (12.0).
 struct SsOut {
     uint8_t* codes;
     uint8_t* scales;
@@ -1206,7 +1217,7 @@ __device__ __forceinline__ uint8_t* slice_scale_set_stage()
 }
 
 template <class FH, int U, int THREADS, class... FL>
-__global__ void __launch_bounds__(THREADS, 12)
+__global__ void __launch_bounds__(THREADS, sizeof...(FL) >= 4 ? 10 : 12)
 slice_scale_set_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits, size_t nscales,
                        const __grid_constant__ SsOuts<(int)sizeof...(FL)> outs)
 {
@@ -1244,7 +1255,7 @@ slice_scale_batched_kernel(const SsDeviceItem* __restrict__ items, const TileInd
     const SsDeviceItem& t = items[find_item(items, *index, blockIdx.x)];
     const size_t tile = item_warp_tile<THREADS>(t.tile_begin);
     if (tile * (32 * U) < t.nunits)                       // whole warps
-        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, false>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
 }
 
 // The same launch with the item table carried in the kernel's parameter space (K items, 56 bytes
@@ -1268,7 +1279,7 @@ slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
     prefetch_tile<U, 4 * FH::bits>(t.codes, tile, t.nunits);
     pdl_acquire();
     if (tile * (32 * U) < t.nunits)                       // whole warps
-        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, false>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
 }
 
 // Two targets from one read of every anchor of a set of tensors (the whole-model conversion of Sec. 3.5
@@ -1332,7 +1343,7 @@ slice_scale_tiled_batched_kernel(const __grid_constant__ SsTiledItemBlock<K> blk
     prefetch_tile<U, 4 * FH::bits>(t.codes, tile, t.nunits);
     pdl_acquire();
     if (tile * (32 * U) < t.nunits)                       // whole warps
-        slice_scale_tile<FH, FL, U>(t.codes, t.scales, t.nunits, t.nunits, t.out_codes, t.out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, false>(t.codes, t.scales, t.nunits, t.nunits, t.out_codes, t.out_scales, tile, stage);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -28,6 +28,10 @@ inline int grid_for_units(size_t nunits, size_t per_cta)
     return need > (size_t)0x7FFFFFFF ? 0 : (int)need;
 }
 
+// Are `ctas` CTAs of 128 threads too few to keep the chip busy (under eight per SM of its 148)?  A launch is then
+// bound by how long one thread takes, and the shape with half the work per thread is faster.
+inline bool grid_is_small(size_t ctas) { return ctas < (size_t)148 * 8; }
+
 int launch_quantize(const void* src, int dtype, size_t n, int fmt, int block, void* codes, uint8_t* scales,
                     cudaStream_t stream);
 int launch_fake_quant(const void* src, int dtype, size_t n, int fmt, int block, int mode, void* dst,
