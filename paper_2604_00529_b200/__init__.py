@@ -1,8 +1,8 @@
 """B200-native block-wise microscaling (MX) quantization for MF-QAT.
 
 The compute lives in ``libmxq.so`` (hand-written CUDA for sm_100a behind the C ABI declared in
-``include/mxq.h``).  This package is a thin ctypes binding with the same entry-point names; it
-marshals arguments and nothing else.  There is no CPU fallback: every call fails loudly when
+``include/mxq.h``).  This package is a thin binding with the same entry-point names (ctypes, and native code for the
+plain case of the per-tensor calls); it marshals arguments and nothing else.  There is no CPU fallback: every call fails loudly when
 the library is missing or the tensors are not CUDA tensors.
 """
 from .binding import (  # noqa: F401

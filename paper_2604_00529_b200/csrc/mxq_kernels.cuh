@@ -989,7 +989,7 @@ __device__ __forceinline__ uint8_t ss_scale_byte(uint32_t b, int de)
 // One warp tile (32 U lane units) of one tensor; shared by the single-tensor and the batched
 // kernels.  The scale bytes are an element-wise stream of their own: lane unit i also converts
 // scale i, or, with HALVES (block 16, two scales per lane unit), its own two as one 16-bit access: MXINT8 -> MXINT4 of
-// 2^25 codes 9.7 us, E4M3 -> E2M3 10.9, where a second pass over the upper half of the scales took 10.7 and 12.7.  (A
+// 2^25 codes 9.1 us, E4M3 -> E2M3 11.3, where a second pass over the upper half of the scales took 10.8 and 12.7.  (A
 // run-time choice between the two forms cost the larger blocks 2 - 9 %.)
 template <class FH, class FL, int U, bool HALVES, class SCALES>
 __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
