@@ -106,8 +106,8 @@ int launch_slice_scale_tiled_batched(const SsTiledDeviceItem* items_host, int co
 size_t ss_batched_tiles(size_t nunits);
 size_t ss_tiled_batched_tiles(const SsTiledDeviceItem& item);      // the same with the padding of its scale tiles
 
-// Item tables ride in the kernel parameters, and a launch pays for their size (host time per launch on the B200
-// box: 2.3 us with 64 bytes of parameters, 2.4 with 4 KB, 3.6 with 16 KB, 5.0 - 5.5 with 32 KB).  So every batched
+// Item tables ride in the kernel parameters, and a launch pays for their size (host time per launch next to a
+// B200: 2.3 us with 64 bytes of parameters, 2.4 with 4 KB, 3.6 with 16 KB, 5.0 - 5.5 with 32 KB).  So every batched
 // kernel exists with a small table, for the sets of a few layers, and with the largest one.
 constexpr int kSmallBatchItems = 64;
 template <int KMAX, class FN>
