@@ -61,7 +61,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
 def build_host_module(force: bool = False) -> str:
     """Builds _mxq_host.so, the CPython module that binding.py imports, against the installed torch."""
     src = os.path.join(CSRC, "host_calls.cpp")
-    if not (force or _stale(HOST_MODULE, [src, os.path.join(ROOT, "include", "mxq.h")])):
+    if not (force or _stale(HOST_MODULE, [src, os.path.join(ROOT, "include", "mxq.h"), os.path.abspath(__file__)])):
         return HOST_MODULE
     import sysconfig
 
@@ -74,7 +74,10 @@ def build_host_module(force: bool = False) -> str:
     for d in (os.path.join(top, "include"), os.path.join(top, "include", "torch", "csrc", "api", "include"),
               os.path.join(cuda, "include"), sysconfig.get_paths()["include"]):
         cmd += ["-isystem", d]
-    cmd += [src, "-o", tmp, "-L" + os.path.join(top, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    # The C++ runtime is named by its shared object: a compiler whose own folder has only libstdc++.a would link a second
+    # copy of the runtime into the module, and a stream or an error message made there then crashes the process.
+    cmd += [src, "-o", tmp, "-L" + os.path.join(top, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+            "-nostdlib++", "-l:libstdc++.so.6"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("g++ failed: %s\n%s" % (" ".join(cmd), r.stderr))
