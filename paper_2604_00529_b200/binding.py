@@ -128,7 +128,8 @@ def load_library() -> ctypes.CDLL:
     for name in ("mxq_quantize", "mxq_slice_scale", "mxq_dequantize", "mxq_fake_quant", "mxq_fake_quant_bwd",
                  "mxq_slice_scale_batched"):
         getattr(L, name).restype = i
-    _host.bind({name: ctypes.cast(getattr(L, name), vp).value for name in _HOST_CALLS}, FORMATS, torch.nn.Parameter)
+    _host.bind({name: ctypes.cast(getattr(L, name), vp).value for name in _HOST_CALLS}, FORMATS, torch.nn.Parameter,
+               MxqError)
     _lib = L
     return L
 

@@ -39,6 +39,7 @@ struct Api {
 
 PyObject* formats = nullptr;          // the binding's name -> id dict
 PyTypeObject* parameter = nullptr;    // torch.nn.Parameter
+PyObject* mxq_error = nullptr;        // the binding's MxqError(status, what)
 
 // ---- arguments ------------------------------------------------------------------------------------------
 
@@ -364,6 +365,19 @@ PyObject* run_prepared(PyObject*, PyObject* const* a, Py_ssize_t nargs)
 
 struct NotPlain {};                    // the launch was refused: the general path raises the error
 
+// MxqError(rc, what) out of a backward pass, which runs without the interpreter's lock and on a thread of its own.
+[[noreturn]] void throw_mxq_error(int rc, const char* what)
+{
+    pybind11::gil_scoped_acquire lock;
+    if (PyObject* e = PyObject_CallFunction(mxq_error, "is", rc, what)) {
+        PyErr_SetObject(mxq_error, e);
+        Py_DECREF(e);
+    }
+    python_error raised;
+    raised.persist();
+    throw python_error(std::move(raised));
+}
+
 struct FakeQuantSTE : torch::autograd::Function<FakeQuantSTE> {
     static at::Tensor forward(torch::autograd::AutogradContext* ctx, const at::Tensor& x, int64_t fmt, int64_t block, int64_t mode,
                               bool copy_grad)
@@ -388,7 +402,7 @@ struct FakeQuantSTE : torch::autograd::Function<FakeQuantSTE> {
             at::NoGradGuard no_grad;
             at::Tensor copy = at::empty_like(src);
             const int rc = api.fake_quant_bwd(src.data_ptr(), dt, (size_t)src.numel(), copy.data_ptr(), current_stream());
-            TORCH_CHECK(rc == MXQ_OK, "mxq_fake_quant_bwd failed with status ", rc);
+            if (rc != MXQ_OK) throw_mxq_error(rc, "mxq_fake_quant_bwd");
             g = copy;
         }
         return {g, at::Tensor(), at::Tensor(), at::Tensor(), at::Tensor()};
@@ -416,11 +430,11 @@ PyObject* fake_quant_ste(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     END_HANDLE_TH_ERRORS
 }
 
-// bind(addresses by name, formats, torch.nn.Parameter)
+// bind(addresses by name, formats, torch.nn.Parameter, MxqError)
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t nargs)
 {
-    if (nargs != 3 || !PyDict_Check(a[0]) || !PyDict_Check(a[1]) || !PyType_Check(a[2])) {
-        PyErr_SetString(PyExc_TypeError, "bind(addresses, formats, parameter type)");
+    if (nargs != 4 || !PyDict_Check(a[0]) || !PyDict_Check(a[1]) || !PyType_Check(a[2]) || !PyType_Check(a[3])) {
+        PyErr_SetString(PyExc_TypeError, "bind(addresses, formats, parameter type, error type)");
         return nullptr;
     }
     bool ok = true;
@@ -448,6 +462,8 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     api = n;
     Py_INCREF(a[1]);
     Py_INCREF(a[2]);
+    Py_INCREF(a[3]);
+    Py_XSETREF(mxq_error, a[3]);
     Py_XSETREF(formats, a[1]);
     Py_XSETREF(parameter, reinterpret_cast<PyTypeObject*>(a[2]));
     Py_RETURN_NONE;

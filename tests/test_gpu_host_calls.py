@@ -119,6 +119,19 @@ def test_straight_through_gradient(general, copy_grad):
     assert first.requires_grad != copy_grad                     # the copied gradient is a constant, as through the general path
 
 
+def test_a_refused_backward_raises_the_library_s_error(general):
+    x = torch.randn(8, 64, device="cuda").requires_grad_()
+    g = torch.randn(513, device="cuda")[1:].view(8, 64)                # contiguous, not 32-byte aligned
+
+    def step():
+        with pytest.raises(mxq.MxqError) as e:
+            torch.autograd.grad(mxq.fake_quant_ste(x, "int4", copy_grad=True), x, g)
+        return (e.value.status, str(e.value))
+
+    status, text = step()
+    assert (status, text) == general(step) and "MXQ_ERR_ALIGN" in text
+
+
 def test_graph_capture_and_side_stream():
     x = torch.randn(64, 128, device="cuda")
     want = [t.clone() for t in mxq.quantize(x, "e4m3")]
