@@ -59,13 +59,15 @@ const at::Tensor* plain(PyObject* o)
     return &t;
 }
 
-bool dtype_id(const at::Tensor& t, int* id)
+bool dtype_id(at::ScalarType t, int* id)
 {
-    if (t.scalar_type() == at::kFloat) *id = MXQ_F32;
-    else if (t.scalar_type() == at::kBFloat16) *id = MXQ_BF16;
+    if (t == at::kFloat) *id = MXQ_F32;
+    else if (t == at::kBFloat16) *id = MXQ_BF16;
     else return false;
     return true;
 }
+
+bool dtype_id(const at::Tensor& t, int* id) { return dtype_id(t.scalar_type(), id); }
 
 bool as_int(PyObject* o, int* v)
 {
@@ -96,38 +98,49 @@ bool format_id(PyObject* o, int* v)
     return as_int(id, v);
 }
 
-// An output argument: the given tensor, or a new one of `nbytes` bytes (`made`) when it is None.
-bool output(PyObject* o, int64_t nbytes, const at::Tensor& like, at::Tensor* made, const at::Tensor** out)
-{
-    if (o == Py_None) {
-        *made = at::empty({nbytes}, at::TensorOptions().dtype(at::kByte).device(like.device()));
-        *out = made;
-        return true;
-    }
-    *out = plain(o);
-    return *out != nullptr;
-}
-
 mxq_stream current_stream() { return static_cast<mxq_stream>(c10::cuda::getCurrentCUDAStream().stream()); }
 
-// A call of the ABI with the interpreter's lock released (a launch waits when the queue is full).
-template <class FN, class... A>
-int enqueue(FN fn, A... a)
+// The interpreter's lock is released while a call allocates and enqueues: a launch waits when the queue is full, an
+// allocation may wait for the device, and other Python threads (or a host callback that the queue itself waits for)
+// have to run meanwhile.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked&) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+// What `fn` returns, run without the lock.
+template <class FN>
+int unlocked(FN&& fn)
 {
-    const mxq_stream s = current_stream();
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = fn(a..., s);
-    Py_END_ALLOW_THREADS
-    return rc;
+    Unlocked u;
+    return fn();
 }
 
-PyObject* result(PyObject* given, const at::Tensor& made)
-{
-    if (given == Py_None) return THPVariable_Wrap(made);
-    Py_INCREF(given);
-    return given;
-}
+// An output argument: the given tensor, or a new one when it is None.
+struct Output {
+    const at::Tensor* tensor = nullptr;
+    at::Tensor made;
+
+    bool take(PyObject* o) { return o == Py_None || (tensor = plain(o)); }
+    void make(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& like)
+    {
+        if (!tensor) tensor = &(made = at::empty(sizes, at::TensorOptions().dtype(type).device(like.device())));
+    }
+    void make_like(const at::Tensor& like)
+    {
+        if (!tensor) tensor = &(made = at::empty_like(like));
+    }
+    void* data() const { return tensor->data_ptr(); }
+    uint8_t* bytes() const { return static_cast<uint8_t*>(tensor->data_ptr()); }
+    PyObject* result(PyObject* given) const
+    {
+        if (given == Py_None) return THPVariable_Wrap(made);
+        Py_INCREF(given);
+        return given;
+    }
+};
 
 PyObject* pair(PyObject* a, PyObject* b)
 {
@@ -156,14 +169,16 @@ PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     int fmt, block, dt;
     GENERAL_UNLESS(nargs == 6 && a[5] == Py_None && format_id(a[1], &fmt) && as_int(a[2], &block) && block > 0 && !modes_active());
     const at::Tensor* src = plain(a[0]);
-    GENERAL_UNLESS(src && dtype_id(*src, &dt));
-    const int64_t n = src->numel();
-    at::Tensor made[2];
-    const at::Tensor *codes, *scales;
-    GENERAL_UNLESS(output(a[3], (int64_t)api.codes_bytes((size_t)n, fmt), *src, &made[0], &codes));
-    GENERAL_UNLESS(output(a[4], n / block, *src, &made[1], &scales));
-    GENERAL_UNLESS(enqueue(api.quantize, src->data_ptr(), dt, (size_t)n, fmt, block, codes->data_ptr(), bytes(*scales)) == MXQ_OK);
-    return pair(result(a[3], made[0]), result(a[4], made[1]));
+    Output codes, scales;
+    GENERAL_UNLESS(src && dtype_id(*src, &dt) && codes.take(a[3]) && scales.take(a[4]));
+    const int rc = unlocked([&] {
+        const int64_t n = src->numel();
+        codes.make({(int64_t)api.codes_bytes((size_t)n, fmt)}, at::kByte, *src);
+        scales.make({n / block}, at::kByte, *src);
+        return api.quantize(src->data_ptr(), dt, (size_t)n, fmt, block, codes.data(), scales.bytes(), current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return pair(codes.result(a[3]), scales.result(a[4]));
     END_HANDLE_TH_ERRORS
 }
 
@@ -176,14 +191,16 @@ PyObject* slice_scale(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     GENERAL_UNLESS(nargs == 9 && a[8] == Py_None && as_count(a[2], &n) && format_id(a[3], &src_fmt) && format_id(a[4], &dst_fmt) &&
                    as_int(a[5], &block) && block > 0 && !modes_active());
     const at::Tensor *codes = plain(a[0]), *scales = plain(a[1]);
-    GENERAL_UNLESS(codes && scales);
-    at::Tensor made[2];
-    const at::Tensor *oc, *os;
-    GENERAL_UNLESS(output(a[6], (int64_t)api.codes_bytes((size_t)n, dst_fmt), *codes, &made[0], &oc));
-    GENERAL_UNLESS(output(a[7], n / block, *codes, &made[1], &os));
-    GENERAL_UNLESS(enqueue(api.slice_scale, codes->data_ptr(), bytes(*scales), (size_t)n, block, src_fmt, dst_fmt, oc->data_ptr(),
-                           bytes(*os)) == MXQ_OK);
-    return pair(result(a[6], made[0]), result(a[7], made[1]));
+    Output oc, os;
+    GENERAL_UNLESS(codes && scales && oc.take(a[6]) && os.take(a[7]));
+    const int rc = unlocked([&] {
+        oc.make({(int64_t)api.codes_bytes((size_t)n, dst_fmt)}, at::kByte, *codes);
+        os.make({n / block}, at::kByte, *codes);
+        return api.slice_scale(codes->data_ptr(), bytes(*scales), (size_t)n, block, src_fmt, dst_fmt, oc.data(), os.bytes(),
+                               current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return pair(oc.result(a[6]), os.result(a[7]));
     END_HANDLE_TH_ERRORS
 }
 
@@ -202,22 +219,24 @@ PyObject* slice_scale_multi(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     GENERAL_UNLESS(codes && scales);
     int fmts[MXQ_MULTI_TARGETS_MAX];
     for (Py_ssize_t t = 0; t < k; ++t) GENERAL_UNLESS(format_id(PySequence_Fast_GET_ITEM(a[4], t), &fmts[t]));
-    at::Tensor oc[MXQ_MULTI_TARGETS_MAX], os[MXQ_MULTI_TARGETS_MAX];
-    void* pc[MXQ_MULTI_TARGETS_MAX];
-    uint8_t* ps[MXQ_MULTI_TARGETS_MAX];
-    const auto options = at::TensorOptions().dtype(at::kByte).device(codes->device());
-    for (Py_ssize_t t = 0; t < k; ++t) {
-        oc[t] = at::empty({(int64_t)api.codes_bytes((size_t)n, fmts[t])}, options);
-        os[t] = at::empty({n / block}, options);
-        pc[t] = oc[t].data_ptr();
-        ps[t] = bytes(os[t]);
-    }
-    GENERAL_UNLESS(enqueue(api.slice_scale_multi, codes->data_ptr(), bytes(*scales), (size_t)n, block, src_fmt, (int)k, fmts, pc,
-                           ps) == MXQ_OK);
+    Output oc[MXQ_MULTI_TARGETS_MAX], os[MXQ_MULTI_TARGETS_MAX];
+    const int rc = unlocked([&] {
+        void* pc[MXQ_MULTI_TARGETS_MAX];
+        uint8_t* ps[MXQ_MULTI_TARGETS_MAX];
+        for (Py_ssize_t t = 0; t < k; ++t) {
+            oc[t].make({(int64_t)api.codes_bytes((size_t)n, fmts[t])}, at::kByte, *codes);
+            os[t].make({n / block}, at::kByte, *codes);
+            pc[t] = oc[t].data();
+            ps[t] = os[t].bytes();
+        }
+        return api.slice_scale_multi(codes->data_ptr(), bytes(*scales), (size_t)n, block, src_fmt, (int)k, fmts, pc, ps,
+                                     current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
     PyObject* list = PyList_New(k);
     if (!list) return nullptr;
     for (Py_ssize_t t = 0; t < k; ++t) {
-        PyObject* p = pair(THPVariable_Wrap(oc[t]), THPVariable_Wrap(os[t]));
+        PyObject* p = pair(oc[t].result(Py_None), os[t].result(Py_None));
         if (!p) {
             Py_DECREF(list);
             return nullptr;
@@ -237,21 +256,22 @@ PyObject* dequantize(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     GENERAL_UNLESS(nargs == 8 && a[7] == Py_None && as_count(a[2], &n) && format_id(a[3], &fmt) && as_int(a[4], &block) &&
                    !modes_active());
     const at::Tensor *codes = plain(a[0]), *scales = plain(a[1]);
-    GENERAL_UNLESS(codes && scales);
-    at::Tensor made;
-    const at::Tensor* dst = &made;
-    if (a[6] != Py_None) {
-        dst = plain(a[6]);
-        GENERAL_UNLESS(dst);
+    Output dst;
+    GENERAL_UNLESS(codes && scales && dst.take(a[6]));
+    at::ScalarType type = at::kFloat;
+    if (dst.tensor) {
+        GENERAL_UNLESS(dtype_id(*dst.tensor, &dt));
     } else {
         GENERAL_UNLESS(THPDtype_Check(a[5]));
-        const at::ScalarType st = reinterpret_cast<THPDtype*>(a[5])->scalar_type;
-        GENERAL_UNLESS(st == at::kFloat || st == at::kBFloat16);
-        made = at::empty({n}, at::TensorOptions().dtype(st).device(codes->device()));
+        type = reinterpret_cast<THPDtype*>(a[5])->scalar_type;
+        GENERAL_UNLESS(dtype_id(type, &dt));
     }
-    GENERAL_UNLESS(dtype_id(*dst, &dt));
-    GENERAL_UNLESS(enqueue(api.dequantize, codes->data_ptr(), bytes(*scales), (size_t)n, fmt, block, dst->data_ptr(), dt) == MXQ_OK);
-    return result(a[6], made);
+    const int rc = unlocked([&] {
+        dst.make({n}, type, *codes);
+        return api.dequantize(codes->data_ptr(), bytes(*scales), (size_t)n, fmt, block, dst.data(), dt, current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return dst.result(a[6]);
     END_HANDLE_TH_ERRORS
 }
 
@@ -262,15 +282,17 @@ PyObject* quantize_tiled(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     int fmt, block, dt;
     GENERAL_UNLESS(nargs == 6 && a[5] == Py_None && format_id(a[1], &fmt) && as_int(a[2], &block) && !modes_active());
     const at::Tensor* src = plain(a[0]);
-    GENERAL_UNLESS(src && dtype_id(*src, &dt) && src->dim() == 2);
-    const int64_t rows = src->size(0), cols = src->size(1);
-    at::Tensor made[2];
-    const at::Tensor *codes, *scales;
-    GENERAL_UNLESS(output(a[3], (int64_t)api.codes_bytes((size_t)(rows * cols), fmt), *src, &made[0], &codes));
-    GENERAL_UNLESS(output(a[4], (int64_t)api.tiled_scales_bytes((size_t)rows, (size_t)(cols / 32)), *src, &made[1], &scales));
-    GENERAL_UNLESS(enqueue(api.quantize_tiled, src->data_ptr(), dt, (size_t)rows, (size_t)cols, fmt, block, codes->data_ptr(),
-                           bytes(*scales)) == MXQ_OK);
-    return pair(result(a[3], made[0]), result(a[4], made[1]));
+    Output codes, scales;
+    GENERAL_UNLESS(src && dtype_id(*src, &dt) && src->dim() == 2 && codes.take(a[3]) && scales.take(a[4]));
+    const int rc = unlocked([&] {
+        const int64_t rows = src->size(0), cols = src->size(1);
+        codes.make({(int64_t)api.codes_bytes((size_t)(rows * cols), fmt)}, at::kByte, *src);
+        scales.make({(int64_t)api.tiled_scales_bytes((size_t)rows, (size_t)(cols / 32))}, at::kByte, *src);
+        return api.quantize_tiled(src->data_ptr(), dt, (size_t)rows, (size_t)cols, fmt, block, codes.data(), scales.bytes(),
+                                  current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return pair(codes.result(a[3]), scales.result(a[4]));
     END_HANDLE_TH_ERRORS
 }
 
@@ -284,14 +306,16 @@ PyObject* slice_scale_tiled(PyObject*, PyObject* const* a, Py_ssize_t nargs)
                    cols < (1ll << 31) && format_id(a[4], &src_fmt) && format_id(a[5], &dst_fmt) && as_int(a[6], &block) &&
                    !modes_active());
     const at::Tensor *codes = plain(a[0]), *scales = plain(a[1]);
-    GENERAL_UNLESS(codes && scales);
-    at::Tensor made[2];
-    const at::Tensor *oc, *os;
-    GENERAL_UNLESS(output(a[7], (int64_t)api.codes_bytes((size_t)(rows * cols), dst_fmt), *codes, &made[0], &oc));
-    GENERAL_UNLESS(output(a[8], (int64_t)api.tiled_scales_bytes((size_t)rows, (size_t)(cols / 32)), *codes, &made[1], &os));
-    GENERAL_UNLESS(enqueue(api.slice_scale_tiled, codes->data_ptr(), bytes(*scales), (size_t)rows, (size_t)cols, block, src_fmt,
-                           dst_fmt, oc->data_ptr(), bytes(*os)) == MXQ_OK);
-    return pair(result(a[7], made[0]), result(a[8], made[1]));
+    Output oc, os;
+    GENERAL_UNLESS(codes && scales && oc.take(a[7]) && os.take(a[8]));
+    const int rc = unlocked([&] {
+        oc.make({(int64_t)api.codes_bytes((size_t)(rows * cols), dst_fmt)}, at::kByte, *codes);
+        os.make({(int64_t)api.tiled_scales_bytes((size_t)rows, (size_t)(cols / 32))}, at::kByte, *codes);
+        return api.slice_scale_tiled(codes->data_ptr(), bytes(*scales), (size_t)rows, (size_t)cols, block, src_fmt, dst_fmt, oc.data(),
+                                     os.bytes(), current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return pair(oc.result(a[7]), os.result(a[8]));
     END_HANDLE_TH_ERRORS
 }
 
@@ -303,14 +327,14 @@ PyObject* fake_quant(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     GENERAL_UNLESS(nargs == 6 && a[5] == Py_None && format_id(a[1], &fmt) && as_int(a[2], &block) && as_int(a[3], &mode) &&
                    !modes_active());
     const at::Tensor* src = plain(a[0]);
-    GENERAL_UNLESS(src && dtype_id(*src, &dt));
-    at::Tensor made;
-    const at::Tensor* dst = &made;
-    if (a[4] == Py_None) made = at::empty_like(*src);
-    else dst = plain(a[4]);
-    GENERAL_UNLESS(dst);
-    GENERAL_UNLESS(enqueue(api.fake_quant, src->data_ptr(), dt, (size_t)src->numel(), fmt, block, mode, dst->data_ptr()) == MXQ_OK);
-    return result(a[4], made);
+    Output dst;
+    GENERAL_UNLESS(src && dtype_id(*src, &dt) && dst.take(a[4]));
+    const int rc = unlocked([&] {
+        dst.make_like(*src);
+        return api.fake_quant(src->data_ptr(), dt, (size_t)src->numel(), fmt, block, mode, dst.data(), current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return dst.result(a[4]);
     END_HANDLE_TH_ERRORS
 }
 
@@ -321,14 +345,14 @@ PyObject* fake_quant_bwd(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     int dt;
     GENERAL_UNLESS(nargs == 3 && a[2] == Py_None && !modes_active());
     const at::Tensor* g = plain(a[0]);
-    GENERAL_UNLESS(g && dtype_id(*g, &dt));
-    at::Tensor made;
-    const at::Tensor* dst = &made;
-    if (a[1] == Py_None) made = at::empty_like(*g);
-    else dst = plain(a[1]);
-    GENERAL_UNLESS(dst);
-    GENERAL_UNLESS(enqueue(api.fake_quant_bwd, g->data_ptr(), dt, (size_t)g->numel(), dst->data_ptr()) == MXQ_OK);
-    return result(a[1], made);
+    Output dst;
+    GENERAL_UNLESS(g && dtype_id(*g, &dt) && dst.take(a[1]));
+    const int rc = unlocked([&] {
+        dst.make_like(*g);
+        return api.fake_quant_bwd(g->data_ptr(), dt, (size_t)g->numel(), dst.data(), current_stream());
+    });
+    GENERAL_UNLESS(rc == MXQ_OK);
+    return dst.result(a[1]);
     END_HANDLE_TH_ERRORS
 }
 
@@ -348,15 +372,18 @@ PyObject* run_prepared(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     auto ptr = [&](int i) { return reinterpret_cast<void*>(v[i]); };
     auto u8 = [&](int i) { return reinterpret_cast<uint8_t*>(v[i]); };
     auto num = [&](int i) { return (int)v[i]; };
-    int rc = MXQ_ERR_FORMAT;
-    switch (PyLong_AsLong(a[0])) {
-    case 0: rc = enqueue(api.quantize, ptr(0), num(1), (size_t)v[2], num(3), num(4), ptr(5), u8(6)); break;
-    case 1: rc = enqueue(api.slice_scale, ptr(0), u8(1), (size_t)v[2], num(3), num(4), num(5), ptr(6), u8(7)); break;
-    case 2: rc = enqueue(api.dequantize, ptr(0), u8(1), (size_t)v[2], num(3), num(4), ptr(5), num(6)); break;
-    case 3: rc = enqueue(api.fake_quant, ptr(0), num(1), (size_t)v[2], num(3), num(4), num(5), ptr(6)); break;
-    case 4: rc = enqueue(api.fake_quant_bwd, ptr(0), num(1), (size_t)v[2], ptr(3)); break;
-    default: break;
-    }
+    const long kind = PyLong_AsLong(a[0]);
+    const int rc = unlocked([&] {
+        const mxq_stream s = current_stream();
+        switch (kind) {
+        case 0: return api.quantize(ptr(0), num(1), (size_t)v[2], num(3), num(4), ptr(5), u8(6), s);
+        case 1: return api.slice_scale(ptr(0), u8(1), (size_t)v[2], num(3), num(4), num(5), ptr(6), u8(7), s);
+        case 2: return api.dequantize(ptr(0), u8(1), (size_t)v[2], num(3), num(4), ptr(5), num(6), s);
+        case 3: return api.fake_quant(ptr(0), num(1), (size_t)v[2], num(3), num(4), num(5), ptr(6), s);
+        case 4: return api.fake_quant_bwd(ptr(0), num(1), (size_t)v[2], ptr(3), s);
+        default: return (int)MXQ_ERR_FORMAT;
+        }
+    });
     return PyLong_FromLong(rc);
     END_HANDLE_TH_ERRORS
 }
@@ -422,6 +449,7 @@ PyObject* fake_quant_ste(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     GENERAL_UNLESS(x && dtype_id(*x, &dt) && !x->_fw_grad(0).defined() && !transforms);
     at::Tensor y;
     try {
+        Unlocked u;
         y = FakeQuantSTE::apply(*x, (int64_t)fmt, (int64_t)block, (int64_t)mode, a[4] == Py_True);
     } catch (const NotPlain&) {
         Py_RETURN_NONE;

@@ -3,6 +3,9 @@ path: the same results with and without given outputs, on given streams, for sub
 the same errors as ever, and the straight-through estimator inside autograd."""
 from __future__ import annotations
 
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -130,6 +133,63 @@ def test_a_refused_backward_raises_the_library_s_error(general):
 
     status, text = step()
     assert (status, text) == general(step) and "MXQ_ERR_ALIGN" in text
+
+
+def per_tensor_calls():
+    """One plain call of every native function, all outputs left to it; nothing but arguments is prepared."""
+    x = torch.randn(64, 128, device="cuda")
+    codes, scales = mxq.quantize(x, "e4m3")
+    n, leaf = x.numel(), torch.randn(8, 64, device="cuda").requires_grad_()
+    h = binding._host
+    return {
+        "quantize": lambda: h.quantize(x, "int6", 32, None, None, None),
+        "slice_scale": lambda: h.slice_scale(codes, scales, n, "e4m3", "e2m3", 32, None, None, None),
+        "slice_scale_multi": lambda: h.slice_scale_multi(codes, scales, n, "e4m3", ["e2m3", "e2m1"], 32, None, None),
+        "dequantize": lambda: h.dequantize(codes, scales, n, "e4m3", 32, torch.float32, None, None),
+        "quantize_tiled": lambda: h.quantize_tiled(x, "e4m3", 32, None, None, None),
+        "slice_scale_tiled": lambda: h.slice_scale_tiled(codes, scales, 64, 128, "e4m3", "e2m1", 32, None, None, None),
+        "fake_quant": lambda: h.fake_quant(x, "int4", 32, mxq.FQ_VIA_ANCHOR, None, None),
+        "fake_quant_bwd": lambda: h.fake_quant_bwd(x, None, None),
+        "fake_quant_ste": lambda: h.fake_quant_ste(leaf, "int4", 32, mxq.FQ_VIA_ANCHOR, False),
+    }
+
+
+def test_launches_and_allocations_leave_the_interpreter_s_lock_to_other_threads(tmp_path):
+    """A launch waits when the queue is full and an allocation may wait for the device.  Every entry point is
+    replaced by PyGILState_Check (0 -- the status of success -- without the lock, 1 with it), and the outputs come from an
+    allocator that notes the same."""
+    calls = per_tensor_calls()
+    torch.cuda.synchronize()
+    src = tmp_path / "note.c"
+    src.write_text("int PyGILState_Check(void);\nint notes, held;\nint (*device_malloc)(void **, unsigned long);\n"
+                   "int (*device_free)(void *);\n"
+                   "void *take(long n, int device, void *stream) { void *p = 0; ++notes; held += PyGILState_Check();"
+                   " return device_malloc(&p, (unsigned long)n) ? 0 : p; }\n"
+                   "void give(void *p, long n, int device, void *stream) { device_free(p); }\n")
+    so = str(tmp_path / "note.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", so, str(src)], check=True)
+    note, runtime, lib = ctypes.CDLL(so), ctypes.CDLL("libcudart.so.12"), mxq.load_library()
+
+    def address(f):
+        return ctypes.cast(f, ctypes.c_void_p).value
+
+    ctypes.c_void_p.in_dll(note, "device_malloc").value = address(runtime.cudaMalloc)
+    ctypes.c_void_p.in_dll(note, "device_free").value = address(runtime.cudaFree)
+    allocator = torch.cuda.memory.CUDAPluggableAllocator(so, "take", "give")
+    real = {name: address(getattr(lib, name)) for name in binding._HOST_CALLS}
+    checks = {name: a if name.endswith("_bytes") else address(ctypes.pythonapi.PyGILState_Check) for name, a in real.items()}
+    p = mxq.prepare_fake_quant(torch.empty(32, device="cuda"), "int4", 32, 0, torch.empty(32, device="cuda"))
+    binding._host.bind(checks, binding.FORMATS, torch.nn.Parameter, mxq.MxqError)
+    try:
+        assert binding._host.run_prepared(p.kind, p.packed) == 0
+        for name, call in calls.items():
+            before = ctypes.c_int.in_dll(note, "notes").value
+            with torch.cuda.use_mem_pool(torch.cuda.MemPool(allocator.allocator())):
+                assert call() is not None, name + " launches with the lock held"
+            assert ctypes.c_int.in_dll(note, "notes").value > before
+            assert ctypes.c_int.in_dll(note, "held").value == 0, name + " allocates with the lock held"
+    finally:
+        binding._host.bind(real, binding.FORMATS, torch.nn.Parameter, mxq.MxqError)
 
 
 def test_graph_capture_and_side_stream():
