@@ -157,6 +157,16 @@ PyObject* pair(PyObject* a, PyObject* b)
 
 uint8_t* bytes(const at::Tensor& t) { return static_cast<uint8_t*>(t.data_ptr()); }
 
+// Sets MxqError(rc, what) as the Python error.
+PyObject* raise_mxq_error(int rc, const char* what)
+{
+    if (PyObject* e = PyObject_CallFunction(mxq_error, "is", rc, what)) {
+        PyErr_SetObject(mxq_error, e);
+        Py_DECREF(e);
+    }
+    return nullptr;
+}
+
 #define GENERAL_UNLESS(cond) \
     if (!(cond)) Py_RETURN_NONE
 
@@ -232,6 +242,8 @@ PyObject* slice_scale_multi(PyObject*, PyObject* const* a, Py_ssize_t nargs)
         return api.slice_scale_multi(codes->data_ptr(), bytes(*scales), (size_t)n, block, src_fmt, (int)k, fmts, pc, ps,
                                      current_stream());
     });
+    // (other launches of the call may precede the one that failed: the general path would enqueue them again)
+    if (rc == MXQ_ERR_CUDA) return raise_mxq_error(rc, "mxq_slice_scale_multi");
     GENERAL_UNLESS(rc == MXQ_OK);
     PyObject* list = PyList_New(k);
     if (!list) return nullptr;
@@ -396,10 +408,7 @@ struct NotPlain {};                    // the launch was refused: the general pa
 [[noreturn]] void throw_mxq_error(int rc, const char* what)
 {
     pybind11::gil_scoped_acquire lock;
-    if (PyObject* e = PyObject_CallFunction(mxq_error, "is", rc, what)) {
-        PyErr_SetObject(mxq_error, e);
-        Py_DECREF(e);
-    }
+    raise_mxq_error(rc, what);
     python_error raised;
     raised.persist();
     throw python_error(std::move(raised));

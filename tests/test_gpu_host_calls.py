@@ -192,6 +192,20 @@ def test_launches_and_allocations_leave_the_interpreter_s_lock_to_other_threads(
         binding._host.bind(real, binding.FORMATS, torch.nn.Parameter, mxq.MxqError)
 
 
+def test_a_failed_launch_among_several_is_not_enqueued_again():
+    x = torch.randn(64, 128, device="cuda")
+    codes, scales = mxq.quantize(x, "int8")
+    real = {name: ctypes.cast(getattr(mxq.load_library(), name), ctypes.c_void_p).value for name in binding._HOST_CALLS}
+    failed = ctypes.CFUNCTYPE(ctypes.c_int)(lambda: -7)                 # MXQ_ERR_CUDA, whatever was launched before it
+    binding._host.bind({**real, "mxq_slice_scale_multi": ctypes.cast(failed, ctypes.c_void_p).value}, binding.FORMATS,
+                       torch.nn.Parameter, mxq.MxqError)
+    try:
+        with pytest.raises(mxq.MxqError, match="mxq_slice_scale_multi.*MXQ_ERR_CUDA"):
+            mxq.slice_scale_multi(codes, scales, x.numel(), "int8", ["int7", "int6", "int5", "int4", "int3"])
+    finally:
+        binding._host.bind(real, binding.FORMATS, torch.nn.Parameter, mxq.MxqError)
+
+
 def test_graph_capture_and_side_stream():
     x = torch.randn(64, 128, device="cuda")
     want = [t.clone() for t in mxq.quantize(x, "e4m3")]
