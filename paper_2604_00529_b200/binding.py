@@ -441,10 +441,14 @@ class PreparedCall:
 
     def __init__(self, fn, args, what, keep):
         self.fn, self.args, self.what, self.keep = fn, args, what, keep
-        self.kind, self.packed = _PREPARED.index(what), struct.pack("9q", *args, *(0,) * (9 - len(args)))
+        self.kind = _PREPARED.index(what)
+        try:
+            self.packed = struct.pack("9q", *args, *(0,) * (9 - len(args)))
+        except struct.error:
+            self.packed = None          # no 64-bit integers: ctypes converts or refuses them at the call
 
     def __call__(self, stream=None) -> None:
-        if stream is None:
+        if stream is None and self.packed is not None:
             rc = _host.run_prepared(self.kind, self.packed)
         else:
             rc = self.fn(*self.args, _stream(stream))

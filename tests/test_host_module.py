@@ -1,9 +1,12 @@
-"""How the binding's native module is built: what it links, and when it is built again."""
+"""How the binding's native module is built, and what the binding hands to it."""
 from __future__ import annotations
 
+import ctypes
 import subprocess
 
-from paper_2604_00529_b200 import build
+import pytest
+
+from paper_2604_00529_b200 import binding, build
 
 
 def test_one_cpp_runtime_in_the_process():
@@ -11,3 +14,16 @@ def test_one_cpp_runtime_in_the_process():
     so = build.build_host_module()
     dynamic = subprocess.run(["readelf", "-d", so], capture_output=True, text=True, check=True).stdout
     assert "[libstdc++.so.6]" in dynamic and "[libtorch_python.so]" in dynamic
+
+
+def test_prepared_calls_leave_other_arguments_to_the_call(monkeypatch):
+    """What is no 64-bit integer is converted (a count beyond 2^63 modulo 2^64) or refused when the call is made."""
+    seen = []
+    fn = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)(
+        lambda *a: seen.append(a) or 0)
+    monkeypatch.setattr(binding, "_stream", lambda stream: 9)
+    binding.PreparedCall(fn, (64, 1, 2 ** 64 - 32, 128), "mxq_fake_quant_bwd", ())()
+    assert seen == [(64, 1, 2 ** 64 - 32, 128, 9)]
+    refused = binding.PreparedCall(fn, (64, 1, 32.0, 128), "mxq_fake_quant_bwd", ())
+    with pytest.raises(ctypes.ArgumentError):
+        refused()
