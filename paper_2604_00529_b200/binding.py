@@ -6,6 +6,7 @@ the current CUDA stream's handle.  Code and scale buffers are ``torch.uint8`` te
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import struct
 from typing import Optional, Sequence, Tuple
@@ -76,15 +77,17 @@ def load_library() -> ctypes.CDLL:
     global _lib, _host
     if _lib is not None:
         return _lib
+    from .build import host_module_path
     if not os.path.exists(_LIB_PATH):
         raise ImportError("libmxq.so is not built: run `python -m paper_2604_00529_b200.build` "
                           "(there is no fallback path)")
     if _host is None:
-        try:
-            from . import _mxq_host
-        except ImportError as e:
-            raise ImportError("_mxq_host.so is not built for this torch: run `python -m paper_2604_00529_b200.build`") from e
-        _host = _mxq_host
+        path = host_module_path()
+        if not os.path.exists(path):
+            raise ImportError("%s, the binding's module for this torch and Python, is not built: run "
+                              "`python -m paper_2604_00529_b200.build`" % os.path.basename(path))
+        spec = importlib.util.spec_from_file_location(__package__ + "._mxq_host", path)
+        _host = importlib.util.module_from_spec(spec)
     L = ctypes.CDLL(_LIB_PATH)
     vp, sz, i = ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int
     L.mxq_status_string.argtypes = [i]

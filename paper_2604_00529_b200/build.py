@@ -3,15 +3,17 @@
     python -m paper_2604_00529_b200.build [--force] [--debug]
 
 One object per translation unit under ``_build/`` (compiled in parallel), linked into
-``paper_2604_00529_b200/libmxq.so``; then ``mxq_abi_timing``, a small C-level caller of the ABI, and ``_mxq_host.so``,
-the native part of the Python binding.  A unit is rebuilt when it or any header is newer than
-its object.
+``paper_2604_00529_b200/libmxq.so``; then ``mxq_abi_timing``, a small C-level caller of the ABI, and ``_mxq_host``,
+the native part of the Python binding (for the torch and Python at hand).  A unit is rebuilt when it or any header is
+newer than its object.
 """
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -19,7 +21,6 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libmxq.so")
-HOST_MODULE = os.path.join(HERE, "_mxq_host.so")       # the binding's native calls (csrc/host_calls.cpp)
 TIMING_EXE = os.path.join(HERE, "mxq_abi_timing")      # C-level caller of the ABI (csrc/abi_timing.cu)
 UNITS = ["mxq_api", "mxq_quantize", "mxq_slice_scale", "mxq_dequantize", "mxq_fake_quant", "mxq_static_batch", "mxq_slice_scale_multi", "mxq_slice_scale_multi_fp", "mxq_layout", "mxq_fake_quant_batched"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-std=c++20", "-O3", "-lineinfo",
@@ -58,17 +59,23 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     return lib
 
 
-def build_host_module(force: bool = False) -> str:
-    """Builds _mxq_host.so, the CPython module that binding.py imports, against the installed torch."""
-    src = os.path.join(CSRC, "host_calls.cpp")
-    if not (force or _stale(HOST_MODULE, [src, os.path.join(ROOT, "include", "mxq.h"), os.path.abspath(__file__)])):
-        return HOST_MODULE
-    import sysconfig
+def host_module_path() -> str:
+    """The file of _mxq_host for the torch and the Python that run: it holds the C++ layouts of the one and the ABI of the
+    other, so each combination has a module of its own."""
+    import torch
+    return os.path.join(HERE, "_mxq_host.torch-%s-abi%d%s" % (re.sub(r"[^0-9A-Za-z.]", "_", torch.__version__),
+                                                             torch.compiled_with_cxx11_abi(), sysconfig.get_config_var("EXT_SUFFIX")))
 
+
+def build_host_module(force: bool = False) -> str:
+    """Builds _mxq_host, the CPython module of binding.py (csrc/host_calls.cpp), against the installed torch."""
+    src, target = os.path.join(CSRC, "host_calls.cpp"), host_module_path()
+    if not (force or _stale(target, [src, os.path.join(ROOT, "include", "mxq.h"), os.path.abspath(__file__)])):
+        return target
     import torch
     top = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
-    tmp = HOST_MODULE + ".tmp.%d" % os.getpid()
+    tmp = target + ".tmp.%d" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
     for d in (os.path.join(top, "include"), os.path.join(top, "include", "torch", "csrc", "api", "include"),
@@ -81,8 +88,8 @@ def build_host_module(force: bool = False) -> str:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("g++ failed: %s\n%s" % (" ".join(cmd), r.stderr))
-    os.replace(tmp, HOST_MODULE)
-    return HOST_MODULE
+    os.replace(tmp, target)
+    return target
 
 
 def _build_library(obj_dir: str, lib: str, extra, force: bool, verbose: bool, timing: bool) -> str:

@@ -5,6 +5,7 @@ import ctypes
 import subprocess
 
 import pytest
+import torch
 
 from paper_2604_00529_b200 import binding, build
 
@@ -27,3 +28,16 @@ def test_prepared_calls_leave_other_arguments_to_the_call(monkeypatch):
     refused = binding.PreparedCall(fn, (64, 1, 32.0, 128), "mxq_fake_quant_bwd", ())
     with pytest.raises(ctypes.ArgumentError):
         refused()
+
+
+def test_each_torch_and_python_has_a_module_of_its_own(monkeypatch):
+    built = build.host_module_path()
+    for target, name, value in ((torch, "__version__", "99.1.0+cu999"), (build.sysconfig, "get_config_var", lambda v: ".cpython-399.so")):
+        with monkeypatch.context() as m:
+            m.setattr(target, name, value)
+            assert build.host_module_path() != built and not build.os.path.exists(build.host_module_path())
+            m.setattr(binding, "_lib", None)
+            m.setattr(binding, "_host", None)
+            with pytest.raises(ImportError, match="not built"):
+                binding.load_library()
+    assert build.host_module_path() == built and binding.load_library() is not None
