@@ -55,8 +55,23 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     if debug:
         return _build_library(os.path.join(ROOT, "_build_debug"), DEBUG_LIB, ["-DMXQ_DEBUG"], force, verbose, timing=False)
     lib = _build_library(OBJ_DIR, LIB, [], force, verbose, timing=True)
-    build_host_module(force)
+    if _torch_folder() is None:
+        print("no torch with CUDA here: the C library is built, the Python binding's _mxq_host is not", file=sys.stderr)
+    else:
+        build_host_module(force)
     return lib
+
+
+def _torch_folder():
+    """The folder of a torch that _mxq_host can be built against (its headers and CUDA libraries), or None: users of the C
+    library alone need neither."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    top = os.path.dirname(torch.__file__)
+    need = (("include", "torch", "csrc", "autograd", "custom_function.h"), ("lib", "libtorch_python.so"), ("lib", "libc10_cuda.so"))
+    return top if all(os.path.exists(os.path.join(top, *n)) for n in need) else None
 
 
 def host_module_path() -> str:
@@ -73,7 +88,9 @@ def build_host_module(force: bool = False) -> str:
     if not (force or _stale(target, [src, os.path.join(ROOT, "include", "mxq.h"), os.path.abspath(__file__)])):
         return target
     import torch
-    top = os.path.dirname(torch.__file__)
+    top = _torch_folder()
+    if top is None:
+        raise RuntimeError("_mxq_host needs a torch with its headers and CUDA libraries; %s has none" % torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
     tmp = target + ".tmp.%d" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",

@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import ctypes
 import subprocess
+import sys
 
 import pytest
 import torch
@@ -41,3 +42,16 @@ def test_each_torch_and_python_has_a_module_of_its_own(monkeypatch):
             with pytest.raises(ImportError, match="not built"):
                 binding.load_library()
     assert build.host_module_path() == built and binding.load_library() is not None
+
+
+def test_the_c_library_builds_without_torch(monkeypatch, tmp_path, capsys):
+    built = []
+    monkeypatch.setattr(build, "_build_library", lambda *a, **k: built.append(a) or "libmxq.so")
+    (tmp_path / "torch").mkdir()
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__file__", str(tmp_path / "torch" / "__init__.py"))        # a torch without CUDA libraries
+        assert build.build() == "libmxq.so"
+    with monkeypatch.context() as m:
+        m.setitem(sys.modules, "torch", None)                                        # none at all
+        assert build.build() == "libmxq.so"
+    assert len(built) == 2 and capsys.readouterr().err.count("_mxq_host is not") == 2
