@@ -1,9 +1,11 @@
 #!/usr/bin/env python
 """Benchmark of the MX (re)quantization hot path on B200.
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl mxq|reference] [--workloads w1,w2,w3,w4,w5]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl mxq|reference] [--workloads w1,w2,w3,w4,w5] [--record FILE]
 
-One invocation times all five workloads of the method and prints ONE JSON line on stdout.
+One invocation times all five workloads of the method and prints ONE JSON line on stdout: the headline with its
+configuration, clocks, roofline and baselines.  The whole record (`kernels`, `workloads` and every note) is some 20 KB and
+goes to --record FILE, or to stderr: whoever reads the line from the tail of a log gets it whole.
 
 Headline (`value`, `config.workload`): the whole-model workload -- the 224 BF16 linear weights of an 8B
 Llama-shaped decoder (6.98 G elements).  A *step* is one pass of the whole hot path over that weight
@@ -14,7 +16,7 @@ of all weights through the anchor (Eq. 6) and its straight-through backward.  18
 traffic per step, every buffer far larger than L2.  K steps run back to back between two CUDA events;
 events between the steps and between the op groups give the spread and the per-kernel durations.
 
-`workloads` in the line carries the other four (and the per-target conversion times of the headline
+`workloads` in the record carries the other four (and the per-target conversion times of the headline
 one): w1 the FP32 4096 x 4096 matrix (quantize -> MXINT8 -> MXINT4 -> reconstruct), w2 the BF16
 8192 x 8192 Student-t matrix through a 12-launch step, w4 the fake-quant of a [8, 4096, 4096]
 activation tensor with the format sampled by seed, w5 the size sweep 2^16 ... 2^31.  Every figure there
@@ -985,9 +987,30 @@ def run_cuda(args):
         "clocks": clocks,
         "bench_seconds": round(time.perf_counter() - t_begin, 1),
     }
-    print(json.dumps(line), flush=True)
+    write_record(line, args.record)
+    print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+def headline(record: dict) -> dict:
+    """The part of the record that is printed on stdout."""
+    line = {k: v for k, v in record.items() if k not in ("kernels", "workloads")}
+    for part, dropped in (("config", ("inputs", "timing")), ("roofline", ("note",)), ("e2e", ("what",))):
+        line[part] = {k: v for k, v in record[part].items() if k not in dropped}
+    cpu = record["cpu_baseline"]
+    if cpu:
+        line["cpu_baseline"] = {**cpu, "single_thread": {k: v for k, v in cpu["single_thread"].items() if k != "sample"}}
+    return line
+
+
+def write_record(record: dict, path: str | None) -> None:
+    text = json.dumps(record)
+    if path:
+        with open(path, "w") as f:
+            f.write(text + "\n")
+    else:
+        print(text, file=sys.stderr, flush=True)
 
 
 def run_ncu_case(args):
@@ -1125,6 +1148,7 @@ def main():
     ap.add_argument("--buffer-sets", type=int, default=4, help="rotating buffer sets of workload 2 (>= 2)")
     ap.add_argument("--case-log2", type=int, default=30,
                     help="--impl ncu-case: 2^N codes for Slice-and-Scale, 2^(N-1) elements for the other kernels")
+    ap.add_argument("--record", help="write the whole record to this file instead of to stderr")
     ap.add_argument("--no-cpu-baseline", action="store_true", help="skip the oracle timing (profiling runs)")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)

@@ -53,6 +53,39 @@ def test_clock_windows():
     assert bench.ClockSampler(0).summary(0, 1)["samples"] == 0
 
 
+def test_the_line_on_stdout_fits_the_tail_of_a_log(tmp_path, capsys):
+    """Everything a run states about the headline, without the per-workload figures, in well under 3000 characters."""
+    names = [name for name, _ in bench.STEP_OPS]
+    cpu = {"value": 0.972, "unit": "GB/s", "cores": 16, "kind": "oracle", "sample": "s" * 130, "melem_s": 375.65,
+           "single_thread": {"value": 0.0635, "unit": "GB/s", "cores": 1, "melem_s": 24.53, "sample": "s" * 130}}
+    record = {
+        "metric": bench.METRIC, "value": 6751.7, "unit": "GB/s", "n_gpus": 8, "steps": 20, "warmup": 5, "ms_per_step": 26.7471,
+        "ms_per_step_spread": {"median": 26.471, "min": 25.836, "max": 28.447}, "higher_is_better": True, "scaling": "weak",
+        "vs_baseline": None, "dtype": "bf16", "data": "synthetic", "impl": "mxq",
+        "config": {"workload": bench.HEADLINE, "elements_per_gpu": 6979321856, "tensors": 224, "block": 32, "ops_per_step": names,
+                   "bytes_per_step_per_gpu": 180589953024, "gelem_per_s": 2609.37, "inputs": "i" * 200, "l2": "l" * 80, "timing": "t" * 250},
+        "e2e": {"value": 383.8, "unit": "GB/s", "h2d_bytes_per_step": 13958643712, "d2h_bytes_per_step": 18320719872, "steps": 3,
+                "ms_per_step": 470.6, "what": "w" * 90},
+        "gpu_launches": 200, "gpu_launches_all_workloads": 123456,
+        "roofline": {"bound": "hbm", "kernel": names[-1], "achieved": 7008.7, "peak": 6457.4, "unit": "GB/s", "frac": 1.0854,
+                     "faster_than_the_copy_peak": True, "peak_kind": "measured", "traffic": 27917287424, "bytes_per_launch": 27917287424,
+                     "ms_per_launch": 3.983, "ncu_dram_pct_of_peak": 84.0, "note": "n" * 230},
+        "kernels": {name: {"ms": 1.0} for name in names}, "workloads": {"w5_size_sweep": {"x": "y" * 15000}}, "cpu_baseline": cpu,
+        "clocks": {"sm_mhz": 1590.0, "sm_min_mhz": 1470.0, "sm_max_mhz": 1965.0, "samples": 53, "how": "h" * 40,
+                   "reasons": ["sw_power_cap"]}, "bench_seconds": 28.1}
+    line = bench.headline(record)
+    assert len(json.dumps(line)) < 2500
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                "dtype", "data", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"):
+        assert key in line
+    assert line["config"]["workload"] == bench.HEADLINE and line["config"]["l2"] and "single_thread" in line["cpu_baseline"]
+    assert bench.headline({**record, "cpu_baseline": None})["cpu_baseline"] is None
+    bench.write_record(record, str(tmp_path / "record.json"))
+    assert json.load(open(tmp_path / "record.json")) == record and capsys.readouterr() == ("", "")
+    bench.write_record(record, None)
+    assert json.loads(capsys.readouterr().err) == record
+
+
 def test_reps_for():
     assert bench.reps_for(3.0) == 50 and bench.reps_for(1000.0) == 2 and bench.reps_for(100.0) == 15
 
