@@ -1029,16 +1029,6 @@ __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ cod
     if constexpr (StagedTile<OB>::use) {
         const size_t first = tile * (32 * U), left = nunits - first;
         flush_stage<32 * U * OB>(stage, out_codes + first * OB, (uint32_t)(left < 32 * U ? left : 32 * U) * OB);
-    }    if constexpr (!HALVES) {
-        // (Not reached by the entry points, whose block 16 takes HALVES; without it the compiler's schedule for the larger
-        // blocks is slower: MXINT8 -> MXINT4 of 2^24 codes and back to FP32 17.5 us against 17.2.)
-        if (nscales > nunits) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const size_t i = nunits + u0 + u * 32;
-                if (i < nscales) put_scale(out_scales, i, ss_scale_byte(ld_u8(scales + i), de));
-            }
-        }
     }
 }
 
