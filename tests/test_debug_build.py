@@ -13,7 +13,7 @@ import torch
 
 from oracle import mxq_oracle as orc
 from paper_2604_00529_b200 import inputs
-from paper_2604_00529_b200.binding import FORMATS, _DqItem, _FqItem, _Item, _QItem
+from paper_2604_00529_b200.binding import FORMATS, _DqItem, _FqItem, _Item, _PairItem, _QItem, _TiledItem
 
 from gpu_util import to_dev, to_host
 
@@ -140,6 +140,85 @@ def test_batched_entry_points_stay_inside_their_buffers(D):
         assert np.array_equal(to_host(lc2[j]), orc.pack(w4, 4)) and np.array_equal(to_host(ls2[j]), s4), j
         want = orc.dequantize(w4, s4, "e2m1", out_dtype=orc.BF16)
         assert np.array_equal(to_host(y[j]), want) and np.array_equal(to_host(f[j]), want), j
+
+
+@pytest.mark.parametrize("src,lows", [("int8", ["int7", "int6", "int5", "int3"]), ("e4m3", ["e3m3", "e2m3", "e2m1"])])
+@pytest.mark.parametrize("units,block", [(1, 32), (31, 16), (257, 16), (258, 64), (516, 128), (771, 32)])
+def test_target_sets_pairs_and_padding_stay_inside_their_buffers(D, src, lows, units, block):
+    """The kernels that read an anchor once for several targets, block 16, and the CTAs that write the padding of tiled
+    scales, in the bounds-checked build."""
+    vp, i = ctypes.c_void_p, ctypes.c_int
+    D.mxq_slice_scale_multi.argtypes = [vp, vp, ctypes.c_size_t, i, i, i, ctypes.POINTER(i), ctypes.POINTER(vp), ctypes.POINTER(vp), vp]
+    D.mxq_slice_scale_pair_batched.argtypes = [ctypes.POINTER(_PairItem), i, i, i, i, i, vp]
+    D.mxq_slice_scale_tiled_batched.argtypes = [ctypes.POINTER(_TiledItem), i, i, i, i, vp]
+    stream = torch.cuda.current_stream().cuda_stream
+    rng = np.random.default_rng(units)
+    n, k = units * 32, len(lows)
+    hc, hs = rng.integers(0, 256, n).astype(np.uint8), rng.integers(0, 256, n // block).astype(np.uint8)
+    codes, scales = to_dev(hc), to_dev(hs)
+    fmts = (i * k)(*[FORMATS[f] for f in lows])
+    launches = 0
+    report(D)
+    sets = [(u8(n * orc.bits(f) // 8), u8(n // block)) for f in lows]
+    assert D.mxq_slice_scale_multi(P(codes), P(scales), n, block, FORMATS[src], k, fmts, (vp * k)(*[P(c) for c, _ in sets]),
+                                   (vp * k)(*[P(s) for _, s in sets]), stream) == 0
+    one = [(u8(n * orc.bits(f) // 8), u8(n // block)) for f in lows]
+    for f, (c, s) in zip(lows, one):
+        assert D.mxq_slice_scale(P(codes), P(scales), n, block, FORMATS[src], FORMATS[f], P(c), P(s), stream) == 0
+    launches += 1 + k
+    results = list(zip(lows * 2, sets + one))
+    if block >= 32:
+        pair = [(u8(n * orc.bits(f) // 8), u8(n // block)) for f in lows[:2]]
+        item = (_PairItem * 1)(_PairItem(P(codes), P(scales), n, P(pair[0][0]), P(pair[0][1]), P(pair[1][0]), P(pair[1][1])))
+        assert D.mxq_slice_scale_pair_batched(item, 1, block, FORMATS[src], FORMATS[lows[0]], FORMATS[lows[1]], stream) == 0
+        launches += 1
+        results += list(zip(lows[:2], pair))
+    if block == 32 and src == "e4m3":
+        rows, kb = (units // 3, 3) if units >= 3 else (1, units)
+        nbytes = D.mxq_tiled_scales_bytes(rows, kb)
+        tiled = [(u8(rows * kb * 16), u8(nbytes)) for _ in range(2)]
+        items = (_TiledItem * 2)(*[_TiledItem(P(codes), P(scales), rows, kb * 32, P(c), P(s)) for c, s in tiled])
+        assert D.mxq_slice_scale_tiled_batched(items, 2, 32, FORMATS[src], FORMATS["e2m1"], stream) == 0
+        launches += 1
+    info = report(D)
+    assert info.checked_launches == launches
+    assert info.violations == 0, "first bad access: %#x (%d bytes)" % (info.first_address, info.first_bytes)
+    for f, (c, s) in results:
+        wc, ws = orc.slice_scale(hc, hs, src, f, block)
+        assert np.array_equal(to_host(c), orc.pack(wc, orc.bits(f))) and np.array_equal(to_host(s), ws), f
+    if block == 32 and src == "e4m3":
+        wc, ws = orc.slice_scale(hc, hs, src, "e2m1", 32)
+        want = orc.tile_scales(ws[:rows * kb].reshape(rows, kb), rows, kb)
+        for c, s in tiled:
+            assert np.array_equal(to_host(c), orc.pack(wc[:rows * kb * 32], 4)) and np.array_equal(to_host(s), want)
+
+
+@pytest.mark.parametrize("block", [16, 32])
+def test_two_unit_kernels_stay_inside_their_buffers(D, block):
+    """A launch large enough for two lane units per thread, with a ragged last warp."""
+    stream = torch.cuda.current_stream().cuda_stream
+    n = (148 * 8 * 256 + 5) * 32
+    period = 1004 * 32                                            # the data repeats; no multiple of a tile
+    rng = np.random.default_rng(block)
+    hc, hs = rng.integers(0, 256, period).astype(np.uint8), rng.integers(0, 256, period // block).astype(np.uint8)
+
+    def whole(pattern, count):
+        p = to_dev(pattern)
+        return p.repeat(-(-count // p.numel()))[:count].contiguous()
+
+    codes, scales = whole(hc, n), whole(hs, n // block)
+    lc, ls = u8(n * 6 // 8), u8(n // block)
+    y = torch.empty(n, dtype=torch.bfloat16, device="cuda")
+    report(D)
+    assert D.mxq_slice_scale(P(codes), P(scales), n, block, FORMATS["e4m3"], FORMATS["e2m3"], P(lc), P(ls), stream) == 0
+    assert D.mxq_dequantize(P(lc), P(ls), n, FORMATS["e2m3"], block, P(y), 1, stream) == 0
+    info = report(D)
+    assert info.checked_launches == 2
+    assert info.violations == 0, "first bad access: %#x (%d bytes)" % (info.first_address, info.first_bytes)
+    wc, ws = orc.slice_scale(hc, hs, "e4m3", "e2m3", block)
+    assert torch.equal(lc, whole(orc.pack(wc, 6), lc.numel())) and torch.equal(ls, whole(ws, ls.numel()))
+    want = orc.dequantize(wc, ws, "e2m3", block, orc.BF16)
+    assert torch.equal(y.view(torch.int16), whole(want.view(np.uint16), n).view(torch.int16))
 
 
 def test_the_checker_counts_and_skips_what_leaves_a_registered_range(D):

@@ -5,10 +5,14 @@ from __future__ import annotations
 
 import ctypes
 import subprocess
+import threading
 
 import numpy as np
 import pytest
 import torch
+import torch.autograd.forward_ad as fwad
+from torch.overrides import TorchFunctionMode
+from torch.utils._python_dispatch import TorchDispatchMode
 
 import paper_2604_00529_b200 as mxq
 from paper_2604_00529_b200 import binding
@@ -115,11 +119,50 @@ def test_straight_through_gradient(general, copy_grad):
         return (y.detach(), *torch.autograd.grad(y * 3, x, g, retain_graph=True))
 
     assert same(step(), general(step))
+    node = mxq.fake_quant_ste(x * 2, "e2m1", copy_grad=copy_grad).grad_fn
+    assert "CppFunction" in type(node).__name__ and "Mul" in type(node.next_functions[0][0]).__name__
     with torch.no_grad():
         assert not mxq.fake_quant_ste(x, "e2m1").requires_grad
     assert not mxq.fake_quant_ste(x.detach(), "e2m1").requires_grad
     (first,) = torch.autograd.grad(mxq.fake_quant_ste(x, "e2m1", copy_grad=copy_grad).pow(3).sum(), x, create_graph=True)
     assert first.requires_grad != copy_grad                     # the copied gradient is a constant, as through the general path
+
+
+@pytest.mark.parametrize("copy_grad", [False, True])
+def test_hooks_batched_gradients_and_forward_mode(general, copy_grad):
+    x = torch.randn(8, 64, device="cuda").requires_grad_()
+
+    def ste(t):
+        return mxq.fake_quant_ste(t, "int4", 32, mxq.FQ_VIA_ANCHOR, copy_grad)
+
+    def hooked():
+        leaf, seen = x.detach().clone().requires_grad_(), []
+        y = ste(leaf * 2)
+        y.retain_grad()
+        y.register_hook(lambda g: seen.append(g) or g * 2)
+        y.grad_fn.register_prehook(lambda go: (go[0] * 3,))
+        y.grad_fn.register_hook(lambda gi, go: seen.append(gi[0]) or seen.append(go[0]))
+        y.pow(2).sum().backward()
+        return (leaf.grad, y.grad, *seen)
+
+    def strided():
+        return torch.autograd.grad(ste(x * 2), x, torch.arange(512.0, device="cuda").view(64, 8).t())
+
+    for step in (hooked, strided):
+        assert same(step(), general(step))
+    grads = torch.randn(3, 8, 64, device="cuda")
+
+    def batched():
+        return torch.autograd.grad(ste(x), x, grads, is_grads_batched=True)
+
+    if copy_grad:                                               # a copy needs memory of its own: refused as ever
+        for run in (lambda fn: fn(), general):
+            with pytest.raises(RuntimeError, match="storage"):
+                run(batched)
+    else:
+        assert same(batched(), (grads,)) and same(general(batched), (grads,))
+    with fwad.dual_level(), pytest.raises(NotImplementedError):
+        ste(fwad.make_dual(x.detach(), torch.ones_like(x)))
 
 
 def test_a_refused_backward_raises_the_library_s_error(general):
@@ -152,6 +195,84 @@ def per_tensor_calls():
         "fake_quant_bwd": lambda: h.fake_quant_bwd(x, None, None),
         "fake_quant_ste": lambda: h.fake_quant_ste(leaf, "int4", 32, mxq.FQ_VIA_ANCHOR, False),
     }
+
+
+class Sub(torch.Tensor):
+    pass
+
+
+class FunctionMode(TorchFunctionMode):
+    def __torch_function__(self, func, types, args=(), kwargs=None):
+        return func(*args, **(kwargs or {}))
+
+
+class DispatchMode(TorchDispatchMode):
+    def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+        return func(*args, **(kwargs or {}))
+
+
+def test_the_plain_case_is_handled_natively_and_nothing_else():
+    calls = per_tensor_calls()
+    for name, call in calls.items():
+        assert call() is not None, name
+        with FunctionMode():
+            assert call() is None, name
+        with DispatchMode():
+            assert call() is None, name
+    h, x = binding._host, torch.randn(64, 128, device="cuda")
+    codes, scales = h.quantize(x, "e4m3", 32, None, None, None)
+    n, stream = x.numel(), torch.cuda.current_stream()
+    out = torch.empty_like(codes)
+    assert h.quantize(x, "e4m3", 32, out, scales, None)[0] is out
+    for given in (out.cpu(), out.view(2, -1).t(), out.as_subclass(Sub)):
+        assert h.quantize(x, "e4m3", 32, given, None, None) is None
+    for src in (x.as_subclass(Sub), x.t(), x.cpu(), x.half(), x.to_sparse(), x.to("meta"), None):
+        assert h.quantize(src, "e4m3", 32, None, None, None) is None
+        assert h.fake_quant(src, "int4", 32, 0, None, None) is None
+        assert h.fake_quant_ste(src, "int4", 32, 0, False) is None
+    assert h.quantize(x, "e4m3", 32, None, None, stream) is None
+    assert h.slice_scale(codes, scales, n, "e4m3", "e2m1", 32, None, None, stream) is None
+    assert h.slice_scale(codes, scales, float(n), "e4m3", "e2m1", 32, None, None, None) is None
+    assert h.slice_scale_multi(codes, scales, n, "e4m3", iter(["e2m1"]), 32, None, None) is None
+    assert h.dequantize(codes, scales, n, "e4m3", 32, torch.float16, None, None) is None
+    assert h.fake_quant(x, "int4", True, 0, None, None) is None
+    with fwad.dual_level():
+        assert h.fake_quant_ste(fwad.make_dual(x.clone(), torch.ones_like(x)), "int4", 32, 0, False) is None
+    seen = []
+    torch.jit.trace(lambda t: seen.append(h.fake_quant_ste(t * 2, "int4", 32, 0, False)) or t * 2, (x,), check_trace=False)
+    torch.func.vmap(lambda t: seen.append(h.fake_quant_ste(x, "int4", 32, 0, False)) or t)(x)
+    torch.func.grad(lambda t: (seen.append(h.fake_quant(t, "int4", 32, 0, None, None)), t.sum())[1])(x)
+    assert seen == [None, None, None]
+
+
+def test_subclasses_modes_and_threads_get_the_results_of_the_general_path(general):
+    x = torch.randn(64, 128, device="cuda")
+    sub = x.as_subclass(Sub)
+    want = general(lambda: (*mxq.quantize(x, "int6"), mxq.fake_quant(x, "int4"), mxq.fake_quant_ste(x, "int4")))
+
+    def all_of(t):
+        return (*mxq.quantize(t, "int6"), mxq.fake_quant(t, "int4"), mxq.fake_quant_ste(t, "int4"))
+
+    assert all(type(a) is type(b) for a, b in zip(all_of(sub), general(lambda: all_of(sub))))
+    got = [tuple(t.as_subclass(torch.Tensor) for t in all_of(sub))]
+    for mode in (FunctionMode, DispatchMode, torch.inference_mode, torch.no_grad):
+        with mode():
+            got.append(all_of(x))
+    stream = torch.cuda.current_stream()
+
+    def worker():
+        with torch.cuda.stream(stream):
+            got.append(all_of(x))
+
+    threads = [threading.Thread(target=worker) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert len(got) == 9
+    for g in got:
+        assert all(torch.equal(a, b) for a, b in zip(g, want))
 
 
 def test_launches_and_allocations_leave_the_interpreter_s_lock_to_other_threads(tmp_path):
