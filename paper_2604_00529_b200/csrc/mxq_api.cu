@@ -261,7 +261,7 @@ int mxq_fake_quant_batched(const mxq_fq_item* items, int count, int dtype, int f
         d.dst = static_cast<uint8_t*>(it.dst);
         d.nunits = it.n / epl;
         d.tile_begin = tiles;
-        tiles += fq_batched_tiles(d.nunits, dtype);
+        tiles += fq_batched_tiles(d.nunits);
         chunk.push_back(d);
         if ((int)chunk.size() == kFqBatchItemsMax)
             if (int rc = flush()) return rc;

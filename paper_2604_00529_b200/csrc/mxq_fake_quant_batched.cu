@@ -6,12 +6,9 @@ namespace mxq {
 namespace {
 
 constexpr int kU = 1;
-// Consecutive warp tiles of one tensor per warp.  1 / 2 / 4 take 547 / 498 / 542 us (BF16, MXINT4 through the anchor) and
-// 539 / 499 / 543 us (BF16, E2M3) over four decoder layers; 1 / 2 take 996 / 1013 us (FP32, MXINT4), 1003 / 1012 (FP32,
-// E2M3) and 986 / 1011 (FP32, E4M3).  A tile is 1 KB in either type: BF16 does twice the arithmetic on it and gains from one
-// lookup for two tiles; FP32 waits for memory alone, and two warps with a tile each ask for it earlier than one.
-template <class T>
-constexpr int kR = T::size == 4 ? 1 : 2;
+// Consecutive warp tiles of one tensor per warp: 1 / 2 / 4 take 996 / 1013 / 1098 us (FP32, MXINT4 through the anchor),
+// 547 / 498 / 542 us (BF16, the same) and 539 / 499 / 543 us (BF16, E2M3) over four decoder layers.
+constexpr int kR = 2;
 constexpr int kThreads = 128;
 
 template <class T, class F, int BLOCK, int MODE>
@@ -24,7 +21,7 @@ int run(const FqDeviceItem* items_host, int count, size_t total_tiles, cudaStrea
             constexpr int K = decltype(k)::value;
             FqItemBlock<K> blk;
             fill_item_block(blk, items_host, count, total_tiles);
-            auto kern = fake_quant_batched_kernel<T, F, BLOCK, MODE, kU, kR<T>, kThreads, K>;
+            auto kern = fake_quant_batched_kernel<T, F, BLOCK, MODE, kU, kR, kThreads, K>;
             return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
         });
     }
@@ -53,11 +50,7 @@ int by_mode(int mode, int block, const FqDeviceItem* items_host, int count, size
 
 }  // namespace
 
-size_t fq_batched_tiles(size_t nunits, int dtype)
-{
-    const size_t per_cta = (size_t)kThreads * kU * (dtype == MXQ_F32 ? kR<F32> : kR<BF16>);
-    return (nunits + per_cta - 1) / per_cta;
-}
+size_t fq_batched_tiles(size_t nunits) { return (nunits + kThreads * kU * kR - 1) / (kThreads * kU * kR); }
 
 int launch_fake_quant_batched(const FqDeviceItem* items_host, int count, size_t total_tiles, int dtype, int fmt,
                               int block, int mode, cudaStream_t stream)

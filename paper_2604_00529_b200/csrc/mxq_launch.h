@@ -69,7 +69,7 @@ struct FqDeviceItem;
 constexpr int kFqBatchItemsMax = 512;
 int launch_fake_quant_batched(const FqDeviceItem* items_host, int count, size_t total_tiles, int dtype, int fmt,
                               int block, int mode, cudaStream_t stream);
-size_t fq_batched_tiles(size_t nunits, int dtype);
+size_t fq_batched_tiles(size_t nunits);
 int launch_copy(const void* src, size_t nbytes, void* dst, cudaStream_t stream);
 // Q_f and the reconstruction over up to 512 tensors in one launch; `items_host` is a HOST array whose
 // tile_begin fields are filled in (tiles counted by q_batched_tiles / dq_batched_tiles of each tensor's
