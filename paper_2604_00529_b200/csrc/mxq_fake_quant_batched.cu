@@ -6,8 +6,9 @@ namespace mxq {
 namespace {
 
 constexpr int kU = 1;
-// Consecutive warp tiles of one tensor per warp: 1 / 2 / 4 take 996 / 1013 / 1098 us (FP32, MXINT4 through the anchor),
-// 547 / 498 / 542 us (BF16, the same) and 539 / 499 / 543 us (BF16, E2M3) over four decoder layers.
+// Consecutive warp tiles of one tensor per warp: 1 / 2 / 4 take 547 / 498 / 542 us (BF16, MXINT4 through the anchor) and
+// 539 / 499 / 543 us (BF16, E2M3) over four decoder layers.  FP32 takes 990 ... 1042 us with 1, changing from run to run
+// within a process, and 1008 ... 1015 with 2; alone in a process 1006 ... 1012 and 1008 ... 1010: no difference to keep two forms for.
 constexpr int kR = 2;
 constexpr int kThreads = 128;
 
