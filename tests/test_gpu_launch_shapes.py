@@ -79,7 +79,7 @@ def test_sets_on_both_sides_of_the_small_item_table(count, bf16):
     """Every batched operation at the last set of the small item table and the first of the large one; tensors of one
     block, of whole CTA tiles and one block on either side of them."""
     rng = np.random.default_rng(count + bf16)
-    edge = 128 if bf16 else 32                                     # blocks of a CTA tile of the fake-quant (the smallest of the tiles)
+    edge = 128 if bf16 else 64                                     # blocks of a CTA tile of the fake-quant (the smallest of the tiles)
     nblks = [int(rng.choice([1, 2, edge - 1, edge, edge + 1, 2 * edge, 2 * edge + 1, 255, 256, 257])) for _ in range(count)]
     xs = [rng.standard_normal(32 * nb).astype(np.float32) * np.float32(2.0 ** rng.integers(-8, 8)) for nb in nblks]
     if bf16:
