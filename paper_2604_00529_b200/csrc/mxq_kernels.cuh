@@ -96,7 +96,7 @@ __device__ __forceinline__ void put_scale(const TiledScales& t, size_t blk, uint
 // their own behind the grid's last data CTA, kPadPerThread pieces per thread: the 4-byte pieces of the rows below
 // the matrix, then the rest of the last piece of every row whose block-columns do not fill it.  (A memset of the
 // whole buffer in front of the kernel cost a launch and, having no programmatic launch, the overlap with the
-// kernel before it: a call on a 1000 x 4096 BF16 matrix, to E4M3, 13.0 us then and 10.4 now.)
+// kernel before it: a call on a 1000 x 4096 BF16 matrix, to E4M3, 13.0 us with it and 10.4 without, through the same binding.)
 constexpr int kPadPerThread = 4;
 
 __host__ __device__ __forceinline__ size_t tiled_pad_pieces(const TiledScales& t)
@@ -1257,6 +1257,8 @@ struct SsItemBlock {
     TileIndex index;
 };
 
+// (Compiled for 12 resident CTAs: without the bound MXINT8 -> MXINT5 of four decoder layers takes 261 us instead of 223, the
+// other targets between 2.6 % less and 2 % more.)
 template <class FH, class FL, int U, int THREADS, int K>
 __global__ void __launch_bounds__(THREADS, 12)
 slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
