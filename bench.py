@@ -4,7 +4,7 @@
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl mxq|reference] [--workloads w1,w2,w3,w4,w5] [--record FILE]
 
 One invocation times all five workloads of the method and prints ONE JSON line on stdout: the headline with its
-configuration, clocks, roofline and baselines.  The whole record (`kernels`, `workloads` and every note) is some 20 KB and
+configuration, clocks, roofline and baselines.  The whole record (`kernels`, `workloads` and every note) is some 55 KB and
 goes to --record FILE, or to stderr: whoever reads the line from the tail of a log gets it whole.
 
 Headline (`value`, `config.workload`): the whole-model workload -- the 224 BF16 linear weights of an 8B
