@@ -4,8 +4,9 @@
 //
 // Every function returns None -- having enqueued nothing -- for anything else: other types and devices, tensor
 // subclasses, tensors without storage (vmap, grad and functionalization wrappers), active torch modes, a stream
-// argument, a status other than MXQ_OK.  The caller in binding.py then takes its general path, which handles the
-// case or raises the error it always raised.
+// argument, a status other than MXQ_OK (a failed launch of slice_scale_multi, which may follow others, is raised at
+// once).  The caller in binding.py then takes its general path, which handles the case or raises the error it
+// always raised.
 #include <Python.h>
 
 #include <ATen/ATen.h>
