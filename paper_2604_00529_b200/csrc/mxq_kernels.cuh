@@ -210,6 +210,81 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v)
 }
 
 // ------------------------------------------------------------------------------------------
+// MXINT rounding on the FP16 pipe
+// ------------------------------------------------------------------------------------------
+// FP16 subnormals are the integers 0 ... 1023 times 2^-24, their bit patterns those integers.  A fused multiply-add whose
+// result lies there therefore rounds to an integer, two elements per instruction, on the FMA pipe; the
+// integer/logic pipe, which bounds these kernels, is left for packing.
+
+__device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+__device__ __forceinline__ uint32_t hfma2_relu(uint32_t a, uint32_t b, uint32_t c)      // negative results become +0
+{
+    uint32_t d;
+    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
+__host__ __device__ constexpr uint32_t both_halves(uint32_t h) { return h | h << 16; }
+
+// m * 2^e as an FP16 bit pattern; exact for integers m of up to 11 significant bits in FP16's range.
+__host__ __device__ constexpr uint32_t half_bits(int m, int e)
+{
+    const uint32_t sign = m < 0 ? 0x8000u : 0u;
+    uint32_t f = (uint32_t)(m < 0 ? -m : m);
+    for (; f >= 2048u; f >>= 1) ++e;
+    for (; f < 1024u && e > -24; f <<= 1) --e;
+    for (; e < -24; f >>= 1) ++e;
+    return sign | (f < 1024u ? f : (f - 1024u) | (uint32_t)(e + 25) << 10);
+}
+
+// The MXINT codes (Eq. 3, Eq. 4) of two values r, given as the FP16 pair p = r 2^-E with |r| <= 128, each XORed with
+// M = 2^(B-1) - 1.  The first multiply-add rounds M + r (1 + 2^-10) to an integer; the factor turns ties away from zero and
+// is too small to carry any other value of eight significant bits (|r| 2^-10 is below their spacing) over a halfway point.
+// Negative sums (r below -M) become 0 = the symmetric clip; the second one is the same clip of the other side:
+// 2M - (M + q) = M - q, and (M - q) ^ M is the two's complement of q in B bits.
+template <int B, int E>
+__device__ __forceinline__ uint32_t round_halves(uint32_t p)
+{
+    constexpr uint32_t M = (1u << (B - 1)) - 1u;
+    constexpr uint32_t c = half_bits(1025, E - 34);                // 2^(E - 24) (1 + 2^-10)
+    const uint32_t r = hfma2_relu(p, both_halves(c), both_halves(M));
+    return hfma2_relu(r, both_halves(half_bits(-1, 0)), both_halves(2 * M));
+}
+
+// Word number `word` of the bitstream that repeats one B-bit code.
+template <int B>
+__host__ __device__ constexpr uint32_t code_pattern(uint32_t code, int word)
+{
+    uint32_t v = 0;
+    for (int i = 0; i < 32; ++i) v |= (code >> ((32 * word + i) % B) & 1u) << i;
+    return v;
+}
+
+// XORs every B-bit code of the bitstream with M = 2^(B-1) - 1 (see round_halves).
+template <int B, int NW>
+__device__ __forceinline__ void unbias_codes(uint32_t (&out)[NW])
+{
+    static_for<NW>([&](auto j) {
+        constexpr uint32_t pattern = code_pattern<B>((1u << (B - 1)) - 1u, decltype(j)::value);
+        out[decltype(j)::value] ^= pattern;
+    });
+}
+
+// Two 2B-bit fields in the low bits of the halves of y -> their 4B-bit stream in the top bits (the rest clear).
+template <int B>
+__device__ __forceinline__ uint32_t join_halves_top(uint32_t y)
+{
+    constexpr uint32_t k = 1u << (16 - 2 * B);
+    return (y & 0xFFFFu) * (k * (k - 1u)) + y * k;
+}
+
+// ------------------------------------------------------------------------------------------
 // Q_f: quantize (Eq. 1-3)
 // ------------------------------------------------------------------------------------------
 
@@ -720,48 +795,24 @@ quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk)
 // Q_{h->l}: Slice-and-Scale (Eq. 4-5).  One lane = 32 codes.
 // ------------------------------------------------------------------------------------------
 
-// Eq. 4 on four MXINT8 codes at once (one per byte): returns the four low-format codes, one per
-// byte, in the TOP BL bits of the byte (the bits below are clear).  Sign-magnitude SWAR; no carry
-// crosses a byte until the last step, whose stray carry lands in a bit that is masked off.
-//   full : 0xFF in the bytes that are negative (byte permute with sign replication)
-//   a    : |p| - s per byte, s the 0/1 sign (one's complement of the negative bytes)
-//   T    : |p| + 2^(de-1) <= 128 + 2^(de-1); the shifted value q = T >> de sits in T's top BL bits.
-//          q reaches 2^(BL-1) exactly when T >= 128, and then those top bits read 100..0: flipping
-//          them (xor with the replicated top bit of T) gives 011..1, the clipped magnitude.
-//   two's complement of the negative bytes: flip the BL bits, add one at bit de.  The add can carry
-//   out of a byte only for q = 0 (the bits are all ones), into bit 0 of the next byte, which is
-//   cleared before (so that it cannot travel) and after.
-// The integer/logic pipe is the scarce resource here, so the per-byte 0/1 sign comes from the
-// 0xFF/0x00 mask by a multiply-add with 255^-1 (mod 2^32), which runs on the multiply pipe:
-// mask = 255 * sum(s_i 256^i), hence mask * 255^-1 = sum(s_i 256^i) exactly.
-// (Checked against the scalar definition for all 2^32 input words on the host.)
-struct Int8Word {
-    uint32_t full, mag;      // 0xFF in the negative bytes; |p| per byte
+// Four MXINT8 codes (one word) as FP16 pairs, the codes 0 and 2 in .a, 1 and 3 in .b: code p is p 2^-17.  The biased code
+// u = p + 128 under the exponent of 1024 is the FP16 number 1024 + u; one multiply-add takes the bias off.
+struct IntHalves {
+    uint32_t a, b;
 };
 
-// What every target needs of four codes (|p| = a + s: one multiply-add; 0x80 reads 128).
-__device__ __forceinline__ Int8Word int8_word(uint32_t x)
+template <class FH, int J, int NW>
+__device__ __forceinline__ IntHalves int_halves(const uint32_t (&in)[NW])
 {
-    constexpr uint32_t kInv255 = 0xFEFEFEFFu;
-    Int8Word w;
-    asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(w.full) : "r"(x));         // selector bit 3: replicate the byte's sign
-    w.mag = w.full * kInv255 + (x ^ w.full);
-    return w;
-}
-
-template <int BL>
-__device__ __forceinline__ uint32_t ss_int8_word_top(const Int8Word& w)
-{
-    constexpr int de = 8 - BL;
-    constexpr uint32_t k01 = 0x01010101u;
-    constexpr uint32_t kInv255 = 0xFEFEFEFFu;
-    constexpr uint32_t kH = k01 * (1u << (de - 1));            // rounding increment
-    constexpr uint32_t kTop = k01 * ((0xFFu << de) & 0xFFu);   // the top BL bits of every byte
-    const uint32_t t = w.mag + kH;
-    uint32_t ov;
-    asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(ov) : "r"(t));   // 0xFF where the magnitude clips
-    const uint32_t m = (t ^ ov ^ w.full) & kTop;
-    return (w.full * (kInv255 << de) + m) & kTop;
+    constexpr int B = FH::bits;
+    static_assert(B == 8, "MXINT8");
+    constexpr uint32_t one = both_halves(half_bits(1, -9 - B));
+    constexpr uint32_t bias = both_halves(half_bits(-(1024 + (1 << (B - 1))), -9 - B));
+    IntHalves h;
+    const uint32_t u = in[J] ^ 0x80808080u;
+    h.a = hfma2(__byte_perm(u, 0x64646464u, 0x4240), one, bias);
+    h.b = hfma2(__byte_perm(u, 0x64646464u, 0x4341), one, bias);
+    return h;
 }
 
 __device__ __forceinline__ bool has_e4m3_nan(uint32_t x)
@@ -885,19 +936,19 @@ __device__ __forceinline__ uint32_t e4m3_word_clean(uint32_t x, uint32_t& nans)
     return x - (m >> 7);
 }
 
-// Eight anchor codes (words 2J and 2J + 1 of a lane's 32) in a lower format: two streams for pack_streams, or,
-// for the 4-bit formats, one finished output word.
+// Eight codes (the quads 2J and 2J + 1 of a lane's 32) in a lower format: two streams for pack_streams, or,
+// for the 4-bit formats, one finished output word.  MXINT codes stay XORed with M until ss_finish.
 template <class FL, int J>
-__device__ __forceinline__ void ss_int8_word_pair(const Int8Word& w0, const Int8Word& w1, uint32_t (&z)[8])
+__device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntHalves& w1, uint32_t (&z)[8])
 {
-    if constexpr (FL::bits == 4) {
-        // the codes come back in the high nibbles: w * 17 drops each one into the low nibble of the
-        // byte above as well, so bytes 1 and 3 of it hold c0 | c1 << 4 and c2 | c3 << 4
-        const uint32_t a = ss_int8_word_top<4>(w0), b = ss_int8_word_top<4>(w1);
-        z[J] = __byte_perm(a * 16u + a, b * 16u + b, 0x7531);
+    constexpr int B = FL::bits, E = 9 + B;                     // r = p / 2^(8-B)
+    const uint32_t y0 = round_halves<B, E>(w0.b) * (1u << B) + round_halves<B, E>(w0.a);
+    const uint32_t y1 = round_halves<B, E>(w1.b) * (1u << B) + round_halves<B, E>(w1.a);
+    if constexpr (B == 4) {
+        z[J] = __byte_perm(y0, y1, 0x6420);
     } else {
-        z[2 * J] = squeeze_top<FL::bits>(ss_int8_word_top<FL::bits>(w0));
-        z[2 * J + 1] = squeeze_top<FL::bits>(ss_int8_word_top<FL::bits>(w1));
+        z[2 * J] = join_halves_top<B>(y0);
+        z[2 * J + 1] = join_halves_top<B>(y1);
     }
 }
 
@@ -921,6 +972,7 @@ __device__ __forceinline__ void ss_finish(const uint32_t (&z)[8], uint32_t (&out
     } else {
         pack_streams<FL::bits>(z, out);
     }
+    if constexpr (FL::kind == KIND_INT) unbias_codes<FL::bits>(out);
 }
 
 template <int I, class... FL>
@@ -938,10 +990,10 @@ __device__ __forceinline__ void ss_anchor_unit(const uint32_t (&in)[8], uint32_t
     static_for<4>([&](auto jj) {
         constexpr int J = decltype(jj)::value;
         if constexpr (FH::kind == KIND_INT) {
-            const Int8Word w0 = int8_word(in[2 * J]), w1 = int8_word(in[2 * J + 1]);
+            const IntHalves w0 = int_halves<FH, 2 * J>(in), w1 = int_halves<FH, 2 * J + 1>(in);
             static_for<(int)sizeof...(FL)>([&](auto i) {
                 constexpr int I = decltype(i)::value;
-                ss_int8_word_pair<ss_target_t<I, FL...>, J>(w0, w1, z[I]);
+                ss_int_quad_pair<ss_target_t<I, FL...>, J>(w0, w1, z[I]);
             });
         } else {
             uint32_t h[4], nans[2] = {0, 0};
