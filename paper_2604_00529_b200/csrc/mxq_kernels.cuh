@@ -795,8 +795,27 @@ quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk)
 // Q_{h->l}: Slice-and-Scale (Eq. 4-5).  One lane = 32 codes.
 // ------------------------------------------------------------------------------------------
 
-// Four MXINT8 codes (one word) as FP16 pairs, the codes 0 and 2 in .a, 1 and 3 in .b: code p is p 2^-17.  The biased code
-// u = p + 128 under the exponent of 1024 is the FP16 number 1024 + u; one multiply-add takes the bias off.
+// Four consecutive codes, number J, of a little-endian bitstream of B-bit codes (B < 8), in 16-bit lanes: c0 | c1 << B in the
+// lower half, c2 | c3 << B in the upper one; the bits above 2B of the upper half are undefined.
+template <int B, int J, int NW>
+__device__ __forceinline__ uint32_t code_quad_lanes(const uint32_t (&in)[NW])
+{
+    constexpr int off = 4 * B * J, wi = off >> 5, sh = off & 31;
+    if constexpr (B == 4) {
+        return __byte_perm(in[wi], 0, sh == 0 ? 0x4140 : 0x4342);
+    } else {
+        uint32_t f;
+        if constexpr (sh == 0) f = in[wi];
+        else if constexpr (sh + 4 * B <= 32) f = in[wi] >> sh;
+        else f = __funnelshift_r(in[wi], in[wi + 1], sh);
+        constexpr uint32_t k = 1u << (16 - 2 * B);
+        return f * k - (f & ((1u << (2 * B)) - 1u)) * (k - 1u);
+    }
+}
+
+// Four MXINT codes, number J of the lane's 32, as FP16 pairs, the codes 0 and 2 in .a, 1 and 3 in .b: the value of code p
+// is p 2^(8-b_h) 2^-17, the same for every source width, so that de = b_h - b_l becomes 8 - b_l below.  The
+// biased code u = p + 2^(b_h - 1) under the exponent of 1024 is the FP16 number 1024 + u; one multiply-add takes the bias off.
 struct IntHalves {
     uint32_t a, b;
 };
@@ -805,13 +824,19 @@ template <class FH, int J, int NW>
 __device__ __forceinline__ IntHalves int_halves(const uint32_t (&in)[NW])
 {
     constexpr int B = FH::bits;
-    static_assert(B == 8, "MXINT8");
     constexpr uint32_t one = both_halves(half_bits(1, -9 - B));
     constexpr uint32_t bias = both_halves(half_bits(-(1024 + (1 << (B - 1))), -9 - B));
     IntHalves h;
-    const uint32_t u = in[J] ^ 0x80808080u;
-    h.a = hfma2(__byte_perm(u, 0x64646464u, 0x4240), one, bias);
-    h.b = hfma2(__byte_perm(u, 0x64646464u, 0x4341), one, bias);
+    if constexpr (B == 8) {
+        const uint32_t u = in[J] ^ 0x80808080u;
+        h.a = hfma2(__byte_perm(u, 0x64646464u, 0x4240), one, bias);
+        h.b = hfma2(__byte_perm(u, 0x64646464u, 0x4341), one, bias);
+    } else {
+        constexpr uint32_t m = both_halves(FH::mask), k = both_halves(0x6400u + (1u << (B - 1)));
+        const uint32_t y = code_quad_lanes<B, J>(in);
+        h.a = hfma2((y & m) ^ k, one, bias);
+        h.b = hfma2(((y >> B) & m) ^ k, one, bias);
+    }
     return h;
 }
 
@@ -832,9 +857,36 @@ __device__ __forceinline__ void e4m3_word_to_f16(uint32_t w, uint32_t& a, uint32
         : "=r"(a), "=r"(b) : "r"(w));
 }
 
+// Four codes, number J of the lane's 32, of an MXFP format below eight bits as two FP16 pairs: one code per byte,
+// then the widening conversion.  E3M3 and E2M2 have none; with the sign bit one position up their codes are codes of E4M3 and E3M2
+// (same mantissa, see SoftFp) that stand for 2^-fp_source_shift() times the value.
+template <class FH>
+__host__ __device__ constexpr int fp_source_shift()
+{
+    return FH::id == MXQ_FP7_E3M3 ? 4 : FH::id == MXQ_FP5_E2M2 ? 2 : 0;
+}
+
+template <class FH, int J, int NW>
+__device__ __forceinline__ void fp_quad_to_f16(const uint32_t (&in)[NW], uint32_t& a, uint32_t& b)
+{
+    constexpr int B = FH::bits;
+    static_assert(FH::kind == KIND_FP && B < 8 && B > 4);
+    const uint32_t y = code_quad_lanes<B, J>(in);
+    uint32_t w = (y & both_halves(FH::mask << B)) * (1u << (8 - B)) + (y & both_halves(FH::mask));
+    if constexpr (!FH::hw_cvt) w += w & (0x01010101u << (B - 1));
+    if constexpr (FH::id == MXQ_FP7_E3M3)
+        e4m3_word_to_f16(w, a, b);
+    else if constexpr (FH::id == MXQ_FP6_E2M3)
+        asm("{ .reg .b16 l, h; mov.b32 {l, h}, %2; cvt.rn.f16x2.e2m3x2 %0, l; cvt.rn.f16x2.e2m3x2 %1, h; }"
+            : "=r"(a), "=r"(b) : "r"(w));
+    else
+        asm("{ .reg .b16 l, h; mov.b32 {l, h}, %2; cvt.rn.f16x2.e3m2x2 %0, l; cvt.rn.f16x2.e3m2x2 %1, h; }"
+            : "=r"(a), "=r"(b) : "r"(w));
+}
+
 // two FP16 pairs (four E4M3 codes of one word), already divided by 2^de, as four FP32 values
 template <int DE>
-__device__ __forceinline__ void e4m3_pairs_scaled(uint32_t a, uint32_t b, float (&f)[4])
+__device__ __forceinline__ void fp_pairs_scaled(uint32_t a, uint32_t b, float (&f)[4])
 {
     constexpr uint32_t kHalf = (uint32_t)(15 - DE) << 10;      // 2^-de as FP16
     asm("{ .reg .b16 l, h; .reg .b32 a, b;\n"
@@ -855,14 +907,19 @@ __device__ __forceinline__ void e4m3_pairs_scaled(uint32_t a, uint32_t b, float 
 //               value rounds to zero either way (anchor codes have four significant bits).
 // Nothing is clipped: the largest anchor value 448 / 2^de (7, 28, 28, 7) does not exceed the target's largest
 // (7.5, 28, 30, 7).
-template <class FL>
-__device__ __forceinline__ uint32_t ss_e4m3_pairs_top(uint32_t a, uint32_t b, uint32_t nans)
+template <class FH, class FL>
+__device__ __forceinline__ uint32_t ss_fp_pairs_top(uint32_t a, uint32_t b, uint32_t nans)
 {
-    constexpr int de = 8 - FL::emax, D = 8 - FL::bits;
+    constexpr int de = FH::emax - FL::emax - fp_source_shift<FH>(), D = 8 - FL::bits;
     constexpr uint32_t k01 = 0x01010101u;
     constexpr uint32_t kMag = k01 * FL::max_mag;
     uint32_t c;
-    if constexpr (FL::id == MXQ_FP5_E2M2) {
+    if constexpr (FL::id == MXQ_FP5_E2M2 && FH::id != MXQ_FP8_E4M3) {
+        // E3M3 and E2M3 go up to 7.5 2^de, which rounds beyond the target's largest: the quantizer's conversion clips it
+        float f[4];
+        fp_pairs_scaled<de + SoftFp<FL>::k>(a, b, f);
+        return quantize_fp_soft_quad<FL>(f[0], f[1], f[2], f[3]) << D;
+    } else if constexpr (FL::id == MXQ_FP5_E2M2) {
         constexpr uint32_t kHalf = 1u << (24 - (de + 14));           // 2^-20 as an FP16 subnormal
         asm("{ .reg .b16 l, h; .reg .b32 a, b; mul.rn.f16x2 a, %1, %3; mul.rn.f16x2 b, %2, %3;\n"
             "  cvt.rn.satfinite.e5m2x2.f16x2 l, a; cvt.rn.satfinite.e5m2x2.f16x2 h, b; mov.b32 %0, {l, h}; }"
@@ -871,7 +928,7 @@ __device__ __forceinline__ uint32_t ss_e4m3_pairs_top(uint32_t a, uint32_t b, ui
     } else {
         constexpr int k = FL::id == MXQ_FP7_E3M3 ? 4 : 0;
         float f[4];
-        e4m3_pairs_scaled<de + k>(a, b, f);
+        fp_pairs_scaled<de + k>(a, b, f);
         if constexpr (FL::id == MXQ_FP7_E3M3)
             asm("{ .reg .b16 l, h; cvt.rn.satfinite.e4m3x2.f32 l, %2, %1; cvt.rn.satfinite.e4m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
                 : "=r"(c) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
@@ -888,11 +945,13 @@ __device__ __forceinline__ uint32_t ss_e4m3_pairs_top(uint32_t a, uint32_t b, ui
 }
 
 // eight E4M3 codes (two words, given as their four FP16 pairs) -> eight E2M1 codes in one word
-__device__ __forceinline__ uint32_t ss_e4m3_pairs_to_e2m1(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1)
+template <class FH>
+__device__ __forceinline__ uint32_t ss_fp_pairs_to_e2m1(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1)
 {
+    constexpr int de = FH::emax - 2 - fp_source_shift<FH>();
     float f[4], g[4];
-    e4m3_pairs_scaled<6>(a0, b0, f);
-    e4m3_pairs_scaled<6>(a1, b1, g);
+    fp_pairs_scaled<de>(a0, b0, f);
+    fp_pairs_scaled<de>(a1, b1, g);
     uint32_t d;
     asm("{ .reg .b8 a, b, c, e;\n"
         "  cvt.rn.satfinite.e2m1x2.f32 a, %2, %1;  cvt.rn.satfinite.e2m1x2.f32 b, %4, %3;\n"
@@ -902,8 +961,7 @@ __device__ __forceinline__ uint32_t ss_e4m3_pairs_to_e2m1(uint32_t a0, uint32_t 
     return d;
 }
 
-// Every legal pair, one element at a time (exact, slow): for sources that are not an 8-bit anchor and for units
-// with E4M3 NaN codes.
+// Every legal pair, one element at a time (exact, slow): for units with E4M3 NaN codes.
 template <class FH, class FL, int NWI, int NWO>
 __device__ __forceinline__ void ss_unit_by_element(const uint32_t (&in)[NWI], uint32_t (&out)[NWO])
 {
@@ -941,7 +999,7 @@ __device__ __forceinline__ uint32_t e4m3_word_clean(uint32_t x, uint32_t& nans)
 template <class FL, int J>
 __device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntHalves& w1, uint32_t (&z)[8])
 {
-    constexpr int B = FL::bits, E = 9 + B;                     // r = p / 2^(8-B)
+    constexpr int B = FL::bits, E = 9 + B;                     // r = p 2^(8-b_h) / 2^(8-B)
     const uint32_t y0 = round_halves<B, E>(w0.b) * (1u << B) + round_halves<B, E>(w0.a);
     const uint32_t y1 = round_halves<B, E>(w1.b) * (1u << B) + round_halves<B, E>(w1.a);
     if constexpr (B == 4) {
@@ -952,14 +1010,14 @@ __device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntH
     }
 }
 
-template <class FL, int J>
-__device__ __forceinline__ void ss_e4m3_word_pair(const uint32_t (&h)[4], const uint32_t (&nans)[2], uint32_t (&z)[8])
+template <class FH, class FL, int J>
+__device__ __forceinline__ void ss_fp_quad_pair(const uint32_t (&h)[4], const uint32_t (&nans)[2], uint32_t (&z)[8])
 {
     if constexpr (FL::bits == 4) {
-        z[J] = ss_e4m3_pairs_to_e2m1(h[0], h[1], h[2], h[3]);
+        z[J] = ss_fp_pairs_to_e2m1<FH>(h[0], h[1], h[2], h[3]);
     } else {
-        z[2 * J] = squeeze_top<FL::bits>(ss_e4m3_pairs_top<FL>(h[0], h[1], nans[0]));
-        z[2 * J + 1] = squeeze_top<FL::bits>(ss_e4m3_pairs_top<FL>(h[2], h[3], nans[1]));
+        z[2 * J] = squeeze_top<FL::bits>(ss_fp_pairs_top<FH, FL>(h[0], h[1], nans[0]));
+        z[2 * J + 1] = squeeze_top<FL::bits>(ss_fp_pairs_top<FH, FL>(h[2], h[3], nans[1]));
     }
 }
 
@@ -978,14 +1036,14 @@ __device__ __forceinline__ void ss_finish(const uint32_t (&z)[8], uint32_t (&out
 template <int I, class... FL>
 using ss_target_t = typename std::tuple_element<I, std::tuple<FL...>>::type;
 
-// The 32 codes of one lane of an 8-bit anchor to one or more lower formats, eight codes at a time so that what
+// The 32 codes of one lane to one or more lower formats, eight codes at a time so that what
 // the targets share (sign masks and magnitudes, FP16 values) lives only that long.  E4M3 anchors:
 // NAN_CODES = false promises that none of the codes is a NaN code.  A NaN code maps to the largest magnitude with
 // its sign: so does the largest finite code, 448, wherever the target's largest mantissa is 1.75 or less
 // (448 / 2^de = 1.75 * 2^emax); for the three-bit mantissas (largest 1.875) the magnitude bits of the target
 // code are set as well.
-template <bool NAN_CODES, class FH, class... FL>
-__device__ __forceinline__ void ss_anchor_unit(const uint32_t (&in)[8], uint32_t (&z)[sizeof...(FL)][8])
+template <bool NAN_CODES, class FH, class... FL, int NW>
+__device__ __forceinline__ void ss_unit(const uint32_t (&in)[NW], uint32_t (&z)[sizeof...(FL)][8])
 {
     static_for<4>([&](auto jj) {
         constexpr int J = decltype(jj)::value;
@@ -997,11 +1055,16 @@ __device__ __forceinline__ void ss_anchor_unit(const uint32_t (&in)[8], uint32_t
             });
         } else {
             uint32_t h[4], nans[2] = {0, 0};
-            e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J], nans[0]) : in[2 * J], h[0], h[1]);
-            e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J + 1], nans[1]) : in[2 * J + 1], h[2], h[3]);
+            if constexpr (FH::bits == 8) {
+                e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J], nans[0]) : in[2 * J], h[0], h[1]);
+                e4m3_word_to_f16(NAN_CODES ? e4m3_word_clean(in[2 * J + 1], nans[1]) : in[2 * J + 1], h[2], h[3]);
+            } else {
+                fp_quad_to_f16<FH, 2 * J>(in, h[0], h[1]);
+                fp_quad_to_f16<FH, 2 * J + 1>(in, h[2], h[3]);
+            }
             static_for<(int)sizeof...(FL)>([&](auto i) {
                 constexpr int I = decltype(i)::value;
-                ss_e4m3_word_pair<ss_target_t<I, FL...>, J>(h, nans, z[I]);
+                ss_fp_quad_pair<FH, ss_target_t<I, FL...>, J>(h, nans, z[I]);
             });
         }
     });
@@ -1014,21 +1077,19 @@ __device__ __forceinline__ void slice_scale_unit(const uint32_t (&in)[NWI], uint
     if constexpr (FH::id == FL::id) {
 #pragma unroll
         for (int j = 0; j < NWO; ++j) out[j] = in[j];
-    } else if constexpr (FH::bits == 8) {
+    } else {
         uint32_t z[1][8];
-        if constexpr (FH::kind == KIND_INT) {
-            ss_anchor_unit<false, FH, FL>(in, z);
+        if constexpr (!FH::has_nan) {
+            ss_unit<false, FH, FL>(in, z);
             ss_finish<FL>(z[0], out);
         } else if (!unit_has_e4m3_nan(in)) {
-            ss_anchor_unit<false, FH, FL>(in, z);
+            ss_unit<false, FH, FL>(in, z);
             ss_finish<FL>(z[0], out);
         } else {
             // an E4M3 NaN code (never produced by the quantizer): the slow path, which costs this kernel nothing
-            // where ss_anchor_unit<true> slows the 6-bit targets by 1.5 %
+            // where ss_unit<true> slows the 6-bit targets by 1.5 %
             ss_unit_by_element<FH, FL>(in, out);
         }
-    } else {
-        ss_unit_by_element<FH, FL>(in, out);          // every other pair, including non-anchor sources
     }
 }
 
@@ -1191,8 +1252,8 @@ __device__ __forceinline__ void slice_scale_set_tile(const uint8_t* __restrict__
         }
         uint32_t z[N][8];
         // one NaN-code check, all conversions in one straight line
-        if (FH::kind == KIND_INT || !unit_has_e4m3_nan(w[u])) ss_anchor_unit<false, FH, FL...>(w[u], z);
-        else if constexpr (FH::kind == KIND_FP) ss_anchor_unit<true, FH, FL...>(w[u], z);
+        if (FH::kind == KIND_INT || !unit_has_e4m3_nan(w[u])) ss_unit<false, FH, FL...>(w[u], z);
+        else if constexpr (FH::kind == KIND_FP) ss_unit<true, FH, FL...>(w[u], z);
         static_for<N>([&](auto i) {
             constexpr int I = decltype(i)::value;
             using F = ss_target_t<I, FL...>;
