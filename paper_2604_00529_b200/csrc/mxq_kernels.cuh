@@ -230,6 +230,13 @@ __device__ __forceinline__ uint32_t hfma2_relu(uint32_t a, uint32_t b, uint32_t 
     return d;
 }
 
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
 __host__ __device__ constexpr uint32_t both_halves(uint32_t h) { return h | h << 16; }
 
 // m * 2^e as an FP16 bit pattern; exact for integers m of up to 11 significant bits in FP16's range.
@@ -337,6 +344,47 @@ __device__ __forceinline__ void pack_streams(const uint32_t (&z)[NZ], uint32_t (
             if constexpr (sh + W > 32) out[wi + 1] = z[J] >> (64 - W - sh);
         });
     }
+}
+
+// Codes of a BF16 lane unit in an MXINT format, inv = 2^-shared_exp, two elements per instruction: r = v inv, exact in BF16
+// wherever it does not round to 0 anyway; r 2^-122, whose BF16 exponent field fits FP16's five bits, so that the
+// pattern moved up by three bits under its sign is the FP16 number r 2^-10 (what is lost below BF16's smallest normal is below
+// r = 2^-4).
+template <class F, int NW>
+__device__ __forceinline__ void quantize_unit_bf16_int(const uint32_t (&w)[8], float inv, uint32_t (&out)[NW])
+{
+    constexpr int B = F::bits;
+    const uint32_t inv2 = __byte_perm(__float_as_uint(inv), 0, 0x3232);
+    constexpr uint32_t k122 = both_halves((127u - 122u) << 7);
+    uint32_t z[4];
+    static_for<4>([&](auto qi) {
+        constexpr int Q = decltype(qi)::value;
+        uint32_t r[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t x = mul_bf16x2(mul_bf16x2(w[2 * Q + i], inv2), k122);
+            r[i] = round_halves<B, 10>(((x & 0x7FFF7FFFu) * 8u) | (x & 0x80008000u));
+        }
+        if constexpr (B == 8) {
+            z[Q] = __byte_perm(r[0], r[1], 0x6420);
+        } else {
+            // c0 | c1 << B of each pair lands in the upper half
+            constexpr uint32_t j = 0x10000u + (1u << B);
+            const uint32_t y = __byte_perm(r[0] * j, r[1] * j, 0x7632);
+            if constexpr (B == 4) z[Q] = y;
+            else z[Q] = join_halves_top<B>(y);
+        }
+    });
+    if constexpr (B == 8) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) out[i] = z[i];
+    } else if constexpr (B == 4) {
+        out[0] = __byte_perm(z[0], z[1], 0x6420);
+        out[1] = __byte_perm(z[2], z[3], 0x6420);
+    } else {
+        pack_streams<B>(z, out);
+    }
+    unbias_codes<B>(out);
 }
 
 // MXINT codes of four consecutive elements (Eq. 3), one per byte in the low F::bits bits.
@@ -467,7 +515,8 @@ __device__ __forceinline__ void quantize_tile(const uint8_t* __restrict__ src, s
         const uint32_t amax = group_max<LPB>(unit_amax_bits<T>(w[u]));
         const BlockScale s = block_scale<F>(amax);
         uint32_t out[NW];
-        quantize_unit<T, F>(w[u], s.inv, out);
+        if constexpr (T::size == 2 && F::kind == KIND_INT) quantize_unit_bf16_int<F>(w[u], s.inv, out);
+        else quantize_unit<T, F>(w[u], s.inv, out);
         if (s.byte == 0xFFu) {
 #pragma unroll
             for (int j = 0; j < NW; ++j) out[j] = 0;
