@@ -177,26 +177,39 @@ struct SoftFp {
     static constexpr int k = e3m3 ? 4 : 2;                                // bias_hw - bias_F
     static constexpr float pre_scale = e3m3 ? 0.0625f : 0.25f;            // 2^-k
     static constexpr float post_scale = e3m3 ? 16.0f : 4.0f;              // 2^k
-    static constexpr uint32_t hw_mag_mask = e3m3 ? 0x7Fu : 0x1Fu;
 };
 
-// Codes of four elements given as r / 2^k (r = v / X exact, |r| < 2^(e_max + 1)), one per byte.
+// Four FP32 values in a format with a narrowing instruction, one code per byte (6-bit codes in the low bits).
 template <class F>
-__device__ __forceinline__ uint32_t quantize_fp_soft_quad(float r0, float r1, float r2, float r3)
+__device__ __forceinline__ uint32_t quantize_fp_hw_quad(float r0, float r1, float r2, float r3)
 {
-    using S = SoftFp<F>;
-    constexpr uint32_t k01 = 0x01010101u;
-    uint32_t c;                                                           // four neighbour codes, one per byte
-    if constexpr (S::e3m3)
+    uint32_t c;
+    if constexpr (F::id == MXQ_FP8_E4M3)
         asm("{ .reg .b16 l, h; cvt.rn.satfinite.e4m3x2.f32 l, %2, %1; cvt.rn.satfinite.e4m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
+            : "=r"(c) : "f"(r0), "f"(r1), "f"(r2), "f"(r3));
+    else if constexpr (F::id == MXQ_FP6_E2M3)
+        asm("{ .reg .b16 l, h; cvt.rn.satfinite.e2m3x2.f32 l, %2, %1; cvt.rn.satfinite.e2m3x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
             : "=r"(c) : "f"(r0), "f"(r1), "f"(r2), "f"(r3));
     else
         asm("{ .reg .b16 l, h; cvt.rn.satfinite.e3m2x2.f32 l, %2, %1; cvt.rn.satfinite.e3m2x2.f32 h, %4, %3; mov.b32 %0, {l, h}; }"
             : "=r"(c) : "f"(r0), "f"(r1), "f"(r2), "f"(r3));
-    uint32_t mag = c & (k01 * S::hw_mag_mask);
-    mag -= (mag >> (F::bits - 1)) & k01;                                  // the one code above F's largest
-    // sign: top bit of the neighbour's code -> top bit of F's code (one position down in both cases)
-    return mag | ((c >> 1) & (k01 << (F::bits - 1)));
+    return c;
+}
+
+// Codes of four elements given as r / 2^k (r = v / X exact, |r| < 2^(e_max + 1)), one per byte in its top bits.
+// The neighbour's code has its overflow bit right above F's magnitude: moved to the top of the byte it
+// selects, by a byte permute with sign replication, the complement of the (then zero) magnitude.
+template <class F>
+__device__ __forceinline__ uint32_t quantize_fp_soft_quad_top(float r0, float r1, float r2, float r3)
+{
+    using H = Fmt<SoftFp<F>::hw>;
+    constexpr uint32_t k01 = 0x01010101u;
+    constexpr int up = 8 - F::bits;                                       // overflow bit F::bits - 1 -> bit 7
+    const uint32_t c = quantize_fp_hw_quad<H>(r0, r1, r2, r3);
+    const uint32_t t = c * (1u << up);
+    uint32_t ov;
+    asm("prmt.b32 %0, %1, %1, 0xBA98;" : "=r"(ov) : "r"(t));              // 0xFF in the bytes that overflow
+    return ((t ^ ov) & (k01 * (F::max_mag << up))) | ((c * (1u << (8 - H::bits))) & 0x80808080u);
 }
 
 // Two elements given as r / 2^k -> their two neighbour-format codes (code(r0) | code(r1) << 8), the
@@ -206,29 +219,6 @@ __device__ __forceinline__ uint32_t quantize_fp_soft_pair(float r0, float r1)
 {
     const uint32_t d = quantize_fp_hw_pair<Fmt<SoftFp<F>::hw>>(r0, r1);
     return d - ((d >> (F::bits - 1)) & 0x0101u);
-}
-
-// Quantize two scaled-on-the-fly elements to an MXFP format; returns the two codes in the low `bits`
-// bits of .x and .y.  (MXINT elements are quantized four at a time, see quantize_int_quad.)
-template <class F>
-__device__ __forceinline__ uint2 quantize_pair(float v0, float v1, float inv)
-{
-    static_assert(F::kind == KIND_FP, "MXFP formats only");
-    uint2 c;
-    if constexpr (F::hw_cvt) {
-        uint32_t d = quantize_fp_hw_pair<F>(v0 * inv, v1 * inv);
-        if constexpr (F::bits == 4) {
-            c.x = d & 0xFu;
-            c.y = (d >> 4) & 0xFu;
-        } else {
-            c.x = d & 0xFFu;
-            c.y = (d >> 8) & 0xFFu;
-        }
-    } else {
-        c.x = quantize_fp_alu<F>(v0 * inv);
-        c.y = quantize_fp_alu<F>(v1 * inv);
-    }
-    return c;
 }
 
 // ------------------------------------------------------------------------------------------
