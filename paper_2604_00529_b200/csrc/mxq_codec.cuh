@@ -212,13 +212,13 @@ __device__ __forceinline__ uint32_t quantize_fp_soft_quad_top(float r0, float r1
     return ((t ^ ov) & (k01 * (F::max_mag << up))) | ((c * (1u << (8 - H::bits))) & 0x80808080u);
 }
 
-// Two elements given as r / 2^k -> their two neighbour-format codes (code(r0) | code(r1) << 8), the
-// one code above F's largest clipped back: decoded as neighbour values they are P / 2^k.
+// The neighbour-format codes of four elements given as r / 2^k, one per byte, the one code above F's largest clipped back:
+// decoded as neighbour values they are P / 2^k.
 template <class F>
-__device__ __forceinline__ uint32_t quantize_fp_soft_pair(float r0, float r1)
+__device__ __forceinline__ uint32_t quantize_fp_soft_quad(float r0, float r1, float r2, float r3)
 {
-    const uint32_t d = quantize_fp_hw_pair<Fmt<SoftFp<F>::hw>>(r0, r1);
-    return d - ((d >> (F::bits - 1)) & 0x0101u);
+    const uint32_t c = quantize_fp_hw_quad<Fmt<SoftFp<F>::hw>>(r0, r1, r2, r3);
+    return c - ((c >> (F::bits - 1)) & 0x01010101u);
 }
 
 // ------------------------------------------------------------------------------------------

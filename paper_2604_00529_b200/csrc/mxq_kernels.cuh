@@ -590,6 +590,31 @@ __device__ __forceinline__ float2 widen_hw_pair(uint32_t d)
     return f;
 }
 
+// Two inputs of an MXFP fake-quant divided by the target's X, in FP32 (exact).  E3M3 / E2M2: divided by a further 2^k,
+// which makes them values of their hardware neighbour format (see SoftFp).
+template <class F, int MODE>
+__device__ __forceinline__ void fake_quant_scaled(float v0, float v1, float inv, float& r0, float& r1)
+{
+    using A = Fmt<MXQ_FP8_E4M3>;
+    constexpr bool via = MODE == MXQ_FQ_VIA_ANCHOR && F::id != A::id;
+    constexpr int de = A::emax - F::emax;
+    constexpr int k = [] { if constexpr (F::hw_cvt) return 0; else return SoftFp<F>::k; }();
+    if constexpr (via) {
+        // anchor codes -> exact FP16 values -> divide by 2^(de + k) (exact) -> FP32
+        uint32_t a = quantize_fp_hw_pair<A>(v0 * inv, v1 * inv);
+        uint32_t h2;
+        asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)a));
+        constexpr uint32_t kHalf = (uint32_t)(15 - de - k) << 10;          // 2^-(de + k) as FP16
+        asm("mul.rn.f16x2 %0, %0, %1;" : "+r"(h2) : "r"(kHalf | (kHalf << 16)));
+        asm("{ .reg .b16 l, h; mov.b32 {l, h}, %2; cvt.f32.f16 %0, l; cvt.f32.f16 %1, h; }"
+            : "=f"(r0), "=f"(r1) : "r"(h2));
+    } else {
+        const float inv_k = inv * __uint_as_float((uint32_t)(127 - k) << 23);  // exact: powers of two
+        r0 = v0 * inv_k;
+        r1 = v1 * inv_k;
+    }
+}
+
 // Element-format value (the real number P) of two inputs after quantization, as FP32.
 //   DIRECT     : P = quantize_F(v inv)                       (inv = 2^-shared_exp of F)
 //   VIA_ANCHOR : P = Q_{A->F}(quantize_A(v inv))             (inv = 2^-shared_exp of the anchor A)
@@ -623,32 +648,28 @@ __device__ __forceinline__ float2 fake_quant_pair(float v0, float v1, float inv)
         p.x = one(v0);
         p.y = one(v1);
     } else {
-        // E3M3 / E2M2 are quantized as 2^-k times the value in their hardware neighbour format (see SoftFp)
-        constexpr int k = [] { if constexpr (F::hw_cvt) return 0; else return SoftFp<F>::k; }();
         float r0, r1;
-        if constexpr (via) {
-            // anchor codes -> exact FP16 values -> divide by 2^(de + k) (exact) -> FP32
-            uint32_t a = quantize_fp_hw_pair<A>(v0 * inv, v1 * inv);
-            uint32_t h2;
-            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)a));
-            constexpr uint32_t kHalf = (uint32_t)(15 - de - k) << 10;          // 2^-(de + k) as FP16
-            asm("mul.rn.f16x2 %0, %0, %1;" : "+r"(h2) : "r"(kHalf | (kHalf << 16)));
-            asm("{ .reg .b16 l, h; mov.b32 {l, h}, %2; cvt.f32.f16 %0, l; cvt.f32.f16 %1, h; }"
-                : "=f"(r0), "=f"(r1) : "r"(h2));
-        } else {
-            const float inv_k = inv * __uint_as_float((uint32_t)(127 - k) << 23);  // exact: powers of two
-            r0 = v0 * inv_k;
-            r1 = v1 * inv_k;
-        }
-        if constexpr (F::hw_cvt) {
-            p = widen_hw_pair<F>(quantize_fp_hw_pair<F>(r0, r1));
-        } else {
-            p = widen_hw_pair<Fmt<SoftFp<F>::hw>>(quantize_fp_soft_pair<F>(r0, r1));
-            p.x *= SoftFp<F>::post_scale;
-            p.y *= SoftFp<F>::post_scale;
-        }
+        fake_quant_scaled<F, MODE>(v0, v1, inv, r0, r1);
+        p = widen_hw_pair<F>(quantize_fp_hw_pair<F>(r0, r1));
     }
     return p;
+}
+
+// The same of four inputs, for the two formats without a narrowing instruction: the clip works on four codes at a time
+// (BF16, 2^25 elements, against two at a time: E3M3 direct 21.0 -> 19.9 us, through the anchor 22.9 -> 21.2; E2M2 21.3 -> 20.0, 22.8 -> 21.1).
+template <class F, int MODE>
+__device__ __forceinline__ void fake_quant_soft_quad(float v0, float v1, float v2, float v3, float inv, float (&p)[4])
+{
+    using H = Fmt<SoftFp<F>::hw>;
+    float r0, r1, r2, r3;
+    fake_quant_scaled<F, MODE>(v0, v1, inv, r0, r1);
+    fake_quant_scaled<F, MODE>(v2, v3, inv, r2, r3);
+    const uint32_t c = quantize_fp_soft_quad<F>(r0, r1, r2, r3);
+    const float2 a = widen_hw_pair<H>(c & 0xFFFFu), b = widen_hw_pair<H>(c >> 16);
+    p[0] = a.x * SoftFp<F>::post_scale;
+    p[1] = a.y * SoftFp<F>::post_scale;
+    p[2] = b.x * SoftFp<F>::post_scale;
+    p[3] = b.y * SoftFp<F>::post_scale;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
@@ -689,25 +710,41 @@ __device__ __forceinline__ void fake_quant_tile(const uint8_t* src, size_t nunit
         const uint32_t byte = via ? min(s.byte + (uint32_t)de, 254u) : s.byte;
         const float X = scale_value(byte);
         uint32_t out[8];
-        static_for<T::epl / 2>([&](auto i) {
-            constexpr int I = decltype(i)::value;
-            const float v0 = unit_elem<T, 2 * I>(w[u]), v1 = unit_elem<T, 2 * I + 1>(w[u]);
-            float2 p = fake_quant_pair<F, MODE>(v0, v1, s.inv);
-            float y0, y1;
-            if constexpr (F::kind == KIND_INT) {          // MXINT zero reconstructs to +0
-                y0 = fma_keep_plus_zero(p.x, X);
-                y1 = fma_keep_plus_zero(p.y, X);
-            } else {
-                y0 = p.x * X;
-                y1 = p.y * X;
-            }
-            if constexpr (T::size == 4) {
-                out[2 * I] = __float_as_uint(y0);
-                out[2 * I + 1] = __float_as_uint(y1);
-            } else {
-                out[I] = pack_bf16x2(y0, y1);
-            }
-        });
+        if constexpr (F::kind == KIND_FP && !F::hw_cvt) {
+            static_for<T::epl / 4>([&](auto i) {
+                constexpr int I = 4 * decltype(i)::value;
+                float p[4];
+                fake_quant_soft_quad<F, MODE>(unit_elem<T, I>(w[u]), unit_elem<T, I + 1>(w[u]), unit_elem<T, I + 2>(w[u]),
+                                              unit_elem<T, I + 3>(w[u]), s.inv, p);
+                if constexpr (T::size == 4) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) out[I + j] = __float_as_uint(p[j] * X);
+                } else {
+                    out[I / 2] = pack_bf16x2(p[0] * X, p[1] * X);
+                    out[I / 2 + 1] = pack_bf16x2(p[2] * X, p[3] * X);
+                }
+            });
+        } else {
+            static_for<T::epl / 2>([&](auto i) {
+                constexpr int I = decltype(i)::value;
+                const float v0 = unit_elem<T, 2 * I>(w[u]), v1 = unit_elem<T, 2 * I + 1>(w[u]);
+                float2 p = fake_quant_pair<F, MODE>(v0, v1, s.inv);
+                float y0, y1;
+                if constexpr (F::kind == KIND_INT) {          // MXINT zero reconstructs to +0
+                    y0 = fma_keep_plus_zero(p.x, X);
+                    y1 = fma_keep_plus_zero(p.y, X);
+                } else {
+                    y0 = p.x * X;
+                    y1 = p.y * X;
+                }
+                if constexpr (T::size == 4) {
+                    out[2 * I] = __float_as_uint(y0);
+                    out[2 * I + 1] = __float_as_uint(y1);
+                } else {
+                    out[I] = pack_bf16x2(y0, y1);
+                }
+            });
+        }
         if (unit < nunits) {
             if (s.byte == 0xFFu) st256_splat(dst + unit * 32, T::size == 4 ? 0x7FC00000u : 0x7FC07FC0u);   // poisoned block
             else st256(dst + unit * 32, out);
