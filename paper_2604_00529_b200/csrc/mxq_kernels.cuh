@@ -1666,7 +1666,8 @@ __device__ __forceinline__ void dequantize_wide_tile(const uint8_t* __restrict__
     for (int u = 0; u < U; ++u) {
         const size_t unit = u0 + u * 32;
         if (unit < nunits) {
-            load_bytes<IB>(w[u], codes + unit * IB);
+            if constexpr (IB == 3 || (IB > 4 && IB < 8)) load_piece<IB>(w[u], codes, unit);
+            else load_bytes<IB>(w[u], codes + unit * IB);
             sb[u] = ld_u8(scales + (unit >> scale_shift));
         } else {
 #pragma unroll
