@@ -256,3 +256,25 @@ def test_release_build_reports_that_it_is_not_a_debug_build():
     assert L.mxq_debug_report(ctypes.byref(info), 0) == 0 and info.enabled == 0 and info.violations == 0
     L.mxq_debug_trim_ranges.argtypes = [ctypes.c_size_t]
     assert L.mxq_debug_trim_ranges(64) == 0
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("src,dst", [("int7", "int5"), ("int5", "int3"), ("e3m3", "e2m2"), ("e3m2", "e2m1")])
+def test_stored_lower_formats_stay_inside_their_buffers(D, n, src, dst):
+    """The unpacking of sources below eight bits, and the FP32 reconstruction's aligned words round 5- and 3-byte pieces."""
+    stream = torch.cuda.current_stream().cuda_stream
+    rng = np.random.default_rng(n)
+    hc = rng.integers(0, 1 << orc.bits(src), n).astype(np.uint8)
+    hs = rng.integers(0, 256, n // 32).astype(np.uint8)
+    codes, scales = to_dev(orc.pack(hc, orc.bits(src))), to_dev(hs)
+    report(D)
+    lc, ls = u8(n * orc.bits(dst) // 8), u8(n // 32)
+    assert D.mxq_slice_scale(P(codes), P(scales), n, 32, FORMATS[src], FORMATS[dst], P(lc), P(ls), stream) == 0
+    y32 = torch.empty(n, dtype=torch.float32, device="cuda")
+    assert D.mxq_dequantize(P(lc), P(ls), n, FORMATS[dst], 32, P(y32), 0, stream) == 0
+    info = report(D)
+    assert info.enabled == 1 and info.checked_launches == 2
+    assert info.violations == 0, "first bad access: %#x (%d bytes)" % (info.first_address, info.first_bytes)
+    wc, ws = orc.slice_scale(hc, hs, src, dst)
+    assert np.array_equal(to_host(lc), orc.pack(wc, orc.bits(dst))) and np.array_equal(to_host(ls), ws)
+    assert np.array_equal(to_host(y32).view(np.uint32), orc.dequantize(wc, ws, dst).view(np.uint32))
