@@ -255,13 +255,20 @@ __host__ __device__ constexpr uint32_t half_bits(int m, int e)
 // is too small to carry any other value of eight significant bits (|r| 2^-10 is below their spacing) over a halfway point.
 // Negative sums (r below -M) become 0 = the symmetric clip; the second one is the same clip of the other side:
 // 2M - (M + q) = M - q, and (M - q) ^ M is the two's complement of q in B bits.
-template <int B, int E>
+//   MIN : the second clip as a packed integer minimum on the logic pipe instead (the first sum then takes -r, so that it is
+//         M - q already).
+template <int B, int E, bool MIN = false>
 __device__ __forceinline__ uint32_t round_halves(uint32_t p)
 {
     constexpr uint32_t M = (1u << (B - 1)) - 1u;
     constexpr uint32_t c = half_bits(1025, E - 34);                // 2^(E - 24) (1 + 2^-10)
-    const uint32_t r = hfma2_relu(p, both_halves(c), both_halves(M));
-    return hfma2_relu(r, both_halves(half_bits(-1, 0)), both_halves(2 * M));
+    if constexpr (MIN) {
+        const uint32_t r = hfma2_relu(p, both_halves(c | 0x8000u), both_halves(M));
+        return __vminu2(r, both_halves(2 * M));
+    } else {
+        const uint32_t r = hfma2_relu(p, both_halves(c), both_halves(M));
+        return hfma2_relu(r, both_halves(half_bits(-1, 0)), both_halves(2 * M));
+    }
 }
 
 // Word number `word` of the bitstream that repeats one B-bit code.
@@ -1083,12 +1090,12 @@ __device__ __forceinline__ uint32_t e4m3_word_clean(uint32_t x, uint32_t& nans)
 
 // Eight codes (the quads 2J and 2J + 1 of a lane's 32) in a lower format: two streams for pack_streams, or,
 // for the 4-bit formats, one finished output word.  MXINT codes stay XORed with M until ss_finish.
-template <class FL, int J>
+template <class FL, int J, bool MIN>
 __device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntHalves& w1, uint32_t (&z)[8])
 {
     constexpr int B = FL::bits, E = 9 + B;                     // r = p 2^(8-b_h) / 2^(8-B)
-    const uint32_t y0 = round_halves<B, E>(w0.b) * (1u << B) + round_halves<B, E>(w0.a);
-    const uint32_t y1 = round_halves<B, E>(w1.b) * (1u << B) + round_halves<B, E>(w1.a);
+    const uint32_t y0 = round_halves<B, E, MIN>(w0.b) * (1u << B) + round_halves<B, E, MIN>(w0.a);
+    const uint32_t y1 = round_halves<B, E, MIN>(w1.b) * (1u << B) + round_halves<B, E, MIN>(w1.a);
     if constexpr (B == 4) {
         z[J] = __byte_perm(y0, y1, 0x6420);
     } else {
@@ -1123,6 +1130,16 @@ __device__ __forceinline__ void ss_finish(const uint32_t (&z)[8], uint32_t (&out
 template <int I, class... FL>
 using ss_target_t = typename std::tuple_element<I, std::tuple<FL...>>::type;
 
+// Which clip of round_halves: the packed minimum from MXINT8, where the FMA pipe has become the fuller one (2^26 codes, multiply-add
+// against minimum: -> 6 + 4 bits 27.6 and 25.3 us, 7 + 5 31.3 and 29.7, 6 + 4 + 2 32.7 and 30.9, -> 2 15.8 and 15.0, -> 7 20.5 and
+// 20.1); the multiply-add from narrower sources, whose unpacking is logic (MXINT6 -> MXINT4 14.3 and 16.2, MXINT4 -> MXINT2 12.4 and
+// 13.7), and to 5 bits, where the minimum costs registers (-> 5 19.3 and 21.5; 5 + 4 over four layers 299 and, spilling, 385).
+template <class FH, class FL>
+__host__ __device__ constexpr bool ss_min_clip()
+{
+    return FH::bits == 8 && FL::bits != 5;
+}
+
 // The 32 codes of one lane to one or more lower formats, eight codes at a time so that what
 // the targets share (sign masks and magnitudes, FP16 values) lives only that long.  E4M3 anchors:
 // NAN_CODES = false promises that none of the codes is a NaN code.  A NaN code maps to the largest magnitude with
@@ -1138,7 +1155,8 @@ __device__ __forceinline__ void ss_unit(const uint32_t (&in)[NW], uint32_t (&z)[
             const IntHalves w0 = int_halves<FH, 2 * J>(in), w1 = int_halves<FH, 2 * J + 1>(in);
             static_for<(int)sizeof...(FL)>([&](auto i) {
                 constexpr int I = decltype(i)::value;
-                ss_int_quad_pair<ss_target_t<I, FL...>, J>(w0, w1, z[I]);
+                using F = ss_target_t<I, FL...>;
+                ss_int_quad_pair<F, J, ss_min_clip<FH, F>()>(w0, w1, z[I]);
             });
         } else {
             uint32_t h[4], nans[2] = {0, 0};
