@@ -1265,19 +1265,19 @@ __device__ __forceinline__ uint8_t* slice_scale_stage()
 }
 
 // Resident CTAs (of 128 threads) per SM the single-tensor kernel is compiled for, i.e. its register
-// budget.  Measured at 2^26 codes with 10 / 12 / 14 / 16 CTAs: the MXINT conversions are fastest with
-// room for 40 - 48 registers (both lane units' arithmetic interleaves; MXINT8 -> MXINT4 8 % faster
-// than at 32 registers), the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
-// registers); with tiled scale outputs 14 CTAs would spill, so those keep 12.
-template <class FH, class SCALES>
+// budget.  MXINT conversions to more than four bits are fastest with room for 40 - 48 registers (2^26 codes, 10 against 14 CTAs:
+// -> 6 19.3 and 20.0 us, -> 5 19.6 and 21.1), to four and fewer in 32 (MXINT8 -> MXINT4 of 2^24 codes 4.13 and 4.01, of 2^26
+// the same; -> 3 17.1 and 16.7; MXINT5 -> MXINT3 16.1 and 15.5); the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
+// registers).  With tiled scale outputs 14 CTAs would spill, so those keep 12.
+template <class FH, class FL, class SCALES>
 __host__ __device__ constexpr int slice_scale_min_ctas()
 {
     if constexpr (!std::is_same_v<SCALES, uint8_t*>) return 12;
-    else return FH::kind == KIND_INT ? 10 : 14;
+    else return FH::kind == KIND_INT && FL::bits > 4 ? 10 : 14;
 }
 
 template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*, bool HALVES = false>
-__global__ void __launch_bounds__(THREADS, slice_scale_min_ctas<FH, SCALES>())
+__global__ void __launch_bounds__(THREADS, slice_scale_min_ctas<FH, FL, SCALES>())
 slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits,
                    size_t nscales, uint8_t* __restrict__ out_codes, SCALES out_scales)
 {
@@ -1509,8 +1509,10 @@ struct SsPairItemBlock {
     TileIndex index;
 };
 
+// (Resident CTAs: for MXINT8 ten, because twelve spill for some pairs -- four layers to 5 + 4 bits 363 us against 292, 6 + 4 305 and
+// 302, 7 + 5 361 and 358; for E4M3 twelve.)
 template <class FH, class FL1, class FL2, int U, int THREADS, int K>
-__global__ void __launch_bounds__(THREADS, 12)
+__global__ void __launch_bounds__(THREADS, FH::kind == KIND_INT ? 10 : 12)
 slice_scale_pair_batched_kernel(const __grid_constant__ SsPairItemBlock<K> blk)
 {
     pdl_release();
