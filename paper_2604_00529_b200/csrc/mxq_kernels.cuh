@@ -14,9 +14,9 @@
 // then waits for its predecessor (see pdl_release / prefetch_tile / pdl_acquire in mxq_access.cuh).
 //
 // All of them are bound by HBM traffic, with the integer/logic pipe (64 lanes per clock per SM) as
-// the second bound; the arithmetic below is shaped to stay under it: packed 16-bit maxima, round-down
-// FP32 adds instead of float->int conversions, four 8-bit codes per register (SWAR), per-byte signs
-// by byte permutes and one multiply, the sm_100a narrowing conversion instructions for MXFP.
+// the second bound; the arithmetic below is shaped to stay under it: packed 16-bit maxima, MXINT rounding as
+// packed FP16 multiply-adds (round-down FP32 adds for FP32 sources), codes packed by multiply-adds, signs
+// by byte permutes, the sm_100a narrowing conversion instructions for MXFP.
 #pragma once
 #include <cstdint>
 #include <tuple>
@@ -1293,12 +1293,11 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
 
 // Several targets from one read of the anchor (the elastic-serving case: one stored checkpoint, several lower
 // precisions wanted at once).  Per element 1.03 bytes are read once instead of once per target, and what the
-// conversions share (sign masks and magnitudes of the MXINT8 codes, the FP16 values of the E4M3 codes) is
-// computed once.  The set of targets is a compile-time list: a kernel that walks a run-time list of formats
-// keeps the shared words in registers across a switch and took 38 - 46 us for MXINT8 -> {7, 5, 3} bits of 2^25.8
-// codes (block 64) where these take 31 (a pass per target: 53; the bytes alone: 26).  Compiled for 12 resident
-// CTAs (40 registers): 10 take 32 us, 14 spill and take 33, one unit per lane at 16 CTAs takes 35.  Sets of four spill at 12
-// (MXINT8 -> {7, 6, 4, 2} of 2^24 codes 12.9 us) and get 10 (12.0).
+// conversions share (the FP16 values of the codes) is computed once.  The set of targets is a compile-time list: a kernel that
+// walks a run-time list of formats keeps the shared words in registers across a switch and took 38 - 46 us for MXINT8 -> {7, 5, 3}
+// bits of 2^25.8 codes (block 64) where these take 30 (a pass per target: 50; the bytes alone: 26.7).  Compiled for 12
+// resident CTAs (40 registers): with 10 that set takes 30.9 us, {6, 4} of 2^26 codes 27.2 against 25.0, {7, 5} 31.2 against 29.0; with 14
+// most sets spill.  Sets of four spill at 12 and get 10.
 struct SsOut {
     uint8_t* codes;
     uint8_t* scales;
