@@ -1266,14 +1266,14 @@ __device__ __forceinline__ uint8_t* slice_scale_stage()
 
 // Resident CTAs (of 128 threads) per SM the single-tensor kernel is compiled for, i.e. its register
 // budget.  MXINT conversions to more than four bits are fastest with room for 40 - 48 registers (2^26 codes, 10 against 14 CTAs:
-// -> 6 19.3 and 20.0 us, -> 5 19.6 and 21.1), to four and fewer in 32 (MXINT8 -> MXINT4 of 2^24 codes 4.13 and 4.01, of 2^26
-// the same; -> 3 17.1 and 16.7; MXINT5 -> MXINT3 16.1 and 15.5); the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
+// -> 6 19.3 and 20.0 us, -> 5 19.6 and 21.1) and to two (14.4 and 14.7), to four and three in 32 (MXINT8 -> MXINT4 of 2^24 codes
+// 4.13 and 4.01, of 2^26 the same; -> 3 17.1 and 16.7; MXINT5 -> MXINT3 16.1 and 15.5); the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
 // registers).  With tiled scale outputs 14 CTAs would spill, so those keep 12.
 template <class FH, class FL, class SCALES>
 __host__ __device__ constexpr int slice_scale_min_ctas()
 {
     if constexpr (!std::is_same_v<SCALES, uint8_t*>) return 12;
-    else return FH::kind == KIND_INT && FL::bits > 4 ? 10 : 14;
+    else return FH::kind == KIND_INT && FL::bits != 4 && FL::bits != 3 ? 10 : 14;
 }
 
 template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*, bool HALVES = false>
