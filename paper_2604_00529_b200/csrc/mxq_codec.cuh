@@ -85,20 +85,18 @@ struct BlockScale {
     float inv;       // 2^-shared_exp (exact power of two)
 };
 
-// `amax_bits` = FP32 bit pattern of max_i |V_i| (sign cleared).  Inf/NaN patterns poison the block.
+// `amax_bits` = FP32 bit pattern of max_i |V_i| (sign cleared; only the exponent field is looked at).  Inf/NaN patterns
+// poison the block.  Field f stands for floor(log2 amax) = f - 127; a subnormal or zero amax (f = 0) is clamped to byte 0 whatever
+// its leading bit, since e_max >= 0.
 template <class F>
 __device__ __forceinline__ BlockScale block_scale(uint32_t amax_bits)
 {
     const uint32_t ex = amax_bits >> 23;
-    // floor(log2 amax): exponent field for normals, position of the leading one for subnormals;
-    // zero gives -150, which the clamp below turns into byte 0.
-    int e = ex ? (int)ex - 127 : (31 - __clz(amax_bits)) - 149;
-    int se = max(e - F::emax, -127);                 // e <= 127 and e_max >= 0: no upper clamp needed
+    const uint32_t b = (uint32_t)max((int)ex - F::emax, 0);
     BlockScale s;
-    s.byte = amax_bits >= 0x7F800000u ? 0xFFu : (uint32_t)(se + 127);
-    uint32_t field = (uint32_t)(127 - se);           // exponent field of 2^-se, in [0, 254]
-    uint32_t ib = field << 23;
-    if constexpr (F::emax == 0) ib = field ? ib : 0x00400000u;   // 2^-127 is an FP32 subnormal
+    s.byte = ex == 255u ? 0xFFu : b;
+    uint32_t ib = (254u << 23) - (b << 23);          // 2^(127 - b): exponent field 254 - b
+    if constexpr (F::emax == 0) ib = b == 254u ? 0x00400000u : ib;   // 2^-127 is an FP32 subnormal
     s.inv = __uint_as_float(ib);
     return s;
 }

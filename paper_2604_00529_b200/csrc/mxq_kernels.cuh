@@ -178,7 +178,7 @@ __device__ __forceinline__ float max3_abs_nan(float a, float b, float c)
     return d;
 }
 
-// FP32 bit pattern of max |element| over the lane unit; any NaN yields a NaN pattern, an
+// FP32 bit pattern of max |element| over the lane unit, for BF16 its upper half; any NaN yields a NaN pattern, an
 // infinity the infinity pattern (both >= 0x7F800000, both larger than every finite pattern).
 template <class T>
 __device__ __forceinline__ uint32_t unit_amax_bits(const uint32_t (&w)[8])
@@ -196,8 +196,8 @@ __device__ __forceinline__ uint32_t unit_amax_bits(const uint32_t (&w)[8])
         uint32_t a = __vimax3_s16x2(w[0] & kAbs, w[1] & kAbs, w[2] & kAbs);
         uint32_t b = __vimax3_s16x2(w[3] & kAbs, w[4] & kAbs, w[5] & kAbs);
         uint32_t c = __vimax3_s16x2(w[6] & kAbs, w[7] & kAbs, a);
-        uint32_t m = __vmaxu2(b, c);
-        return max(m << 16, m & 0xFFFF0000u);
+        const uint32_t m = __vmaxu2(b, c);
+        return max(m, m << 16);                               // (the low half is not part of the result)
     }
 }
 
