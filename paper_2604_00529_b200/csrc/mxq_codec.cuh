@@ -242,21 +242,8 @@ __device__ __forceinline__ float decode(uint32_t code)
 }
 
 // ------------------------------------------------------------------------------------------
-// Slice-and-Scale element maps (Eq. 4-5), scalar forms
+// Slice-and-Scale element map (Eq. 5), scalar form
 // ------------------------------------------------------------------------------------------
-
-// Eq. 4 on one sign-extended anchor element: shift the magnitude right by de, round on the most
-// significant dropped bit, clip, restore the sign.
-template <class FH, class FL>
-__device__ __forceinline__ uint32_t ss_int_elem(uint32_t code)
-{
-    constexpr int de = FH::emax - FL::emax;
-    int32_t p = (int32_t)(code << (32 - FH::bits)) >> (32 - FH::bits);
-    uint32_t mag = (uint32_t)(p < 0 ? -p : p);
-    uint32_t q = de > 0 ? (mag + (1u << (de > 0 ? de - 1 : 0))) >> de : mag;
-    q = min(q, FL::max_mag);
-    return (p < 0 ? 0u - q : q) & FL::mask;
-}
 
 // Eq. 5 on one anchor element: decode, divide by 2^de (exact), quantize to the low format.
 // An E4M3 NaN code maps to the sign-preserved largest magnitude.

@@ -422,21 +422,14 @@ __device__ __forceinline__ uint32_t quantize_int_quad(float v0, float v1, float 
     }
 }
 
-// 0xFF / 0x00 per byte: the signs of elements 4Q .. 4Q+3 of a lane unit, straight from the raw words.
-template <class T, int Q>
+// 0xFF / 0x00 per byte: the signs of elements 4Q .. 4Q+3 of an FP32 lane unit, straight from the raw words.
+template <int Q>
 __device__ __forceinline__ uint32_t unit_sign_bytes(const uint32_t (&w)[8])
 {
-    uint32_t full;
-    if constexpr (T::size == 2) {
-        // two BF16 per word: sign bits sit at the top of bytes 1 and 3 (selector bit 3 replicates it)
-        asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(full) : "r"(w[2 * Q]), "r"(w[2 * Q + 1]));
-    } else {
-        uint32_t a, b;
-        asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(a) : "r"(w[4 * Q]), "r"(w[4 * Q + 1]));
-        asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(b) : "r"(w[4 * Q + 2]), "r"(w[4 * Q + 3]));
-        full = __byte_perm(a, b, 0x5410);
-    }
-    return full;
+    uint32_t a, b;
+    asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(a) : "r"(w[4 * Q]), "r"(w[4 * Q + 1]));
+    asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(b) : "r"(w[4 * Q + 2]), "r"(w[4 * Q + 3]));
+    return __byte_perm(a, b, 0x5410);
 }
 
 // Codes of one lane unit, packed as a little-endian bitstream.
@@ -444,12 +437,13 @@ template <class T, class F, int NW>
 __device__ __forceinline__ void quantize_unit(const uint32_t (&w)[8], float inv, uint32_t (&out)[NW])
 {
     if constexpr (F::kind == KIND_INT) {
+        static_assert(T::size == 4, "BF16 -> MXINT: quantize_unit_bf16_int");
         constexpr int NQ = T::epl / 4;
         uint32_t z[NQ];
         static_for<NQ>([&](auto qi) {
             constexpr int Q = decltype(qi)::value;
             z[Q] = quantize_int_quad<F>(unit_elem<T, 4 * Q>(w), unit_elem<T, 4 * Q + 1>(w), unit_elem<T, 4 * Q + 2>(w),
-                                        unit_elem<T, 4 * Q + 3>(w), inv, unit_sign_bytes<T, Q>(w));
+                                        unit_elem<T, 4 * Q + 3>(w), inv, unit_sign_bytes<Q>(w));
         });
         if constexpr (F::bits == 8) {
 #pragma unroll
@@ -1064,10 +1058,7 @@ __device__ __forceinline__ void ss_unit_by_element(const uint32_t (&in)[NWI], ui
     static_for<32>([&](auto i) {
         constexpr int I = decltype(i)::value;
         const uint32_t c = get_code<FH::bits, I>(in);
-        uint32_t d;
-        if constexpr (FH::kind == KIND_INT) d = ss_int_elem<FH, FL>(c);
-        else d = ss_fp_elem<FH, FL>(c);
-        put_code<FL::bits, I>(out, d);
+        put_code<FL::bits, I>(out, ss_fp_elem<FH, FL>(c));
     });
 }
 
