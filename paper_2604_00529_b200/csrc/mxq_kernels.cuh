@@ -298,6 +298,38 @@ __device__ __forceinline__ uint32_t join_halves_top(uint32_t y)
     return (y & 0xFFFFu) * (k * (k - 1u)) + y * k;
 }
 
+// Two W-bit fields in the low bits of the halves of y -> their 2W-bit stream in the low bits (the rest clear): one operation less
+// than join_halves_top, on the logic pipe.
+template <int W>
+__device__ __forceinline__ uint32_t join_halves_low(uint32_t y)
+{
+    return (y >> 16) * ((1u << W) - (1u << 16)) + y;
+}
+
+// NZ streams of W bits, each in the low bits of its word (the rest clear) -> the little-endian bitstream: a multiply-add
+// per stream and a shift where one crosses a word; three byte permutes join four streams of 24 bits.
+template <int W, int NZ, int NW>
+__device__ __forceinline__ void pack_low_streams(const uint32_t (&z)[NZ], uint32_t (&out)[NW])
+{
+    static_assert(NW * 32 >= NZ * W, "output too small");
+    if constexpr (W == 24 && NZ % 4 == 0) {
+#pragma unroll
+        for (int g = 0; g < NZ / 4; ++g) {
+            out[3 * g + 0] = __byte_perm(z[4 * g + 0], z[4 * g + 1], 0x4210);
+            out[3 * g + 1] = __byte_perm(z[4 * g + 1], z[4 * g + 2], 0x5421);
+            out[3 * g + 2] = __byte_perm(z[4 * g + 2], z[4 * g + 3], 0x6542);
+        }
+    } else {
+        static_for<NZ>([&](auto j) {
+            constexpr int J = decltype(j)::value;
+            constexpr int off = J * W, wi = off >> 5, sh = off & 31;
+            if constexpr (sh == 0) out[wi] = z[J];
+            else out[wi] += z[J] * (1u << sh);
+            if constexpr (sh + W > 32) out[wi + 1] = z[J] >> (32 - sh);
+        });
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // Q_f: quantize (Eq. 1-3)
 // ------------------------------------------------------------------------------------------
@@ -1166,13 +1198,75 @@ __device__ __forceinline__ void ss_unit(const uint32_t (&in)[NW], uint32_t (&z)[
     });
 }
 
-// Convert the 32 codes of one lane.  in: 8*FH::bits/8... words of the high format's bitstream.
-template <class FH, class FL, int NWI, int NWO>
+// The 32 MXINT8 codes of one lane to ONE lower format, with fewer instructions than the general form above takes for a
+// single target: the codes come as sign-extended 16-bit pairs (one byte permute per pair, no exclusive OR), one packed
+// add-with-maximum brings them under the exponent of 1024 and clips the negative side at -M, and the rounding's relu clips the other
+// one.  For 3 and 2 bits the pairs hold codes four apart, so that eight codes join inside the halves.  Instructions per
+// lane unit against the general form: -> 7 bits 186 and 197, 6 175 and 185, 4 127 and 131, 3 141 and 166, 2 130 and 155.  Where it is
+// used and where not: see the kernels.
+template <class FL, int NWO>
+__device__ __forceinline__ void ss_int8_unit(const uint32_t (&in)[8], uint32_t (&out)[NWO])
+{
+    constexpr int B = FL::bits;
+    constexpr uint32_t M = FL::max_mag;
+    constexpr uint32_t one = both_halves(half_bits(1, -17)), bias = both_halves(half_bits(-(1024 + 128), -17));
+    constexpr uint32_t factor = both_halves(half_bits(1025, B - 25) | 0x8000u);        // -(1 + 2^-10), see round_halves
+    const auto round_pair = [&](uint32_t p) {                                          // -> M - q
+        const uint32_t h = __viaddmax_s16x2(p, both_halves(0x6480u), both_halves(0x6480u - (M << (8 - B))));
+        return hfma2_relu(hfma2(h, one, bias), factor, both_halves(M));
+    };
+    // selector bit 3 replicates the sign of the byte
+    if constexpr (B <= 3) {
+        uint32_t z[4];
+        static_for<4>([&](auto jj) {
+            constexpr int J = decltype(jj)::value;
+            const uint32_t w0 = in[2 * J], w1 = in[2 * J + 1];
+            uint32_t p0, p1, p2, p3;
+            asm("prmt.b32 %0, %1, %2, 0xC480;" : "=r"(p0) : "r"(w0), "r"(w1));
+            asm("prmt.b32 %0, %1, %2, 0xD591;" : "=r"(p1) : "r"(w0), "r"(w1));
+            asm("prmt.b32 %0, %1, %2, 0xE6A2;" : "=r"(p2) : "r"(w0), "r"(w1));
+            asm("prmt.b32 %0, %1, %2, 0xF7B3;" : "=r"(p3) : "r"(w0), "r"(w1));
+            constexpr uint32_t k = 1u << B;
+            const uint32_t y = (round_pair(p3) * k + round_pair(p2)) * (k * k) + (round_pair(p1) * k + round_pair(p0));
+            if constexpr (B == 3) z[J] = join_halves_low<12>(y);
+            else z[J] = y;
+        });
+        if constexpr (B == 3) {
+            pack_low_streams<24>(z, out);
+        } else {
+            out[0] = __byte_perm(z[0], z[1], 0x6420);
+            out[1] = __byte_perm(z[2], z[3], 0x6420);
+        }
+    } else {
+        uint32_t y[8];
+        static_for<8>([&](auto jj) {
+            constexpr int J = decltype(jj)::value;
+            uint32_t a, b;
+            asm("prmt.b32 %0, %1, %1, 0xA280;" : "=r"(a) : "r"(in[J]));
+            asm("prmt.b32 %0, %1, %1, 0xB391;" : "=r"(b) : "r"(in[J]));
+            y[J] = round_pair(b) * (1u << B) + round_pair(a);
+            if constexpr (B > 4) y[J] = join_halves_low<2 * B>(y[J]);
+        });
+        if constexpr (B == 4) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) out[j] = __byte_perm(y[2 * j], y[2 * j + 1], 0x6420);
+        } else {
+            pack_low_streams<4 * B>(y, out);
+        }
+    }
+    unbias_codes<B>(out);
+}
+
+// Convert the 32 codes of one lane.  in: 8*FH::bits/8... words of the high format's bitstream.  SHORT: by ss_int8_unit (MXINT8 only).
+template <class FH, class FL, bool SHORT, int NWI, int NWO>
 __device__ __forceinline__ void slice_scale_unit(const uint32_t (&in)[NWI], uint32_t (&out)[NWO])
 {
     if constexpr (FH::id == FL::id) {
 #pragma unroll
         for (int j = 0; j < NWO; ++j) out[j] = in[j];
+    } else if constexpr (SHORT) {
+        static_assert(FH::id == MXQ_INT8, "MXINT8 only");
+        ss_int8_unit<FL>(in, out);
     } else {
         uint32_t z[1][8];
         if constexpr (!FH::has_nan) {
@@ -1200,7 +1294,7 @@ __device__ __forceinline__ uint8_t ss_scale_byte(uint32_t b, int de)
 // scale i, or, with HALVES (block 16, two scales per lane unit), its own two as one 16-bit access: MXINT8 -> MXINT4 of
 // 2^25 codes 9.1 us, E4M3 -> E2M3 11.3, where a second pass over the upper half of the scales took 10.8 and 12.7.  (A
 // run-time choice between the two forms cost the larger blocks 2 - 9 %.)
-template <class FH, class FL, int U, bool HALVES, class SCALES>
+template <class FH, class FL, int U, bool HALVES, bool SHORT = false, class SCALES>
 __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
                                                  size_t nunits, size_t nscales, uint8_t* __restrict__ out_codes,
                                                  const SCALES& out_scales, size_t tile, uint8_t* stage)
@@ -1231,7 +1325,7 @@ __device__ __forceinline__ void slice_scale_tile(const uint8_t* __restrict__ cod
             if (unit < nscales) put_scale(out_scales, unit, ss_scale_byte(sb[u], de));
         }
         uint32_t out[NWO];
-        slice_scale_unit<FH, FL>(w[u], out);
+        slice_scale_unit<FH, FL, SHORT>(w[u], out);
         if constexpr (StagedTile<OB>::use) store_bytes<OB>(stage + (u * 32 + (threadIdx.x & 31)) * OB, out);
         else if (unit < nunits) store_bytes<OB>(out_codes + unit * OB, out);
     }
@@ -1260,18 +1354,41 @@ __device__ __forceinline__ uint8_t* slice_scale_stage()
 // -> 6 19.3 and 20.0 us, -> 5 19.6 and 21.1) and to two (14.4 and 14.7), to four and three in 32 (MXINT8 -> MXINT4 of 2^24 codes
 // 4.13 and 4.01, of 2^26 the same; -> 3 17.1 and 16.7; MXINT5 -> MXINT3 16.1 and 15.5); the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
 // registers).  With tiled scale outputs 14 CTAs would spill, so those keep 12.
-template <class FH, class FL, class SCALES>
+//   SMALL : see slice_scale_is_small.
+template <class FH, class FL, class SCALES, bool SMALL>
 __host__ __device__ constexpr int slice_scale_min_ctas()
 {
     if constexpr (!std::is_same_v<SCALES, uint8_t*>) return 12;
-    else return FH::kind == KIND_INT && FL::bits != 4 && FL::bits != 3 ? 10 : 14;
+    else return SMALL || (FH::kind == KIND_INT && FL::bits != 4 && FL::bits != 3) ? 10 : 14;
 }
 
-template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*, bool HALVES = false>
-__global__ void __launch_bounds__(THREADS, slice_scale_min_ctas<FH, FL, SCALES>())
+// MXINT8 in a launch of about one wave.  The next launch's CTAs are resident early (see mxq_access.cuh): as many as fit beside
+// this one's at once, the others wherever one of this one's has ended, so the more fit the more unevenly they spread, which a grid of
+// one wave does not make up for.  Kernels with ss_int8_unit and at most 10 CTAs to an SM (12 to 4 bits, whose code leaves room for no
+// fewer), against the larger launches' kernels: 2^23.25 codes -> 7 bits 3.9 and 4.4 us, 6 3.8 and 4.3, 4 3.3 and 4.0, 3 3.6 and 4.3; 2^22 -> 7 3.2
+// and 3.5, 3 3.0 and 3.2.  They stop at one wave (2^24 codes -> 6 bits 5.4 and 5.2), and to 4 bits also below five CTAs per SM, where the
+// other one is the faster (2^22 codes 2.65 and 2.4).  5 and 2 bits have one kernel (5 bits with 10 CTAs: 2^22.75 codes 4.2 us
+// against 3.2; 2 bits: at most 12 either way).
+template <class FH, class FL>
+__host__ __device__ constexpr bool slice_scale_has_small()
+{
+    return FH::id == MXQ_INT8 && (FL::bits == 7 || FL::bits == 6 || FL::bits == 4 || FL::bits == 3);
+}
+
+template <class FL>
+inline bool slice_scale_is_small(size_t ctas)
+{
+    return ctas > (size_t)148 * (FL::bits == 4 ? 5 : 0) && ctas <= (size_t)148 * (FL::bits > 4 ? 10 : 12);
+}
+
+template <class FH, class FL, int U, int THREADS, class SCALES = uint8_t*, bool HALVES = false, bool SMALL = false>
+__global__ void __launch_bounds__(THREADS, slice_scale_min_ctas<FH, FL, SCALES, SMALL>())
 slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, size_t nunits,
                    size_t nscales, uint8_t* __restrict__ out_codes, SCALES out_scales)
 {
+    // (to 7 bits the general form is as fast in larger launches, to 6, 5 and 4 faster: 2^25 codes -> 6 9.8 us against 10.1, 2^24.5 -> 5
+    // 7.5 and 7.7; to 3 bits it takes 8.9 against 8.0, to 2 the same but 4.25 against 3.4 at 2^23.5)
+    constexpr bool kShort = FH::id == MXQ_INT8 && (SMALL || FL::bits <= 3);
     pdl_release();
     const size_t tile = (size_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5);
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
@@ -1279,7 +1396,7 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
     prefetch_tile<U, 4 * FH::bits>(codes, tile, nunits);
     pdl_acquire();
     if (tile * (32 * U) < nunits)
-        slice_scale_tile<FH, FL, U, HALVES>(codes, scales, nunits, nscales, out_codes, out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, HALVES, kShort>(codes, scales, nunits, nscales, out_codes, out_scales, tile, stage);
 }
 
 // Several targets from one read of the anchor (the elastic-serving case: one stored checkpoint, several lower
@@ -1466,11 +1583,14 @@ struct SsItemBlock {
 };
 
 // (Compiled for 12 resident CTAs: without the bound MXINT8 -> MXINT5 of four decoder layers takes 261 us instead of 223, the
-// other targets between 2.6 % less and 2 % more.)
-template <class FH, class FL, int U, int THREADS, int K>
-__global__ void __launch_bounds__(THREADS, 12)
+// other targets between 2.6 % less and 2 % more.  SMALL: see slice_scale_is_small; seven tensors of 2^23 codes in all -> 7 bits 4.0 us
+// against 4.4, 6 3.8 and 4.3, 3 3.4 and 3.8.)
+template <class FH, class FL, int U, int THREADS, int K, bool SMALL = false>
+__global__ void __launch_bounds__(THREADS, SMALL ? 10 : 12)
 slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
 {
+    // (2^25 codes, short against general form: -> 7 bits 10.7 us and 11.5, 3 8.4 and 8.9, 2^24 -> 2 4.05 and 4.3, 4 4.2 and 4.3)
+    constexpr bool kShort = FH::id == MXQ_INT8 && FL::bits < 8 && (SMALL || (FL::bits != 6 && FL::bits != 5));
     pdl_release();
     uint8_t* stage = slice_scale_stage<FL, U, THREADS>();
     // parameters: readable before the wait
@@ -1479,7 +1599,7 @@ slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
     prefetch_tile<U, 4 * FH::bits>(t.codes, tile, t.nunits);
     pdl_acquire();
     if (tile * (32 * U) < t.nunits)                       // whole warps
-        slice_scale_tile<FH, FL, U, false>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
+        slice_scale_tile<FH, FL, U, false, kShort>(t.codes, t.scales, t.nunits, t.nscales, t.out_codes, t.out_scales, tile, stage);
 }
 
 // Two targets from one read of every anchor of a set of tensors (the whole-model conversion of Sec. 3.5

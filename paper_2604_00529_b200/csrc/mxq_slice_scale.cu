@@ -29,6 +29,12 @@ int run_single(const void* codes, const uint8_t* scales, size_t n, int block, vo
                 ntiles = (nunits + 31) / 32;
             }
         }
+        // MXINT8 in about one wave: the kernel with fewer resident CTAs (measured at slice_scale_is_small).
+        if constexpr (slice_scale_has_small<FH, FL>()) {
+            if (slice_scale_is_small<FL>((ntiles + kThreads / 32 - 1) / (kThreads / 32)))
+                kern = block == 16 ? slice_scale_kernel<FH, FL, kU, kThreads, uint8_t*, true, true>
+                                   : slice_scale_kernel<FH, FL, kU, kThreads, uint8_t*, false, true>;
+        }
         return launch_kernel(kern, grid_for_tiles(ntiles, kThreads), kThreads, stream, static_cast<const uint8_t*>(codes),
                              scales, nunits, nscales, static_cast<uint8_t*>(out_codes), out_scales);
     } else {
@@ -72,6 +78,9 @@ int run_params(const SsDeviceItem* items_host, int count, size_t total_tiles, cu
             SsItemBlock<K> blk;
             fill_item_block(blk, items_host, count, total_tiles);
             auto kern = slice_scale_batched_param_kernel<FH, FL, kU, kThreads, K>;
+            if constexpr (slice_scale_has_small<FH, FL>() && FL::bits != 4 && K == kSmallBatchItems) {
+                if (slice_scale_is_small<FL>(total_tiles)) kern = slice_scale_batched_param_kernel<FH, FL, kU, kThreads, K, true>;
+            }
             return launch_kernel(kern, grid_for_units(total_tiles, 1), kThreads, stream, blk);
         });
     } else {

@@ -58,6 +58,45 @@ def test_slice_scale_on_both_sides_of_the_small_launch_rule(dst, block):
         assert torch.equal(os_.view, repeated(ws, os_.nbytes)), units
 
 
+@pytest.mark.parametrize("block", [16, 32, 64])
+@pytest.mark.parametrize("dst", ["int7", "int6", "int4", "int3", "int2"])
+def test_slice_scale_from_mxint8_on_both_sides_of_its_one_wave_rules(dst, block):
+    """Ten CTAs per SM (twelve to four and three bits; to four bits also five), and the smallest tensors."""
+    codes, scales = codes_and_scales("int8", block, 5 * block)
+    wc, ws = orc.slice_scale(codes, scales, "int8", dst, block)
+    packed = orc.pack(wc, orc.bits(dst))
+    for units in [1, 65, 3 * CTA - 2] + unit_counts(148 * 5) + unit_counts(148 * 10) + unit_counts(148 * 12):
+        n = max(units * 32, block) // block * block
+        oc, os_ = Guarded(mxq.codes_bytes(n, dst)), Guarded(n // block)
+        mxq.slice_scale(repeated(codes, n), repeated(scales, n // block), n, "int8", dst, block, oc.view, os_.view)
+        torch.cuda.synchronize()
+        oc.check()
+        os_.check()
+        assert torch.equal(oc.view, repeated(packed, oc.nbytes)), units
+        assert torch.equal(os_.view, repeated(ws, os_.nbytes)), units
+
+
+@pytest.mark.parametrize("ctas", [148 * 10, 148 * 10 + 1, 148 * 12, 148 * 12 + 1])
+@pytest.mark.parametrize("dst", ["int7", "int6", "int3"])
+def test_mxint8_sets_on_both_sides_of_the_one_wave_rules(dst, ctas):
+    codes, scales = codes_and_scales("int8", 32, 9)
+    wc, ws = orc.slice_scale(codes, scales, "int8", dst, 32)
+    packed = orc.pack(wc, orc.bits(dst))
+    items, outs = [], []
+    for units in (1, 2 * CTA - 3, (ctas - 4) * CTA - 64, CTA):        # 1 + 2 + (ctas - 4) + 1 CTAs
+        n = units * 32
+        oc, os_ = Guarded(mxq.codes_bytes(n, dst)), Guarded(units)
+        items.append((repeated(codes, n), repeated(scales, units), n, oc.view, os_.view))
+        outs.append((oc, os_))
+    mxq.slice_scale_batched(items, "int8", dst)
+    torch.cuda.synchronize()
+    for oc, os_ in outs:
+        oc.check()
+        os_.check()
+        assert torch.equal(oc.view, repeated(packed, oc.nbytes))
+        assert torch.equal(os_.view, repeated(ws, os_.nbytes))
+
+
 @pytest.mark.parametrize("block", [16, 32, 64, 128])
 @pytest.mark.parametrize("fmt", ["int8", "e4m3", "int7", "e2m3", "e2m2", "int4", "e2m1", "int3"])
 def test_reconstruction_on_both_sides_of_the_small_launch_rule(fmt, block):
