@@ -185,19 +185,21 @@ __device__ __forceinline__ void load_bytes(uint32_t (&w)[NW], const void* p)
 }
 
 // Piece number `piece` of NB bytes (3, 5, 6 or 7: no vector) of a stream that starts and ends on a word: the two or three aligned
-// words that hold it and a funnel shift, in place of NB or NB / 2 narrow loads (FP32 from 2^25 codes of 7 bits 31.1 -> 27.0 us,
-// 6 bits 28.3 -> 26.5, 5 bits 28.0 -> 25.7, 3 bits 26.3 -> 24.1).  No word behind the one with the piece's
+// words that hold it and a funnel shift, in place of NB or NB / 2 narrow loads (FP32 from 2^25 codes of 7 bits 30.8 -> 26.7 us,
+// 6 bits 28.3 -> 25.8, 5 bits 27.9 -> 25.2, 3 bits 26.2 -> 24.1).  No word behind the one with the piece's
 // last byte is read; the bytes of `w` beyond NB are undefined.
 template <int NB, int NW>
 __device__ __forceinline__ void load_piece(uint32_t (&w)[NW], const uint8_t* base, size_t piece)
 {
     static_assert(NB < 8 && NB > 2 && NB != 4 && NW == (NB + 3) / 4, "3, 5, 6 or 7 bytes");
-    const size_t off = piece * NB, at = off & ~(size_t)3, last = (off + NB - 1) & ~(size_t)3;
+    const size_t off = piece * NB;
     const uint32_t sh = ((uint32_t)off & 3u) * 8u;
-    const uint32_t w0 = ld_u32(base + at);
-    const uint32_t w1 = ld_u32(base + (at + 4 < last ? at + 4 : last));
+    base += off & ~(size_t)3;
+    // 5 and 6 bytes always reach into the second word, 3 and 7 bytes into the second and the third one if they start in the upper half
+    const uint32_t w0 = ld_u32(base);
+    const uint32_t w1 = ld_u32(base + (NB == 3 && sh < 16 ? 0 : 4));
     w[0] = __funnelshift_r(w0, w1, sh);
-    if constexpr (NB == 7) w[1] = __funnelshift_r(w1, ld_u32(base + last), sh);
+    if constexpr (NB == 7) w[1] = __funnelshift_r(w1, ld_u32(base + (sh < 16 ? 4 : 8)), sh);
     else if constexpr (NB > 4) w[1] = w1 >> sh;
 }
 

@@ -1795,9 +1795,14 @@ __device__ __forceinline__ void dequantize_wide_tile(const uint8_t* __restrict__
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const size_t unit = u0 + u * 32;
-        if (unit < nunits) {
-            if constexpr (IB == 3 || (IB > 4 && IB < 8)) load_piece<IB>(w[u], codes, unit);
-            else load_bytes<IB>(w[u], codes + unit * IB);
+        if constexpr (IB == 3 || (IB > 4 && IB < 8)) {
+            // lanes beyond the end take the last unit: inside a branch the shifts would wait for one unit's words before the
+            // next unit's are asked for (2^14 codes of 6 bits 1.7 us instead of 1.4)
+            const size_t mine = unit < nunits ? unit : nunits - 1;
+            load_piece<IB>(w[u], codes, mine);
+            sb[u] = ld_u8(scales + (mine >> scale_shift));
+        } else if (unit < nunits) {
+            load_bytes<IB>(w[u], codes + unit * IB);
             sb[u] = ld_u8(scales + (unit >> scale_shift));
         } else {
 #pragma unroll

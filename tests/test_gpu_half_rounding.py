@@ -4,9 +4,11 @@ from __future__ import annotations
 
 import numpy as np
 import pytest
+import torch
 
+import paper_2604_00529_b200 as mxq
 from oracle import mxq_oracle as orc
-from gpu_util import INT_FORMATS, bits_equal, first_diff, gpu_dequantize, gpu_quantize, gpu_slice_scale, ss_pairs
+from gpu_util import Guarded, INT_FORMATS, bits_equal, first_diff, gpu_dequantize, gpu_quantize, gpu_slice_scale, ss_pairs, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -80,3 +82,20 @@ def test_reconstruction_to_f32_of_pieces_that_are_no_vector(fmt):
         got = gpu_dequantize(orc.pack(codes, orc.bits(fmt)), scales, n, fmt)
         want = orc.dequantize(codes, scales, fmt)
         assert bits_equal(got, want), (units, first_diff(got, want))
+
+
+@pytest.mark.parametrize("fmt", ["int7", "int6", "int5", "int3", "e3m3", "e2m3", "e2m2"])
+def test_batched_reconstruction_to_f32_of_pieces_that_are_no_vector(fmt):
+    """The same pieces in one launch over tensors that end inside a warp's tile: lanes beyond an end read its last piece."""
+    rng = np.random.default_rng(11)
+    sets = []
+    for units in [1, 2, 15, 16, 17, 33, 65, 257]:
+        n = 32 * units
+        codes = rng.integers(0, 1 << orc.bits(fmt), n).astype(np.uint8)
+        scales = rng.integers(0, 256, units).astype(np.uint8)
+        sets.append((to_dev(orc.pack(codes, orc.bits(fmt))), to_dev(scales), n, Guarded(4 * n, torch.float32), orc.dequantize(codes, scales, fmt)))
+    mxq.dequantize_batched([(c, s, n, y.view) for c, s, n, y, _ in sets], fmt)
+    torch.cuda.synchronize()
+    for _, _, n, y, want in sets:
+        y.check()
+        assert bits_equal(to_host(y.view), want), (n, first_diff(to_host(y.view), want))
