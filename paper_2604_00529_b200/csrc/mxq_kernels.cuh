@@ -904,8 +904,17 @@ struct QItemBlock {
     TileIndex index;
 };
 
+// Resident CTAs (of 128 threads) per SM: 14 (against the compiler's own choice BF16 -> MXINT7 and MXINT5 of 2^25 elements and more take
+// 3 % less, the other formats the same to 1 %), but 12 from BF16 to E3M3 and E2M2, whose four-code clip wants more registers in small
+// sets (2^16 elements 2.09 us with 14, 2.0 with 12; 2^22.5 5.06 and 4.5, 2^25 17.2 and 16.7, 2^28 131 either way).
+template <class T, class F>
+__host__ __device__ constexpr int quantize_batched_min_ctas()
+{
+    return T::size == 2 && F::kind == KIND_FP && !F::hw_cvt ? 12 : 14;
+}
+
 template <class T, class F, int BLOCK, int U, int THREADS, int K>
-__global__ void __launch_bounds__(THREADS, 14)     // 14 resident CTAs: the MXINT8 anchor of the 224-tensor set 3.01 ms against 3.30
+__global__ void __launch_bounds__(THREADS, quantize_batched_min_ctas<T, F>())
 quantize_batched_kernel(const __grid_constant__ QItemBlock<K> blk)
 {
     pdl_release();
