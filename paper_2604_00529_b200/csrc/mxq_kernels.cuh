@@ -1130,7 +1130,7 @@ __device__ __forceinline__ uint32_t e4m3_word_clean(uint32_t x, uint32_t& nans)
 
 // Eight codes (the quads 2J and 2J + 1 of a lane's 32) in a lower format: two streams for pack_streams, or,
 // for the 4-bit formats, one finished output word.  MXINT codes stay XORed with M until ss_finish.
-template <class FL, int J, bool MIN>
+template <class FL, int J, bool MIN, bool LOW>
 __device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntHalves& w1, uint32_t (&z)[8])
 {
     constexpr int B = FL::bits, E = 9 + B;                     // r = p 2^(8-b_h) / 2^(8-B)
@@ -1139,8 +1139,8 @@ __device__ __forceinline__ void ss_int_quad_pair(const IntHalves& w0, const IntH
     if constexpr (B == 4) {
         z[J] = __byte_perm(y0, y1, 0x6420);
     } else {
-        z[2 * J] = join_halves_top<B>(y0);
-        z[2 * J + 1] = join_halves_top<B>(y1);
+        z[2 * J] = LOW ? join_halves_low<2 * B>(y0) : join_halves_top<B>(y0);
+        z[2 * J + 1] = LOW ? join_halves_low<2 * B>(y1) : join_halves_top<B>(y1);
     }
 }
 
@@ -1155,12 +1155,14 @@ __device__ __forceinline__ void ss_fp_quad_pair(const uint32_t (&h)[4], const ui
     }
 }
 
-template <class FL, int NWO>
+template <class FL, bool LOW = false, int NWO>
 __device__ __forceinline__ void ss_finish(const uint32_t (&z)[8], uint32_t (&out)[NWO])
 {
     if constexpr (FL::bits == 4) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) out[j] = z[j];
+    } else if constexpr (LOW) {
+        pack_low_streams<4 * FL::bits>(z, out);
     } else {
         pack_streams<FL::bits>(z, out);
     }
@@ -1180,6 +1182,15 @@ __host__ __device__ constexpr bool ss_min_clip()
     return FH::bits == 8 && FL::bits != 5;
 }
 
+// Streams joined in the low bits instead of the top ones: in a set whose targets all have more than five bits, which is 7 + 6 (2^24 codes 8.6 us
+// against 9.9, 2^22 4.0 and 4.7, 2^25.8 24.8 and 25.4).  With a narrower target the top form is the faster one or the
+// difference is small: 7 + 4 bits 9.2 and 7.8, 6 + 4 8.6 and 7.4, 7 + 5 8.9 and 8.8.
+template <class FH, class... FL>
+__host__ __device__ constexpr bool ss_low_join()
+{
+    return FH::id == MXQ_INT8 && sizeof...(FL) > 1 && ((FL::bits > 5) && ...);
+}
+
 // The 32 codes of one lane to one or more lower formats, eight codes at a time so that what
 // the targets share (sign masks and magnitudes, FP16 values) lives only that long.  E4M3 anchors:
 // NAN_CODES = false promises that none of the codes is a NaN code.  A NaN code maps to the largest magnitude with
@@ -1196,7 +1207,7 @@ __device__ __forceinline__ void ss_unit(const uint32_t (&in)[NW], uint32_t (&z)[
             static_for<(int)sizeof...(FL)>([&](auto i) {
                 constexpr int I = decltype(i)::value;
                 using F = ss_target_t<I, FL...>;
-                ss_int_quad_pair<F, J, ss_min_clip<FH, F>()>(w0, w1, z[I]);
+                ss_int_quad_pair<F, J, ss_min_clip<FH, F>(), ss_low_join<FH, FL...>()>(w0, w1, z[I]);
             });
         } else {
             uint32_t h[4], nans[2] = {0, 0};
@@ -1488,7 +1499,7 @@ __device__ __forceinline__ void slice_scale_set_tile(const uint8_t* __restrict__
             using F = ss_target_t<I, FL...>;
             constexpr int OB = 4 * F::bits;
             uint32_t out[OB / 4];
-            ss_finish<F>(z[I], out);
+            ss_finish<F, ss_low_join<FH, FL...>()>(z[I], out);
             if constexpr (StagedTile<OB>::use)
                 store_bytes<OB>(stage + 32 * U * ss_stage_offset<I, FL...>() + (u * 32 + lane) * OB, out);
             else if (l0 + u * 32 < valid) store_bytes<OB>(outs[I].codes + first * OB + (l0 + u * 32) * OB, out);
