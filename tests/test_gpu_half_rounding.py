@@ -37,10 +37,9 @@ def test_bf16_blocks_of_every_exponent(fmt, block):
     assert bits_equal(codes, orc.pack(wc, orc.bits(fmt))), first_diff(codes, orc.pack(wc, orc.bits(fmt)))
 
 
-@pytest.mark.parametrize("fmt", INT_FORMATS)
-def test_bf16_halfway_points(fmt):
-    """Every multiple of 1/4 below the next binade with its BF16 neighbours, both signs, under six scales: ties go away
-    from zero, the neighbours do not follow them, the upper end is clipped."""
+def halfway_points(fmt, s):
+    """Blocks of every multiple of 1/4 below the next binade that BF16 holds with its BF16 neighbours, both signs, times 2^s; each block's
+    scale byte is 127 + s.  (The neighbours of 0 are subnormals, which an exponent shift does not scale: signed zeros.)"""
     top = 1 << (orc.bits(fmt) - 1)
     r = np.arange(0, 4 * top, dtype=np.float32) / 4
     bits = (r.view(np.uint32) >> 16).astype(np.int64)
@@ -49,10 +48,20 @@ def test_bf16_halfway_points(fmt):
     near = np.resize(near, -(-near.size // 31) * 31).reshape(-1, 31)
     fix = np.full((near.shape[0], 1), int(np.float32(top / 2).view(np.uint32) >> 16))      # sets the block's exponent
     blocks = np.concatenate([near, fix], axis=1)
-    scaled = [np.where(blocks & 0x7FFF, blocks + s * 128, blocks) for s in (-60, -20, -7, 0, 5, 40)]
-    x = np.concatenate(scaled).reshape(-1).astype(np.uint16)
-    codes, scales = gpu_quantize(x, fmt)
+    field = blocks >> 7 & 0xFF
+    assert np.all((field == 0) | (1 <= field + s) & (field + s <= 254))
+    return np.where(field, blocks + s * 128, blocks & 0x8000).reshape(-1).astype(np.uint16)
+
+
+@pytest.mark.parametrize("s", [-60, -20, -7, 0, 5, 40])
+@pytest.mark.parametrize("fmt", INT_FORMATS)
+def test_bf16_halfway_points(fmt, s):
+    """Ties go away from zero, their neighbours do not follow them, the upper end is clipped, under each of six scales."""
+    x = halfway_points(fmt, s)
     wc, ws = orc.quantize(x, fmt)
+    assert np.all(ws == 127 + s)                                     # no block lost to a larger element than meant
+    assert np.unique(wc).size == (1 << orc.bits(fmt)) - 1            # every code but -2^(b-1), which is never produced
+    codes, scales = gpu_quantize(x, fmt)
     assert bits_equal(scales, ws), first_diff(scales, ws)
     assert bits_equal(codes, orc.pack(wc, orc.bits(fmt))), first_diff(codes, orc.pack(wc, orc.bits(fmt)))
 
