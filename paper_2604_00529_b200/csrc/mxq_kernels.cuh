@@ -581,10 +581,10 @@ __device__ __forceinline__ uint8_t* quantize_stage()
     }
 }
 
-// Resident CTAs (of 128 threads) per SM the quantizer is compiled for: 16, i.e. 32 registers (against the compiler's own choice the MXINT
-// and 6-bit quantizers are 2 - 4 % faster at 2^26 elements, the others unchanged), but 12 from FP32 to tiled E4M3, which in 32 registers
-// loads one lane unit after the other (2^23.5 elements 10.7 us against 9.2, 2^25 25.6 and 24.6; the other tiled formats lose up to
-// 5 % with 12 in the largest launches).
+// Resident CTAs (of 128 threads) per SM the quantizer is compiled for: 16, i.e. 32 registers (against the compiler's own choice, 2^25 elements
+// and more, BF16 -> MXINT7 and MXINT3 and FP32 -> MXINT7 3 - 4 % faster, MXINT5, 4 and 2 1 %, E3M3 4 %, E2M2 6 %, MXINT8 and MXINT6 1 %
+// slower, E4M3 4 %, E2M1 3 %), but 12 from FP32 to tiled E4M3, which in 32 registers loads one lane unit after the other (2^23.5
+// elements 10.7 us against 9.2, 2^25 25.6 and 24.6; the other tiled formats lose up to 5 % with 12 in the largest launches).
 template <class T, class F, class SCALES>
 __host__ __device__ constexpr int quantize_min_ctas()
 {
@@ -1021,7 +1021,7 @@ __device__ __forceinline__ void fp_quad_to_f16(const uint32_t (&in)[NW], uint32_
             : "=r"(a), "=r"(b) : "r"(w));
 }
 
-// two FP16 pairs (four E4M3 codes of one word), already divided by 2^de, as four FP32 values
+// two FP16 pairs (four MXFP codes), divided by 2^DE, as four FP32 values
 template <int DE>
 __device__ __forceinline__ void fp_pairs_scaled(uint32_t a, uint32_t b, float (&f)[4])
 {
@@ -1033,7 +1033,7 @@ __device__ __forceinline__ void fp_pairs_scaled(uint32_t a, uint32_t b, float (&
         : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]) : "r"(a), "r"(b), "r"(kHalf | (kHalf << 16)));
 }
 
-// Four E4M3 codes, given as two FP16 pairs, in a 5-, 6- or 7-bit MXFP format, the codes in the top bits of their
+// Four MXFP codes, given as two FP16 pairs, in a 5-, 6- or 7-bit MXFP format, the codes in the top bits of their
 // bytes.  `nans` has 0x7F in the bytes whose anchor code was a NaN code (see e4m3_word_clean).
 //   E2M3, E3M2: divided by 2^de (exact in FP16), widened to FP32, narrowing conversion.
 //   E3M3      : no narrowing instruction, but it is E4M3 with fewer binades (see SoftFp): the same through the
@@ -1042,8 +1042,9 @@ __device__ __forceinline__ void fp_pairs_scaled(uint32_t a, uint32_t b, float (&
 //               the trip through FP32 (the E4M3 conversion of FP16 pairs is slower than that trip).  The FP16 product
 //               is exact where it matters: it loses bits only below the smallest halfway point 2^-17, where every
 //               value rounds to zero either way (anchor codes have four significant bits).
-// Nothing is clipped: the largest anchor value 448 / 2^de (7, 28, 28, 7) does not exceed the target's largest
-// (7.5, 28, 30, 7).
+// From E4M3 nothing is clipped: its largest value 448 / 2^de (7, 28, 28, 7) does not exceed the target's largest (7.5, 28, 30, 7;
+// E2M3, E3M2, E3M3, E2M2).  From the narrower sources E3M3 -> E3M2 (30 against 28) relies on the conversion's saturation, and E2M2 as a
+// target on a clip of its own (7.5 against 7).
 template <class FH, class FL>
 __device__ __forceinline__ uint32_t ss_fp_pairs_top(uint32_t a, uint32_t b, uint32_t nans)
 {
@@ -1081,7 +1082,7 @@ __device__ __forceinline__ uint32_t ss_fp_pairs_top(uint32_t a, uint32_t b, uint
     }
 }
 
-// eight E4M3 codes (two words, given as their four FP16 pairs) -> eight E2M1 codes in one word
+// eight MXFP codes (given as their four FP16 pairs) -> eight E2M1 codes in one word; values up to 7 or 7.5 saturate at 6
 template <class FH>
 __device__ __forceinline__ uint32_t ss_fp_pairs_to_e2m1(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1)
 {
@@ -1098,7 +1099,7 @@ __device__ __forceinline__ uint32_t ss_fp_pairs_to_e2m1(uint32_t a0, uint32_t b0
     return d;
 }
 
-// Every legal pair, one element at a time (exact, slow): for units with E4M3 NaN codes.
+// From E4M3 to every target, one element at a time (exact, slow): for units with NaN codes.
 template <class FH, class FL, int NWI, int NWO>
 __device__ __forceinline__ void ss_unit_by_element(const uint32_t (&in)[NWI], uint32_t (&out)[NWO])
 {
@@ -1192,7 +1193,7 @@ __host__ __device__ constexpr bool ss_low_join()
 }
 
 // The 32 codes of one lane to one or more lower formats, eight codes at a time so that what
-// the targets share (sign masks and magnitudes, FP16 values) lives only that long.  E4M3 anchors:
+// the targets share (the FP16 values, and which codes are NaN) lives only that long.  E4M3 anchors:
 // NAN_CODES = false promises that none of the codes is a NaN code.  A NaN code maps to the largest magnitude with
 // its sign: so does the largest finite code, 448, wherever the target's largest mantissa is 1.75 or less
 // (448 / 2^de = 1.75 * 2^emax); for the three-bit mantissas (largest 1.875) the magnitude bits of the target
@@ -1432,8 +1433,12 @@ slice_scale_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict_
 // conversions share (the FP16 values of the codes) is computed once.  The set of targets is a compile-time list: a kernel that
 // walks a run-time list of formats keeps the shared words in registers across a switch and took 38 - 46 us for MXINT8 -> {7, 5, 3}
 // bits of 2^25.8 codes (block 64) where these take 30 (a pass per target: 50; the bytes alone: 26.7).  Compiled for 12
-// resident CTAs (40 registers): with 10 that set takes 30.9 us, {6, 4} of 2^26 codes 27.2 against 25.0, {7, 5} 31.2 against 29.0; with 14
-// most sets spill.  Sets of four spill at 12 and get 10.
+// resident CTAs (40 registers): with 10, 2^25.8 codes to {7, 5, 3} take 29.0 us against 28.9, {6, 4} 21.7 and 21.5, {7, 5} 25.1 and 24.7,
+// and launches of one or two waves gain or lose up to 20 % with their size ({6, 4} of 2^23.5 codes 4.9 against 5.4, 2^24 7.6 and 7.25); with
+// 14 most sets spill.  Sets of four spill at 12 and get 10.  A few still spill: {5, 3, 2} 48 bytes, {4, 3}, {4, 2}, {5, 4, 3}, {5, 4, 2} and
+// {7, 6, 4, 3} 4, {7, 6, 4, 2}, {7, 4, 3, 2} and {6, 4, 3, 2} 8, {E3M3, E3M2, E2M3} 12, {E3M3, E3M2, E2M2} 4.  Of the MXINT8 ones none is
+// slower for it than with the integer rounding, which spilled in one of them (2^26 codes: {5, 3, 2} 31.3 -> 30.8 us, {4, 2} 22.6 -> 20.3,
+// {5, 4, 2} 30.6 -> 27.5, {7, 6, 4, 2} 40.8 -> 38.2; 2^24: 10.7 -> 9.8, 6.7 -> 6.2, 10.6 -> 9.2, 12.5 -> 11.8).
 struct SsOut {
     uint8_t* codes;
     uint8_t* scales;
@@ -1610,9 +1615,9 @@ struct SsItemBlock {
     TileIndex index;
 };
 
-// (Compiled for 12 resident CTAs: without the bound MXINT8 -> MXINT5 of four decoder layers takes 261 us instead of 223, the
-// other targets between 2.6 % less and 2 % more.  SMALL: see slice_scale_is_small; seven tensors of 2^23 codes in all -> 7 bits 4.0 us
-// against 4.4, 6 3.8 and 4.3, 3 3.4 and 3.8.)
+// (Compiled for 12 resident CTAs: against the compiler's own choice, seven tensors of 2^25 to 2^28 codes in all, E4M3 -> E2M3 and E3M2 7 % faster,
+// MXINT8 -> 3 bits 5 %, -> 7, 5 and E3M3, E2M2 2 %, the others the same but MXINT8 -> 6 bits, 3 % slower.  SMALL: see
+// slice_scale_is_small; seven tensors of 2^23 codes -> 7 bits 4.0 us against 4.4, 6 3.8 and 4.3, 3 3.4 and 3.8.)
 template <class FH, class FL, int U, int THREADS, int K, bool SMALL = false>
 __global__ void __launch_bounds__(THREADS, SMALL ? 10 : 12)
 slice_scale_batched_param_kernel(const __grid_constant__ SsItemBlock<K> blk)
