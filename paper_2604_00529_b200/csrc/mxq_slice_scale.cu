@@ -29,11 +29,19 @@ int run_single(const void* codes, const uint8_t* scales, size_t n, int block, vo
                 ntiles = (nunits + 31) / 32;
             }
         }
-        // MXINT8 in about one wave: the kernel with fewer resident CTAs (measured at slice_scale_is_small).
+        // MXINT8 in about one wave: the kernel with fewer resident CTAs (measured at slice_scale_is_small); to 3 bits, up to four CTAs per
+        // SM, one unit per thread (2^14 codes 1.6 -> 1.4 us, 2^20 1.8 -> 1.6, 2^22 2.9 -> 2.55; 2^22.25 3.0 -> 3.05).
         if constexpr (slice_scale_has_small<FH, FL>()) {
-            if (slice_scale_is_small<FL>((ntiles + kThreads / 32 - 1) / (kThreads / 32)))
+            const size_t ctas = (ntiles + kThreads / 32 - 1) / (kThreads / 32);
+            if (slice_scale_is_small<FL>(ctas))
                 kern = block == 16 ? slice_scale_kernel<FH, FL, kU, kThreads, uint8_t*, true, true>
                                    : slice_scale_kernel<FH, FL, kU, kThreads, uint8_t*, false, true>;
+            if constexpr (FL::bits == 3) {
+                if (ctas <= (size_t)148 * 4) {
+                    kern = block == 16 ? slice_scale_kernel<FH, FL, 1, kThreads, uint8_t*, true> : slice_scale_kernel<FH, FL, 1, kThreads>;
+                    ntiles = (nunits + 31) / 32;
+                }
+            }
         }
         return launch_kernel(kern, grid_for_tiles(ntiles, kThreads), kThreads, stream, static_cast<const uint8_t*>(codes),
                              scales, nunits, nscales, static_cast<uint8_t*>(out_codes), out_scales);

@@ -61,11 +61,11 @@ def test_slice_scale_on_both_sides_of_the_small_launch_rule(dst, block):
 @pytest.mark.parametrize("block", [16, 32, 64])
 @pytest.mark.parametrize("dst", ["int7", "int6", "int4", "int3", "int2"])
 def test_slice_scale_from_mxint8_on_both_sides_of_its_one_wave_rules(dst, block):
-    """Ten CTAs per SM (twelve to four and three bits; to four bits also five), and the smallest tensors."""
+    """Ten CTAs per SM (twelve to four and three bits; to four bits also five, to three also four), and the smallest tensors."""
     codes, scales = codes_and_scales("int8", block, 5 * block)
     wc, ws = orc.slice_scale(codes, scales, "int8", dst, block)
     packed = orc.pack(wc, orc.bits(dst))
-    for units in [1, 65, 3 * CTA - 2] + unit_counts(148 * 5) + unit_counts(148 * 10) + unit_counts(148 * 12):
+    for units in [1, 65, 3 * CTA - 2] + unit_counts(148 * 4) + unit_counts(148 * 5) + unit_counts(148 * 10) + unit_counts(148 * 12):
         n = max(units * 32, block) // block * block
         oc, os_ = Guarded(mxq.codes_bytes(n, dst)), Guarded(n // block)
         mxq.slice_scale(repeated(codes, n), repeated(scales, n // block), n, "int8", dst, block, oc.view, os_.view)
