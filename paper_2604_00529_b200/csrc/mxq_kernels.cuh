@@ -1378,11 +1378,11 @@ __device__ __forceinline__ uint8_t* slice_scale_stage()
     }
 }
 
-// Resident CTAs (of 128 threads) per SM the single-tensor kernel is compiled for, i.e. its register
-// budget.  MXINT conversions to more than four bits are fastest with room for 40 - 48 registers (2^26 codes, 10 against 14 CTAs:
-// -> 6 19.3 and 20.0 us, -> 5 19.6 and 21.1) and to two (14.4 and 14.7), to four and three in 32 (MXINT8 -> MXINT4 of 2^24 codes
-// 4.13 and 4.01, of 2^26 the same; -> 3 17.1 and 16.7; MXINT5 -> MXINT3 16.1 and 15.5); the MXFP ones with 14 - 16 CTAs (E4M3 -> E2M3 8 % faster than at 50
-// registers).  With tiled scale outputs 14 CTAs would spill, so those keep 12.
+// Resident CTAs (of 128 threads) per SM the single-tensor kernel is compiled for, i.e. its register budget; 10 against 14, mean over
+// 2^24 to 2^26.5 codes.  MXINT to five bits and more and to two gets room for 48 registers (with 14 MXINT8 -> 7 / 6 / 5 / 2 bits are 7 / 8 / 6 / 5 %
+// slower), MXINT8 -> 4 and 3 fit 32 (with 10 1 and 5 % slower; from MXINT7, 6 and 5 to 3 bits 10 would be 3 - 6 % faster, the other narrow
+// sources take the same), and so do the MXFP ones (block 32: the same to 2 %).  With tiled scale outputs 14 CTAs would spill, so
+// those keep 12.
 //   SMALL : see slice_scale_is_small.
 template <class FH, class FL, class SCALES, bool SMALL>
 __host__ __device__ constexpr int slice_scale_min_ctas()
